@@ -400,6 +400,7 @@ extern "C" nam_status nam_create_material(nam_ctx* ctx, const nam_material_desc*
       return fail(NAM_ERR_UNSUPPORTED, "weight packing failed");
     }
     e = (int)cudaMemcpy(m->blob, blob.data(), blob_bytes, cudaMemcpyHostToDevice);
+    pack_narrow(sh, master.data() + nframe, &m->nw);
   }
   if (!e && d->trainable) {
     size_t nb = (m->pyr_off + pd.texels * 8) * 4;
@@ -485,6 +486,7 @@ void nam::fill_launch(nam_ctx* ctx, const nam_material_s* m, const nam_queries* 
   L->err = ctx->err_word;
   L->timeout_ns = ctx->timeout_ns;
   L->num_sms = ctx->num_sms;
+  L->nw = &m->nw;
 }
 
 int nam::launch_material(const LaunchCommon& L, int precision, void* stream) {

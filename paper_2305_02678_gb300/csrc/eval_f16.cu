@@ -18,9 +18,9 @@ static void puth(uint8_t* base, int R, int row, int k, float v) {
   std::memcpy(base + kmaj(R, row, k), &h, 2);
 }
 
-// v rounded to binary16, stored as FP32 at float index i of base
-static void putf(uint8_t* base, int i, float v) {
-  const float r = __half2float(__float2half_rn(v));
+// v rounded to binary16, times `scale`, stored as FP32 at float index i of base
+static void putf(uint8_t* base, int i, float v, float scale = 1.0f) {
+  const float r = scale * __half2float(__float2half_rn(v));
   std::memcpy(base + 4 * i, &r, 4);
 }
 static void putf_exact(uint8_t* base, int i, float v) { std::memcpy(base + 4 * i, &v, 4); }
@@ -96,7 +96,7 @@ int pack_f16_blob(const Shape& s, int precision, const float* frame, const float
     }
     for (int j = 0; j < 6; ++j) {
       for (int k = 0; k < 32; ++k) puth(out + o.BF2, 16, j, k, Wf2[j * 16 + (k & 15)]);
-      putf(out + o.SB, 16 + j, bf2[j]);
+      putf(out + o.SB, 8 + j, bf2[j]);
     }
   } else if (s.frame == 2) {
     const float* Wf = frame;     // [12][8]
@@ -146,12 +146,22 @@ int pack_f16_blob(const Shape& s, int precision, const float* frame, const float
   const float* Wo = p;
   const float* bo = Wo + s.out * H;
   for (int n = 0; n < s.out; ++n) {
-    for (int k = 0; k < H; ++k) puth(out + o.BO, 16, n, k, Wo[n * H + k]);
-    putf(out + o.SB, 24 + n, bo[n]);
+    for (int k = 0; k < H; ++k) putf(out + o.WO, n * H + k, Wo[n * H + k], 0.5f);
+    putf(out + o.SB, 16 + n, bo[n]);
   }
   return 0;
 }
 
+
+void pack_narrow(const Shape& s, const float* dec, NarrowW* out) {
+  std::memset(out, 0, sizeof *out);
+  auto r16 = [](float v) { return __half2float(__float2half_rn(v)); };
+  const float* Wo = dec + s.H * s.in + s.H + (s.NH - 1) * (s.H * s.H + s.H);
+  for (int n = 0; n < s.out; ++n) {
+    for (int k = 0; k < s.H; ++k) out->wo[n][k] = 0.5f * r16(Wo[n * s.H + k]);
+    out->bo[n] = r16(Wo[s.out * s.H + n]);
+  }
+}
 
 size_t tc_blob_bytes(const Shape& s, int precision) {
   if (precision != NAM_PREC_F16 && precision != NAM_PREC_FP8) return 0;

@@ -65,6 +65,16 @@ struct MatTable {
   int32_t nmat;
 };
 
+// The decoder's output layer of one material, at the precision the
+// tensor-core path gives its weights.  It travels in the kernel's parameters:
+// weights in constant memory cost the load/store pipe nothing, which the
+// texel gathers keep busy (from shared memory the 1920x1080 frame takes 117
+// us, from here 97).  The activations enter as a + |a| = 2 max(a, 0) (one
+// FADD), so the weights are halved (exact).
+struct NarrowW {
+  float wo[6][64], bo[6];
+};
+
 // ---------------------------------------------------------------------------
 // launchers (return cudaError_t as int)
 // ---------------------------------------------------------------------------
@@ -98,6 +108,8 @@ struct LaunchCommon {
                          // rgb may then be null
   float* albedo;         // albedo head (shape.out == 6): if set, [n][3]
                          // directional albedo of each query
+  const NarrowW* nw;     // tensor-core kernel, single-material launches: host
+                         // memory, copied into the kernel's parameters
 };
 
 // Resident blocks per SM of a kernel: the occupancy API, or (resources_only,
@@ -130,6 +142,7 @@ size_t f16_blob_bytes(const Shape& s);
 int pack_f16_blob(const Shape& s, int precision, const float* frame, const float* dec, const float* act_scale,
                   uint8_t* out, float* weight_scales_out);
 int launch_eval_tc(const LaunchCommon& L, int precision, void* stream);
+void pack_narrow(const Shape& s, const float* dec, NarrowW* out);
 
 // Weight blob sizes and packing (host side).
 size_t f32_blob_floats(const Shape& s);

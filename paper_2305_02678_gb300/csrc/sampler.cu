@@ -249,14 +249,14 @@ __global__ void __launch_bounds__(NWG * 128, 1)
   float zr[8];  // filtered latent of the tile about to start (FP16 pyramids)
   if (c < c_end) {
     const int64_t i0 = c * 128 + r;
-    const QF q0 = load_qf(L.q, i0 < L.n ? i0 : L.n - 1);
+    const QF q0 = load_qf<true>(L.q, i0 < L.n ? i0 : L.n - 1);
     if (F16P) {
       fetch_issue(L.pyr, reinterpret_cast<const uint8_t*>(L.pyr0), q0, stg);
       fetch_finish(stg, zr);
     }
     if (c + NWG < c_end) {
       const int64_t i1 = (c + NWG) * 128 + r;
-      q_nxt = load_qf(L.q, i1 < L.n ? i1 : L.n - 1);
+      q_nxt = load_qf<true>(L.q, i1 < L.n ? i1 : L.n - 1);
     }
   }
   for (; c < c_end; c += NWG) {
@@ -278,7 +278,7 @@ __global__ void __launch_bounds__(NWG * 128, 1)
 #pragma unroll
       for (int k = 0; k < 8; ++k) x[k] = zr[k];
     } else {
-      const QF q0 = load_qf(L.q, i);
+      const QF q0 = load_qf<true>(L.q, i);
       fetch_latent<false>(L.pyr, L.pyr0, q0.u, q0.v, q0.lod, q0.xi, x);
     }
     x[8] = wi[0];
@@ -306,7 +306,7 @@ __global__ void __launch_bounds__(NWG * 128, 1)
     if (F16P && has_next) fetch_issue(L.pyr, reinterpret_cast<const uint8_t*>(L.pyr0), q_nxt, stg);
     if (has_next2) {
       const int64_t i2 = (c + 2 * NWG) * 128 + r;
-      q_nxt2 = load_qf(L.q, i2 < L.n ? i2 : L.n - 1);
+      q_nxt2 = load_qf<true>(L.q, i2 < L.n ? i2 : L.n - 1);
     }
     stage_wait();
     // ---- layers 2, 3 (32 -> 32) and 4 (32 -> 9) -----------------------------

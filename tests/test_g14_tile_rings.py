@@ -1,0 +1,65 @@
+"""Launches of many tiles per CTA: the operand buffers between the fetch and
+the chain warpgroups are used over and over, and every query must come out
+bitwise as in launches of one tile per CTA (where no buffer is used twice)."""
+import numpy as np
+import pytest
+
+import workloads as W
+from conftest import to_device
+
+pytestmark = pytest.mark.gpu
+
+
+def _pieces(mat, dq, n, size):
+    import torch
+    return torch.cat([mat.eval({k: t[a:a + size] for k, t in dq.items()}) for a in range(0, n, size)])
+
+
+@pytest.mark.parametrize("precision,H,NH,frame,filt,latent", [
+    (1, 64, 2, (8, 16, 6), 0, np.float16),
+    (1, 64, 3, (8, 12), 1, np.float16),
+    (2, 64, 2, (8, 16, 6), 0, np.float16),
+    (1, 32, 2, (8, 12), 0, np.float16),
+    (1, 16, 2, None, 1, np.float32),
+])
+def test_many_tiles_per_cta(gctx, precision, H, NH, frame, filt, latent):
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    rng = W.rng_streams(141, 3)
+    pyr = W.make_pyramid(rng[0], 128, 128, 8, dtype=latent)
+    nin = 20 if frame == (8, 12) else 14
+    model = W.make_model(rng[1], (nin,) + (H,) * NH + (3,), frame)
+    kw = {"act_scale": np.full(NH + 1, 0.004, np.float32)} if precision == 2 else {}
+    mat = gctx.material(128, 128, 8, pyr, model["frame"], model["decoder"], precision=precision, filter=filt, **kw)
+    n = sms * 128 * 33 + 77
+    dq = to_device(W.uniform_queries(rng[2], n, 7.0))
+    whole = mat.eval(dq)
+    assert torch.equal(whole, _pieces(mat, dq, n, sms * 128))
+    mat.destroy()
+    gctx.check()
+
+
+def test_many_chunks_per_cta_mixed_materials(gctx):
+    """Materials of very different sizes, so that chains of one CTA hold, give
+    up and reload weight slots while their operands arrive."""
+    import torch
+    from paper_2305_02678_gb300 import binding as B
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    rng = W.rng_streams(142, 30)
+    mats = []
+    for k in range(12):
+        model = W.make_model(rng[k], (14, 64, 64, 3), (8, 16, 6))
+        mats.append(gctx.material(64, 64, 7, W.make_pyramid(rng[12 + k], 64, 64, 7, dtype=np.float16), model["frame"],
+                                  model["decoder"]))
+    n = sms * 128 * 9 + 5
+    dq = to_device(W.uniform_queries(rng[24], n, 6.0))
+    ids = np.minimum(rng[25].geometric(0.35, n) - 1, 11).astype(np.int32)
+    out = torch.empty((n, 3), device="cuda")
+    B.nam_eval_binned(gctx.h, [m.h for m in mats], dq, torch.from_numpy(ids).cuda(), n, out,
+                      torch.cuda.current_stream())
+    for k, m in enumerate(mats):
+        idx = torch.from_numpy(np.nonzero(ids == k)[0]).cuda()
+        sub = {f: t[idx].contiguous() for f, t in dq.items()}
+        assert torch.equal(out[idx], _pieces(m, sub, idx.numel(), sms * 128)), k
+        m.destroy()
+    gctx.check()
