@@ -344,8 +344,16 @@ extern "C" nam_status nam_create_material(nam_ctx* ctx, const nam_material_desc*
   m->pyr = pd;
   m->n_params = np;
   size_t blob_bytes = 0;
+  std::vector<uint8_t> f32_blob;
   if (d->precision == NAM_PREC_F32) {
-    blob_bytes = 0;  // the FP32 kernels read the master layout directly
+    // fixed weights run on the tensor cores as split operands; the per-thread
+    // kernel reads the master layout directly (trainable materials, and
+    // weights without a split)
+    if (!d->trainable) {
+      f32_blob.resize(f32_tc_blob_bytes(sh));
+      if (f32_blob.empty() || pack_f32_tc_blob(sh, master.data(), master.data() + nframe, f32_blob.data(), &m->nw) != 0) f32_blob.clear();
+      blob_bytes = f32_blob.size();
+    }
   } else {
     blob_bytes = tc_blob_bytes(sh, d->precision);
     if (!blob_bytes) {
@@ -392,7 +400,9 @@ extern "C" nam_status nam_create_material(nam_ctx* ctx, const nam_material_desc*
     e = (int)cudaMemcpy(m->enc, encw.data(), encw.size() * 4, cudaMemcpyHostToDevice);
     if (!e) e = (int)cudaMemset(m->enc + encw.size(), 0, 3 * encw.size() * 4);  // gradient, Adam m, v
   }
-  if (!e && blob_bytes) {
+  if (!e && !f32_blob.empty()) {
+    e = (int)cudaMemcpy(m->blob, f32_blob.data(), blob_bytes, cudaMemcpyHostToDevice);
+  } else if (!e && blob_bytes) {
     std::vector<uint8_t> blob(blob_bytes);
     if (pack_tc_blob(sh, d->precision, nframe ? master.data() : nullptr, master.data() + nframe,
                      d->fp8_act_scale, blob.data(), m->info.fp8_weight_scale) != 0) {
@@ -480,7 +490,8 @@ void nam::fill_launch(nam_ctx* ctx, const nam_material_s* m, const nam_queries* 
   L->rgb = rgb;
   L->n = n;
   L->pyr0 = m->pyramid;
-  L->w0 = m->desc.precision == NAM_PREC_F32 ? (const void*)m->params : m->blob;
+  L->w0 = m->blob ? m->blob : (const void*)m->params;
+  if (m->desc.precision == NAM_PREC_F32 && m->blob) L->masters = m->params;
   L->mats.nmat = 1;
   L->flags = flags;
   L->err = ctx->err_word;
@@ -490,7 +501,7 @@ void nam::fill_launch(nam_ctx* ctx, const nam_material_s* m, const nam_queries* 
 }
 
 int nam::launch_material(const LaunchCommon& L, int precision, void* stream) {
-  if (precision == NAM_PREC_F32) return launch_eval_f32(L, stream);
+  if (precision == NAM_PREC_F32) return L.masters ? launch_eval_f32_tc(L, stream) : launch_eval_f32(L, stream);
   return launch_eval_tc(L, precision, stream);
 }
 

@@ -259,17 +259,33 @@ __device__ __forceinline__ void fetch_finish(uint32_t stg, float z[8]) {
 // result holds the integer in its low mantissa bits (no conversion
 // instructions, which run at a quarter of the rate), and W_l, H_l from the
 // exponents of level 0's sizes.
+// EXACT (the FP32 kernel): fractions and weights as in tap_axis and
+// bilinear_acc, bit for bit.
+template <bool EXACT>
 __device__ __forceinline__ void level_taps(const PyrDesc& P, int l, float u, float v, bool fast, int lw0, int lh0,
                                            float wl, uint32_t idx[4], float* w) {
   int x0, x1, y0, y1, W;
   float fx, fy;
   if (fast) {
     const int ew = max(lw0 - l, 0), eh = max(lh0 - l, 0);
-    const float xs = u * __int_as_float((127 + ew) << 23) - 0.5f, ys = v * __int_as_float((127 + eh) << 23) - 0.5f;
-    const float tx = __fadd_rd(xs, 12582912.0f), ty = __fadd_rd(ys, 12582912.0f);
-    fx = xs - (tx - 12582912.0f);
-    fy = ys - (ty - 12582912.0f);
-    const int kx = __float_as_int(tx), ky = __float_as_int(ty);
+    const float X = u * __int_as_float((127 + ew) << 23), Y = v * __int_as_float((127 + eh) << 23);
+    int kx, ky;
+    if (EXACT) {
+      // the 1/2 comes off the fractional part (tap_axis)
+      const float tx = __fadd_rd(X, 12582912.0f), ty = __fadd_rd(Y, 12582912.0f);
+      const float rx = X - (tx - 12582912.0f), ry = Y - (ty - 12582912.0f);
+      kx = __float_as_int(tx) - (rx >= 0.5f ? 0 : 1);
+      ky = __float_as_int(ty) - (ry >= 0.5f ? 0 : 1);
+      fx = rx >= 0.5f ? rx - 0.5f : rx + 0.5f;
+      fy = ry >= 0.5f ? ry - 0.5f : ry + 0.5f;
+    } else {
+      const float xs = X - 0.5f, ys = Y - 0.5f;
+      const float tx = __fadd_rd(xs, 12582912.0f), ty = __fadd_rd(ys, 12582912.0f);
+      fx = xs - (tx - 12582912.0f);
+      fy = ys - (ty - 12582912.0f);
+      kx = __float_as_int(tx);
+      ky = __float_as_int(ty);
+    }
     W = 1 << ew;
     const int mx = W - 1, my = (1 << eh) - 1;
     x0 = kx & mx;
@@ -284,11 +300,18 @@ __device__ __forceinline__ void level_taps(const PyrDesc& P, int l, float u, flo
   const uint32_t base = (uint32_t)P.off[l];
   const uint32_t r0 = base + (uint32_t)y0 * (uint32_t)W, r1 = base + (uint32_t)y1 * (uint32_t)W;
   const float gx = 1.0f - fx, gy = 1.0f - fy;
-  const float a = gy * wl, b = fy * wl;
-  w[0] = gx * a;
-  w[1] = fx * a;
-  w[2] = gx * b;
-  w[3] = fx * b;
+  if (EXACT) {
+    w[0] = gx * gy * wl;
+    w[1] = fx * gy * wl;
+    w[2] = gx * fy * wl;
+    w[3] = fx * fy * wl;
+  } else {
+    const float a = gy * wl, b = fy * wl;
+    w[0] = gx * a;
+    w[1] = fx * a;
+    w[2] = gx * b;
+    w[3] = fx * b;
+  }
   idx[0] = r0 + x0;
   idx[1] = r0 + x1;
   idx[2] = r1 + x0;
@@ -331,7 +354,7 @@ __device__ __forceinline__ void load4(const uint8_t* pyr, const uint32_t idx[4],
 
 // z of one query (Sec. 4.1): levels l0 (weight 1 - t) and l1 (weight t; not
 // read when t = 0), or the stochastic pick of one of them.
-template <bool F16P>
+template <bool F16P, bool EXACT>
 __device__ __forceinline__ void fetch_direct(const PyrDesc& P, const uint8_t* pyr, const QF& q, int lw0, int lh0,
                                              float z[8]) {
   const float l = fminf(fmaxf(q.lod, 0.0f), (float)(P.levels - 1));  // NaN -> 0
@@ -349,12 +372,12 @@ __device__ __forceinline__ void fetch_direct(const PyrDesc& P, const uint8_t* py
   uint32_t idx[4];
   float wa[4];
   uint4 ta[F16P ? 4 : 8];
-  level_taps(P, la, q.u, q.v, fast, lw0, lh0, stoch ? 1.0f : 1.0f - t, idx, wa);
+  level_taps<EXACT>(P, la, q.u, q.v, fast, lw0, lh0, stoch ? 1.0f : 1.0f - t, idx, wa);
   load4<F16P>(pyr, idx, ta);
   if (!stoch) {
     float wb[4];
     uint4 tb[F16P ? 4 : 8];
-    level_taps(P, l1, q.u, q.v, fast, lw0, lh0, t, idx, wb);
+    level_taps<EXACT>(P, l1, q.u, q.v, fast, lw0, lh0, t, idx, wb);
     if (t != 0.0f) {
       load4<F16P>(pyr, idx, tb);
     } else {
@@ -371,6 +394,48 @@ __device__ __forceinline__ void fetch_direct(const PyrDesc& P, const uint8_t* py
     z[2 * c] = acc[c].x;
     z[2 * c + 1] = acc[c].y;
   }
+}
+
+// The loop of one fetch warpgroup (fw of NF): it takes tiles fw, fw + NF, ...
+// of the CTA's range [c_begin, c_end), each warp its own 32 rows, and hands
+// tile t's filtered latents to the chains through ring entry t % NZ:
+// emit(slot, z) writes this row's; bar_f[slot] counts the four warps that
+// filled it, bar_e[slot] its reading.  The next tile's query fields are in
+// flight while this tile's texels are.  False if a wait ran out.
+template <bool F16P, bool MULTI, bool EXACT, int NF, int NZ, class PyrFor, class RowOf, class Emit>
+__device__ __forceinline__ bool fetch_loop(const LaunchCommon& L, int64_t c_begin, int64_t c_end, int fw, uint32_t bar_f,
+                                           uint32_t bar_e, bool bad, PyrFor pyr_for, RowOf row_of, Emit emit) {
+  const int lw0 = 31 - __clz(L.pyr.w[0]), lh0 = 31 - __clz(L.pyr.h[0]);
+  int64_t c = c_begin + fw;
+  int slot = fw, pass = 0;
+  TileRef nxt{};
+  QF qn{};
+  if (c < c_end) {
+    nxt = tile_at(L, c);
+    if (nxt.count > 0) qn = load_qf<MULTI>(L.q, row_of(nxt));
+  }
+  for (; c < c_end; c += NF) {
+    const TileRef cur = nxt;
+    const QF q = qn;
+    if (c + NF < c_end) {
+      nxt = tile_at(L, c + NF);
+      if (nxt.count > 0) qn = load_qf<MULTI>(L.q, row_of(nxt));
+    }
+    float z[8];
+    if (cur.count > 0) fetch_direct<F16P, EXACT>(L.pyr, pyr_for(cur), q, lw0, lh0, z);
+    // the entry's previous latents have been read
+    if (pass > 0) bad |= !ptx::mbar_wait(bar_e + 8 * slot, (uint32_t)(pass - 1) & 1u, L.timeout_ns);
+    if (__any_sync(0xffffffffu, bad)) return false;
+    if (cur.count > 0) emit(slot, z);
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) ptx::mbar_arrive(bar_f + 8 * slot);
+    slot += NF;
+    if (slot >= NZ) {
+      slot -= NZ;
+      ++pass;
+    }
+  }
+  return true;
 }
 
 // ---------------------------------------------------------------------------
@@ -531,58 +596,21 @@ __global__ void __launch_bounds__((NCH + NF) * 128, 1) eval_f16_kernel(const __g
   auto row_of = [&](const TileRef& t) -> int64_t { return src(t.start + (r < t.count ? r : 0)); };
 
   if (wg >= NCH) {
-    // ======================= fetch warpgroups ==============================
-    // Warpgroup fw takes tiles fw, fw + NF, ... of the CTA's range; each
-    // warp works on its own 32 rows.
-    const int fw = wg - NCH;
-    const int lw0 = 31 - __clz(L.pyr.w[0]), lh0 = 31 - __clz(L.pyr.h[0]);
     auto pyr_for = [&](const TileRef& t) -> const uint8_t* {
       return reinterpret_cast<const uint8_t*>(MULTI ? L.mats.pyramid[t.mat] : L.pyr0);
     };
-    int64_t c = c_begin + fw;
-    int slot = fw, pass = 0;
-    TileRef nxt{};
-    QF qn{};
-    if (c < c_end) {
-      nxt = tile_at(L, c);
-      if (nxt.count > 0) qn = load_qf<MULTI>(L.q, row_of(nxt));
-    }
-    for (; c < c_end; c += NF) {
-      const TileRef cur = nxt;
-      const QF q = qn;
-      if (c + NF < c_end) {
-        nxt = tile_at(L, c + NF);
-        if (nxt.count > 0) qn = load_qf<MULTI>(L.q, row_of(nxt));
-      }
-      uint32_t v[8];
-      if (cur.count > 0) {
-        float z[8];
-        fetch_direct<F16P>(L.pyr, pyr_for(cur), q, lw0, lh0, z);
-        split_pair<false>(z[0], z[1], v[0], v[4]);
-        split_pair<false>(z[2], z[3], v[1], v[5]);
-        split_pair<false>(z[4], z[5], v[2], v[6]);
-        split_pair<false>(z[6], z[7], v[3], v[7]);
-      }
-      // the chain has read its previous operand
-      if (pass > 0) bad |= !ptx::mbar_wait(bar_e + 8 * slot, (uint32_t)(pass - 1) & 1u, L.timeout_ns);
-      if (__any_sync(0xffffffffu, bad)) {
-        bad = true;
-        break;
-      }
-      if (cur.count > 0) {
-        const uint32_t zs = ptx::smem_u32(smem + S::Z_OFF + slot * S::ZB) + r * 16;
-        ptx::st_shared_v4(zs, v[0], v[1], v[2], v[3]);         // z hi
-        ptx::st_shared_v4(zs + 2048, v[4], v[5], v[6], v[7]);  // z lo
-        ptx::fence_proxy_async();
-      }
-      __syncwarp();
-      if ((tid & 31) == 0) ptx::mbar_arrive(bar_f + 8 * slot);
-      slot += NF;
-      if (slot >= NZ) {
-        slot -= NZ;
-        ++pass;
-      }
-    }
+    bad = !fetch_loop<F16P, MULTI, false, NF, NZ>(
+        L, c_begin, c_end, wg - NCH, bar_f, bar_e, bad, pyr_for, row_of, [&](int slot, const float z[8]) {
+          uint32_t v[8];
+          split_pair<false>(z[0], z[1], v[0], v[4]);
+          split_pair<false>(z[2], z[3], v[1], v[5]);
+          split_pair<false>(z[4], z[5], v[2], v[6]);
+          split_pair<false>(z[6], z[7], v[3], v[7]);
+          const uint32_t zs = ptx::smem_u32(smem + S::Z_OFF) + slot * S::ZB + r * 16;
+          ptx::st_shared_v4(zs, v[0], v[1], v[2], v[3]);         // z hi
+          ptx::st_shared_v4(zs + 2048, v[4], v[5], v[6], v[7]);  // z lo
+          ptx::fence_proxy_async();
+        });
   } else {
   // ========================= chain warpgroups ==============================
   const uint32_t bar_m = bar0 + 8 * wg;

@@ -20,8 +20,8 @@ struct nam_material_s {
   nam::PyrDesc pyr;
   int64_t n_params = 0;
   void* pyramid = nullptr;    // device pyramid (FP16 or FP32 texels)
-  void* blob = nullptr;       // tensor-core weight blob (F16 / FP8)
-  nam::NarrowW nw{};          // its output layer, passed in the kernel's parameters
+  void* blob = nullptr;       // tensor-core weight blob (F16, FP8; F32 unless trainable)
+  nam::NarrowW nw{};          // its narrow layers, passed in the kernel's parameters
   float* params = nullptr;    // FP32 masters (frame then decoder)
   void* sampler = nullptr;    // importance-sampler weights as tensor-core operands, or null
   int64_t pyr_off = 0;        // trainable: offset of the pyramid block in

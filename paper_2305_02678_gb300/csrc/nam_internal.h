@@ -73,6 +73,9 @@ struct MatTable {
 // FADD), so the weights are halved (exact).
 struct NarrowW {
   float wo[6][64], bo[6];
+  // FP32 arithmetic on the tensor cores (eval_f32_tc.cu; wo not halved
+  // there): its frame layers too
+  float f1[8][16], fb1[16], f2[6][16], fb2[6];
 };
 
 // ---------------------------------------------------------------------------
@@ -110,6 +113,8 @@ struct LaunchCommon {
                          // directional albedo of each query
   const NarrowW* nw;     // tensor-core kernel, single-material launches: host
                          // memory, copied into the kernel's parameters
+  // FP32 arithmetic on the tensor cores (w0 is the split-weight blob then)
+  const float* masters;       // device: FP32 masters; null: the per-thread kernel runs
 };
 
 // Resident blocks per SM of a kernel: the occupancy API, or (resources_only,
@@ -142,6 +147,11 @@ size_t f16_blob_bytes(const Shape& s);
 int pack_f16_blob(const Shape& s, int precision, const float* frame, const float* dec, const float* act_scale,
                   uint8_t* out, float* weight_scales_out);
 int launch_eval_tc(const LaunchCommon& L, int precision, void* stream);
+// FP32 evaluation on the tensor cores (weights packed once; -1 if a weight is
+// too large to round to bfloat16)
+int launch_eval_f32_tc(const LaunchCommon& L, void* stream);
+size_t f32_tc_blob_bytes(const Shape& s);
+int pack_f32_tc_blob(const Shape& s, const float* frame, const float* dec, uint8_t* out, NarrowW* nw);
 void pack_narrow(const Shape& s, const float* dec, NarrowW* out);
 
 // Weight blob sizes and packing (host side).
