@@ -198,7 +198,7 @@ __global__ void __launch_bounds__((NCH + NF) * 128, 1)
     bad = !fetch_loop<F16P, false, true, NF, NZ>(
         L, c_begin, c_end, wg - NCH, bar_f, bar_e, bad,
         [&](const TileRef&) { return reinterpret_cast<const uint8_t*>(L.pyr0); }, row_of,
-        [&](int slot, const float z[8]) {
+        [](const TileRef&) {}, [&](int slot, const float z[8]) {
           const uint32_t zs = ptx::smem_u32(smem + S::Z_OFF) + slot * S::ZB + r * 16;
           auto u = [](float v) { return __float_as_uint(v); };
           ptx::st_shared_v4(zs, u(z[0]), u(z[1]), u(z[2]), u(z[3]));

@@ -151,116 +151,16 @@ __device__ __forceinline__ TileRef tile_at(const LaunchCommon& L, int64_t c) {
   return t;
 }
 
-// Per-warpgroup staging of one tile's latent fetch in shared memory: tap k of
-// row r at k * 2048 + r * 16 (8 binary16 channels), the eight tap weights
-// at 16384 + j * 2048 + r * 16 (two float4).  Each thread reads back only
-// what it wrote itself.
-constexpr int kStageBytes = 16384 + 4096;
-
-// Bilinear taps of level l (Sec. 4.1; texel centres at (i + 1/2) / W):
-// issues the four 16-byte copies into slots dst + k * 2048 (zero-filled and
-// not read when `load` is false) and writes the weights wl * (bilinear
-// weight) to w[0..3].  `fast` (warp-uniform): power-of-two wrap with every
-// lane's |u W0|, |v H0| < 2^22, where X = u W is exact and the continuous
-// coordinate x = X - 1/2 is exact except for X in (-1/2, 1/2) (fraction moved
-// by at most 2^-25); otherwise the exact general addressing of tap_axis.
-__device__ __forceinline__ void level_issue(const PyrDesc& P, const uint8_t* pyr, int l, float u, float v,
-                                            bool fast, float wl, bool load, uint32_t dst, float* w) {
-  const int W = P.w[l], H = P.h[l];
-  int x0, x1, y0, y1;
-  float fx, fy;
-  if (fast) {
-    const float xs = u * (float)W - 0.5f, ys = v * (float)H - 0.5f;
-    const float xf = floorf(xs), yf = floorf(ys);
-    fx = xs - xf;
-    fy = ys - yf;
-    const int kx = (int)xf, ky = (int)yf;
-    x0 = kx & (W - 1);
-    x1 = (kx + 1) & (W - 1);
-    y0 = ky & (H - 1);
-    y1 = (ky + 1) & (H - 1);
-  } else {
-    tap_axis(P, u, W, x0, x1, fx);
-    tap_axis(P, v, H, y0, y1, fy);
-  }
-  const uint32_t base = (uint32_t)P.off[l];
-  const uint32_t r0 = base + (uint32_t)y0 * (uint32_t)W, r1 = base + (uint32_t)y1 * (uint32_t)W;
-  const float gx = 1.0f - fx, gy = 1.0f - fy;
-  const float a = gy * wl, b = fy * wl;
-  w[0] = gx * a;
-  w[1] = fx * a;
-  w[2] = gx * b;
-  w[3] = fx * b;
-  const uint32_t sz = load ? 16u : 0u;
-  ptx::cp_async16(dst, pyr + (size_t)(r0 + x0) * 16, sz);
-  ptx::cp_async16(dst + 2048, pyr + (size_t)(r0 + x1) * 16, sz);
-  ptx::cp_async16(dst + 4096, pyr + (size_t)(r1 + x0) * 16, sz);
-  ptx::cp_async16(dst + 6144, pyr + (size_t)(r1 + x1) * 16, sz);
-}
-
-// Start the latent fetch of one query into its staging slots (FP16 pyramid).
-// Trilinear: levels l0 (weight 1 - t) and l1 (weight t; not read when t = 0);
-// stochastic: level l1 if xi < t else l0, weight 1 (Sec. 4.1).
-__device__ __forceinline__ void fetch_issue(const PyrDesc& P, const uint8_t* pyr, const QF& q, uint32_t stg) {
-  const float l = fminf(fmaxf(q.lod, 0.0f), (float)(P.levels - 1));  // NaN -> 0
-  const float fl = floorf(l);
-  const int l0 = (int)fl;
-  const int l1 = min(l0 + 1, P.levels - 1);
-  const float t = l - fl;
-  int la = l0, lb = l1;
-  float wa = 1.0f - t, wb = t;
-  if (P.filter == NAM_FILTER_STOCHASTIC) {
-    la = q.xi < t ? l1 : l0;
-    wa = 1.0f;
-    wb = 0.0f;
-  }
-  // the whole warp takes the general path if any lane needs it (huge or
-  // non-finite coordinates), so that the common case has no divergence
-  const bool in_range = fabsf(q.u * (float)P.w[0]) < 4194304.0f && fabsf(q.v * (float)P.h[0]) < 4194304.0f;
-  const bool fast = P.pow2 && P.address == NAM_ADDRESS_WRAP && __all_sync(0xffffffffu, in_range);
-  float w[8];
-  level_issue(P, pyr, la, q.u, q.v, fast, wa, true, stg, w);
-  level_issue(P, pyr, lb, q.u, q.v, fast, wb, wb != 0.0f, stg + 8192, w + 4);
-  ptx::st_shared_v4(stg + 16384, __float_as_uint(w[0]), __float_as_uint(w[1]), __float_as_uint(w[2]),
-                    __float_as_uint(w[3]));
-  ptx::st_shared_v4(stg + 16384 + 2048, __float_as_uint(w[4]), __float_as_uint(w[5]), __float_as_uint(w[6]),
-                    __float_as_uint(w[7]));
-  ptx::cp_async_commit();
-}
-
-// Wait for this thread's copies and filter: z = sum_k w_k texel_k in FP32.
-__device__ __forceinline__ void fetch_finish(uint32_t stg, float z[8]) {
-  ptx::cp_async_wait_all();
-  const uint4 wa = ptx::ld_shared_v4(stg + 16384), wb = ptx::ld_shared_v4(stg + 16384 + 2048);
-  const float w[8] = {f32_of(wa.x), f32_of(wa.y), f32_of(wa.z), f32_of(wa.w),
-                      f32_of(wb.x), f32_of(wb.y), f32_of(wb.z), f32_of(wb.w)};
-  float2 acc[4];
-#pragma unroll
-  for (int c = 0; c < 4; ++c) acc[c] = make_float2(0.0f, 0.0f);
-#pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    const uint4 t = ptx::ld_shared_v4(stg + k * 2048);
-    const __half2* h = reinterpret_cast<const __half2*>(&t);
-    const float2 wk = make_float2(w[k], w[k]);
-#pragma unroll
-    for (int c = 0; c < 4; ++c) acc[c] = ptx::fma2(wk, __half22float2(h[c]), acc[c]);
-  }
-#pragma unroll
-  for (int c = 0; c < 4; ++c) {
-    z[2 * c] = acc[c].x;
-    z[2 * c + 1] = acc[c].y;
-  }
-}
-
-// The same fetch for warps that do nothing else: the texels go through
-// registers (no staging, the other warps hide the latency).
+// Latent fetch of warps that do nothing else: the texels go through registers
+// (no staging, the other warps hide the latency).  Bilinear taps of level l
+// (Sec. 4.1; texel centres at (i + 1/2) / W): texel indices and weights wl *
+// (bilinear weight).
 // Power-of-two wrap, every lane's |u W0|, |v H0| < 2^22 - 1 (warp-uniform
 // `fast`): floor(x) comes from one round-down addition of 1.5 2^23, whose
 // result holds the integer in its low mantissa bits (no conversion
 // instructions, which run at a quarter of the rate), and W_l, H_l from the
 // exponents of level 0's sizes.
-// EXACT (the FP32 kernel): fractions and weights as in tap_axis and
-// bilinear_acc, bit for bit.
+// EXACT: fractions and weights as in tap_axis and bilinear_acc, bit for bit.
 template <bool EXACT>
 __device__ __forceinline__ void level_taps(const PyrDesc& P, int l, float u, float v, bool fast, int lw0, int lh0,
                                            float wl, uint32_t idx[4], float* w) {
@@ -399,12 +299,14 @@ __device__ __forceinline__ void fetch_direct(const PyrDesc& P, const uint8_t* py
 // The loop of one fetch warpgroup (fw of NF): it takes tiles fw, fw + NF, ...
 // of the CTA's range [c_begin, c_end), each warp its own 32 rows, and hands
 // tile t's filtered latents to the chains through ring entry t % NZ:
-// emit(slot, z) writes this row's; bar_f[slot] counts the four warps that
+// begin(tile) may start loads of its own, emit(slot, z) writes this row's;
+// bar_f[slot] counts the four warps that
 // filled it, bar_e[slot] its reading.  The next tile's query fields are in
 // flight while this tile's texels are.  False if a wait ran out.
-template <bool F16P, bool MULTI, bool EXACT, int NF, int NZ, class PyrFor, class RowOf, class Emit>
+template <bool F16P, bool MULTI, bool EXACT, int NF, int NZ, class PyrFor, class RowOf, class Begin, class Emit>
 __device__ __forceinline__ bool fetch_loop(const LaunchCommon& L, int64_t c_begin, int64_t c_end, int fw, uint32_t bar_f,
-                                           uint32_t bar_e, bool bad, PyrFor pyr_for, RowOf row_of, Emit emit) {
+                                           uint32_t bar_e, bool bad, PyrFor pyr_for, RowOf row_of, Begin begin,
+                                           Emit emit) {
   const int lw0 = 31 - __clz(L.pyr.w[0]), lh0 = 31 - __clz(L.pyr.h[0]);
   int64_t c = c_begin + fw;
   int slot = fw, pass = 0;
@@ -421,6 +323,7 @@ __device__ __forceinline__ bool fetch_loop(const LaunchCommon& L, int64_t c_begi
       nxt = tile_at(L, c + NF);
       if (nxt.count > 0) qn = load_qf<MULTI>(L.q, row_of(nxt));
     }
+    if (cur.count > 0) begin(cur);
     float z[8];
     if (cur.count > 0) fetch_direct<F16P, EXACT>(L.pyr, pyr_for(cur), q, lw0, lh0, z);
     // the entry's previous latents have been read
@@ -599,8 +502,10 @@ __global__ void __launch_bounds__((NCH + NF) * 128, 1) eval_f16_kernel(const __g
     auto pyr_for = [&](const TileRef& t) -> const uint8_t* {
       return reinterpret_cast<const uint8_t*>(MULTI ? L.mats.pyramid[t.mat] : L.pyr0);
     };
-    bad = !fetch_loop<F16P, MULTI, false, NF, NZ>(
-        L, c_begin, c_end, wg - NCH, bar_f, bar_e, bad, pyr_for, row_of, [&](int slot, const float z[8]) {
+    // (FP32 texels: bilinear_acc's operation order)
+    bad = !fetch_loop<F16P, MULTI, !F16P, NF, NZ>(
+        L, c_begin, c_end, wg - NCH, bar_f, bar_e, bad, pyr_for, row_of, [](const TileRef&) {},
+        [&](int slot, const float z[8]) {
           uint32_t v[8];
           split_pair<false>(z[0], z[1], v[0], v[4]);
           split_pair<false>(z[2], z[3], v[1], v[5]);

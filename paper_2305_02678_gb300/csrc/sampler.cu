@@ -6,14 +6,17 @@
 // Sampler weights (FP32 masters) are laid out per layer as W (out x in) then
 // b (out).
 //
-// The MLP runs on the tensor cores at FP32 accuracy, tiles of 128 queries
-// per warpgroup as in the evaluation kernel (thread r = query r = TMEM lane
-// r).  Each weight is split into two binary16 values, W = W_hi + W_lo, and
-// each layer input into x = x_hi + x_lo (hi: x with its 13 low mantissa bits
-// cleared, exact in binary16); one MMA over [x_hi | x_lo | 1 1] x [W_hi |
-// W_hi | b_hi b_lo] and one over x_hi x W_lo give W x + b up to the dropped
-// W_lo x_lo term, a relative 2^-22.  The proxy's activations, density and
-// sampling run per thread in FP32.
+// The MLP runs on the tensor cores at FP32 accuracy, tiles of 128 queries as
+// in the evaluation kernel: fetch warpgroups filter the latents and write
+// layer 1's operand, chain warpgroups (thread r = query r = TMEM lane r) take
+// a tile through the four layers.  Each weight is split into two binary16
+// values, W = W_hi + W_lo, and each layer input into x = x_hi + x_lo (hi: x
+// with its 13 low mantissa bits cleared, exact in binary16); one MMA over
+// [x_hi | x_lo | 1 1] x [W_hi | W_hi | b_hi b_lo] and one over x_hi x W_lo give
+// W x + b up to the dropped W_lo x_lo term, a relative 2^-22.  The proxy's
+// activations, density and sampling run per thread in FP32.
+// What bounds it: instruction issue (73 % of the slots); 1920x1080, sample and
+// density: 97 us, 146 with the fetch in the chains' own warps.
 #include <cuda_runtime.h>
 
 #include "eval_tc.cuh"
@@ -130,39 +133,41 @@ __device__ __forceinline__ void sample_dir(const Proxy& p, const float wi[3], fl
 constexpr int kSA1 = 0, kSL1 = 2048, kSA2 = 3072, kSL2 = 8192, kSA3 = 10240, kSL3 = 15360, kSA4 = 17408,
               kSL4 = 19968, kSamplerBlobBytes = 20992;
 
-// TMEM columns of one warpgroup: the accumulator [0, 32), the A operand
-// [32, 72): (x_hi, x_lo) of layer 1 in [32, 48); (h_hi, h_lo, 1 1 0 ...) of
-// the later layers in [32, 72), the constant pair (1, 1) at column 64 written
-// once.
+// TMEM columns of one chain: the accumulator [0, 32), the A operand of layers
+// 2 to 4 [32, 72): (h_hi, h_lo, 1 1 0 ...), the constant pair (1, 1) at
+// column 64 written once.  Layer 1's operand comes from shared memory.
 constexpr int kSD = 0, kSA = 32, kSCols = 72;
-constexpr int kSamplerNwg = 5;
 
-template <bool F16P, int NWG>
+template <int NCH, int NF>
 struct SamplerSmem {
-  static constexpr int STG_OFF = kSamplerBlobBytes;
-  static constexpr int STG = F16P ? kStageBytes : 0;
-  static constexpr int BAR_OFF = STG_OFF + NWG * STG;
-  static constexpr int BYTES = BAR_OFF + NWG * 8 + 8 + 16;
+  static constexpr int ZB = 8192;  // layer 1's operand: (x_hi, x_lo), 16 wide each, of 128 rows
+  static constexpr int NZ = NCH % NF ? NCH * NF : NCH;  // as F16Smem::NZ
+  static constexpr int Z_OFF = kSamplerBlobBytes;
+  static constexpr int BAR_OFF = Z_OFF + NZ * ZB;
+  static constexpr int BYTES = BAR_OFF + (NCH + 2 * NZ + 1) * 8 + 16;
 };
 
-template <bool F16P, int NWG>
-__global__ void __launch_bounds__(NWG * 128, 1)
-    sampler_tc_kernel(const LaunchCommon L, const uint8_t* __restrict__ blob, int mode, const float* __restrict__ u,
-                      float* __restrict__ wo_out, float* __restrict__ pdf_out) {
-  using S = SamplerSmem<F16P, NWG>;
+template <bool F16P, int NCH, int NF>
+__global__ void __launch_bounds__((NCH + NF) * 128, 1)
+    sampler_tc_kernel(const __grid_constant__ LaunchCommon L, const uint8_t* __restrict__ blob, int mode,
+                      const float* __restrict__ u, float* __restrict__ wo_out, float* __restrict__ pdf_out) {
+  using S = SamplerSmem<NCH, NF>;
+  constexpr int NZ = S::NZ;
   extern __shared__ __align__(1024) uint8_t smem[];
-  const int tid = threadIdx.x, wg = tid >> 7, r = tid & 127, warp = tid >> 5;
+  const int tid = threadIdx.x, r = tid & 127;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0), wg = warp >> 2;
   const uint32_t aW = ptx::smem_u32(smem);
-  const uint32_t stg = ptx::smem_u32(smem + S::STG_OFF + wg * S::STG) + r * 16;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + S::BAR_OFF);
-  const uint32_t bar_m = ptx::smem_u32(&bars[wg]);
-  const uint32_t bar_w = ptx::smem_u32(&bars[NWG]);
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(smem + S::BAR_OFF + NWG * 8 + 8);
-  const uint32_t bar_id = 1 + wg;
+  const uint32_t bar0 = ptx::smem_u32(smem + S::BAR_OFF);
+  const uint32_t bar_f = bar0 + 8 * NCH, bar_e = bar0 + 8 * (NCH + NZ), bar_w = bar0 + 8 * (NCH + 2 * NZ);
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(smem + S::BAR_OFF + (NCH + 2 * NZ + 1) * 8);
 
-  if (r == 0) {
-    ptx::mbar_init(bar_m, 1);
-    if (tid == 0) ptx::mbar_init(bar_w, 1);
+  if (tid == 0) {
+    for (int k = 0; k < NCH; ++k) ptx::mbar_init(bar0 + 8 * k, 1);
+    for (int k = 0; k < NZ; ++k) {
+      ptx::mbar_init(bar_f + 8 * k, 4);  // the four warps of a fetch warpgroup
+      ptx::mbar_init(bar_e + 8 * k, 1);
+    }
+    ptx::mbar_init(bar_w, 1);
     ptx::fence_mbar_init();
   }
   if (warp == 0) {
@@ -172,186 +177,179 @@ __global__ void __launch_bounds__(NWG * 128, 1)
   ptx::tc_fence_before();
   __syncthreads();
   ptx::tc_fence_after();
-  const uint32_t tmem = *tslot;
-  const uint32_t tB = tmem + wg * kSCols;
-  const uint32_t tBl = tB + ((uint32_t)((warp & 3) * 32) << 16);
+  constexpr uint32_t tmem = 0;  // all 512 columns are allocated
 
   const int64_t ntiles = (L.n + 127) / 128;
   const int64_t per = (ntiles + gridDim.x - 1) / gridDim.x;
   const int64_t c_begin = (int64_t)blockIdx.x * per;
   const int64_t c_end = c_begin + per < ntiles ? c_begin + per : ntiles;
-
+  bool bad = *tslot != tmem, mma_pending = false, w_pending = false;
   uint32_t ph_m = 0;
-  bool bad = false, mma_pending = false, w_pending = false;
-  if (tid == 0 && c_begin < c_end) {
-    ptx::fence_proxy_async();
-    ptx::mbar_arrive_expect_tx(bar_w, kSamplerBlobBytes);
-    ptx::bulk_g2s(aW, blob, kSamplerBlobBytes, bar_w);
-    w_pending = true;
-  }
-  {
-    // the constant pair (1, 1) that meets the bias columns (b_hi, b_lo)
-    uint32_t one[8] = {0x3C003C00u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
-    ptx::tmem_st8(tBl + kSA + 32, one);
-  }
-  constexpr uint32_t ID32 = ptx::idesc_f16(128, 32);
-  constexpr uint32_t ID16 = ptx::idesc_f16(128, 16);
+  auto row_of = [&](const TileRef& t) -> int64_t { return t.start + (r < t.count ? r : 0); };
 
-  auto stage_issue = [&](auto issue) -> bool {
-    ptx::tmem_st_wait();
-    ptx::tc_fence_before();
-    if (ptx::bar_red_or(bar_id, 128, bad)) {
-      bad = true;
-      return false;
+  if (wg >= NCH) {
+    // ---- fetch: layer 1's input (z, wi, 1) as (hi, lo) -----------------------
+    float wx, wy, wz;
+    bad = !fetch_loop<F16P, false, !F16P, NF, NZ>(
+        L, c_begin, c_end, wg - NCH, bar_f, bar_e, bad,
+        [&](const TileRef&) { return reinterpret_cast<const uint8_t*>(L.pyr0); }, row_of,
+        [&](const TileRef& t) {
+          const int64_t i = row_of(t);
+          wx = ptx::ld_nc_pinned(L.q.wix + i);
+          wy = ptx::ld_nc_pinned(L.q.wiy + i);
+          wz = ptx::ld_nc_pinned(L.q.wiz + i);
+        },
+        [&](int slot, const float z[8]) {
+          uint32_t v[16];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) split_pair<false>(z[2 * j], z[2 * j + 1], v[j], v[8 + j]);
+          split_pair<false>(wx, wy, v[4], v[12]);
+          split_pair<false>(wz, 1.0f, v[5], v[13]);
+          v[13] = (v[13] & 0x0000FFFFu) | 0x3C000000u;  // lo block: the 1 meets b1_lo
+          v[6] = v[7] = v[14] = v[15] = 0u;
+          const uint32_t zs = aW + S::Z_OFF + slot * S::ZB + r * 16;
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            ptx::st_shared_v4(zs + j * 2048, v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+          ptx::fence_proxy_async();
+        });
+  } else {
+    // ---- chains ---------------------------------------------------------------
+    const uint32_t bar_m = bar0 + 8 * wg, bar_id = 1 + wg;
+    const uint32_t tB = tmem + wg * kSCols;
+    const uint32_t tBl = tB + ((uint32_t)((warp & 3) * 32) << 16);
+    if (tid == 0 && c_begin < c_end) {
+      ptx::fence_proxy_async();
+      ptx::mbar_arrive_expect_tx(bar_w, kSamplerBlobBytes);
+      ptx::bulk_g2s(aW, blob, kSamplerBlobBytes, bar_w);
+      w_pending = true;
     }
-    if (r == 0) {
+    {
+      // the constant pair (1, 1) that meets the bias columns (b_hi, b_lo)
+      uint32_t one[8] = {0x3C003C00u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+      ptx::tmem_st8(tBl + kSA + 32, one);
+    }
+    constexpr uint32_t ID32 = ptx::idesc_f16(128, 32);
+    constexpr uint32_t ID16 = ptx::idesc_f16(128, 16);
+    auto leader = [&]() -> bool { return ((warp ^ wg) & 3) == 0 && ptx::elect(); };
+
+    auto stage_issue = [&](auto issue) -> bool {
+      ptx::tmem_st_wait();
+      ptx::tc_fence_before();
+      if (ptx::bar_red_or(bar_id, 128, bad)) {
+        bad = true;
+        return false;
+      }
+      if (leader()) {
+        ptx::tc_fence_after();
+        issue();
+        ptx::mma_commit(bar_m);
+      }
+      mma_pending = true;
+      return true;
+    };
+    auto stage_wait = [&]() {
+      bad |= !ptx::mbar_wait(bar_m, ph_m, L.timeout_ns);
+      ph_m ^= 1;
+      if (!bad) mma_pending = false;
       ptx::tc_fence_after();
-      issue();
-      ptx::mma_commit(bar_m);
-    }
-    mma_pending = true;
-    return true;
-  };
-  auto stage_wait = [&]() {
-    bad |= !ptx::mbar_wait(bar_m, ph_m, L.timeout_ns);
-    ph_m ^= 1;
-    if (!bad) mma_pending = false;
-    ptx::tc_fence_after();
-  };
-  // ReLU of the 32 accumulator columns, split into (h_hi, h_lo), 16 at a time
-  auto hidden_operand = [&]() {
+    };
+    // ReLU of the 32 accumulator columns, split into (h_hi, h_lo), 16 at a time
+    auto hidden_operand = [&]() {
 #pragma unroll
-    for (int c0 = 0; c0 < 32; c0 += 16) {
-      uint32_t acc[16];
-      ptx::tmem_ld16(tBl + kSD + c0, acc);
-      ptx::tmem_ld_wait();
-      uint32_t hi[8], lo[8];
+      for (int c0 = 0; c0 < 32; c0 += 16) {
+        uint32_t acc[16];
+        ptx::tmem_ld16(tBl + kSD + c0, acc);
+        ptx::tmem_ld_wait();
+        uint32_t hi[8], lo[8];
 #pragma unroll
-      for (int j = 0; j < 8; ++j) split_pair<true>(f32_of(acc[2 * j]), f32_of(acc[2 * j + 1]), hi[j], lo[j]);
-      ptx::tmem_st8(tBl + kSA + c0 / 2, hi);
-      ptx::tmem_st8(tBl + kSA + 16 + c0 / 2, lo);
-    }
-  };
-  // one hidden or output layer: [h_hi | h_lo | 1 1] x [W_hi | W_hi | b], then h_hi x W_lo
-  auto layer_mmas = [&](int a_off, int l_off, int rows, uint32_t id) {
-    const uint32_t lbo = (uint32_t)rows * 16, step = (uint32_t)rows * 32;
+        for (int j = 0; j < 8; ++j) split_pair<true>(f32_of(acc[2 * j]), f32_of(acc[2 * j + 1]), hi[j], lo[j]);
+        ptx::tmem_st8(tBl + kSA + c0 / 2, hi);
+        ptx::tmem_st8(tBl + kSA + 16 + c0 / 2, lo);
+      }
+    };
+    // one hidden or output layer: [h_hi | h_lo | 1 1] x [W_hi | W_hi | b], then h_hi x W_lo
+    auto layer_mmas = [&](int a_off, int l_off, int rows, uint32_t id) {
+      const uint32_t lbo = (uint32_t)rows * 16, step = (uint32_t)rows * 32;
 #pragma unroll
-    for (int s = 0; s < 5; ++s)
-      ptx::mma_f16_ts(tB + kSD, tB + kSA + 8 * s, ptx::sdesc(aW + a_off + s * step, lbo, 128), id, s > 0 ? 1u : 0u);
+      for (int s = 0; s < 5; ++s)
+        ptx::mma_f16_ts(tB + kSD, tB + kSA + 8 * s, ptx::sdesc(aW + a_off + s * step, lbo, 128), id, s > 0 ? 1u : 0u);
 #pragma unroll
-    for (int s = 0; s < 2; ++s)
-      ptx::mma_f16_ts(tB + kSD, tB + kSA + 8 * s, ptx::sdesc(aW + l_off + s * step, lbo, 128), id, 1u);
-  };
+      for (int s = 0; s < 2; ++s)
+        ptx::mma_f16_ts(tB + kSD, tB + kSA + 8 * s, ptx::sdesc(aW + l_off + s * step, lbo, 128), id, 1u);
+    };
 
-  int64_t c = c_begin + wg;
-  QF q_nxt{};
-  bool w_ready = false;
-  float zr[8];  // filtered latent of the tile about to start (FP16 pyramids)
-  if (c < c_end) {
-    const int64_t i0 = c * 128 + r;
-    const QF q0 = load_qf<true>(L.q, i0 < L.n ? i0 : L.n - 1);
-    if (F16P) {
-      fetch_issue(L.pyr, reinterpret_cast<const uint8_t*>(L.pyr0), q0, stg);
-      fetch_finish(stg, zr);
-    }
-    if (c + NWG < c_end) {
-      const int64_t i1 = (c + NWG) * 128 + r;
-      q_nxt = load_qf<true>(L.q, i1 < L.n ? i1 : L.n - 1);
-    }
-  }
-  for (; c < c_end; c += NWG) {
-    const bool has_next = c + NWG < c_end, has_next2 = c + 2 * NWG < c_end;
-    const int64_t i_raw = c * 128 + r;
-    const bool valid = i_raw < L.n;
-    const int64_t i = valid ? i_raw : L.n - 1;
-    const float wi[3] = {ptx::ld_nc_pinned(L.q.wix + i), ptx::ld_nc_pinned(L.q.wiy + i),
-                         ptx::ld_nc_pinned(L.q.wiz + i)};
-    if (!w_ready) {
-      bad |= !ptx::mbar_wait(bar_w, 0, L.timeout_ns);
-      if (!bad && tid == 0) w_pending = false;
-      w_ready = true;
-    }
-    // ---- layer 1 input (z, wi, 1) as (hi, lo) ------------------------------
-    float x[16];
-    if (F16P) {
-      // filtered while the previous tile's last layer ran
+    int slot = wg;
+    uint32_t ph_f = 0;
+    bool w_ready = false;
+    for (int64_t c = c_begin + wg; c < c_end; c += NCH) {
+      const int64_t i_raw = c * 128 + r;
+      const bool valid = i_raw < L.n;
+      const int64_t i = valid ? i_raw : L.n - 1;
+      if (!w_ready) {
+        bad |= !ptx::mbar_wait(bar_w, 0, L.timeout_ns);
+        if (!bad && tid == 0) w_pending = false;
+        w_ready = true;
+      }
+      const uint32_t aZ = aW + S::Z_OFF + slot * S::ZB, be = bar_e + 8 * slot;
+      bad |= !ptx::mbar_wait(bar_f + 8 * slot, ph_f, L.timeout_ns);
+      slot += NCH;
+      if (slot >= NZ) {
+        slot -= NZ;
+        ph_f ^= 1u;
+      }
+      if (!stage_issue([&] {
 #pragma unroll
-      for (int k = 0; k < 8; ++k) x[k] = zr[k];
-    } else {
-      const QF q0 = load_qf<true>(L.q, i);
-      fetch_latent<false>(L.pyr, L.pyr0, q0.u, q0.v, q0.lod, q0.xi, x);
-    }
-    x[8] = wi[0];
-    x[9] = wi[1];
-    x[10] = wi[2];
-    x[11] = 1.0f;
-    x[12] = x[13] = x[14] = x[15] = 0.0f;
-    {
-      uint32_t v[16];
+            for (int s = 0; s < 2; ++s)
+              ptx::mma_f16(tB + kSD, ptx::sdesc(aZ + s * 4096, 2048, 128), ptx::sdesc(aW + kSA1 + s * 1024, 512, 128),
+                           ID32, s > 0 ? 1u : 0u);
+            ptx::mma_f16(tB + kSD, ptx::sdesc(aZ, 2048, 128), ptx::sdesc(aW + kSL1, 512, 128), ID32, 1u);
+            ptx::mma_commit(be);
+          }))
+        break;
+      const float wi[3] = {ptx::ld_nc_pinned(L.q.wix + i), ptx::ld_nc_pinned(L.q.wiy + i),
+                           ptx::ld_nc_pinned(L.q.wiz + i)};
+      stage_wait();
+      // ---- layers 2, 3 (32 -> 32) and 4 (32 -> 9) -----------------------------
+      hidden_operand();
+      if (!stage_issue([&] { layer_mmas(kSA2, kSL2, 32, ID32); })) break;
+      stage_wait();
+      hidden_operand();
+      if (!stage_issue([&] { layer_mmas(kSA3, kSL3, 32, ID32); })) break;
+      stage_wait();
+      hidden_operand();
+      if (!stage_issue([&] { layer_mmas(kSA4, kSL4, 16, ID16); })) break;
+      stage_wait();
+      // ---- proxy parameters, density or sample --------------------------------
+      float o[9];
+      {
+        uint32_t acc[16];
+        ptx::tmem_ld16(tBl + kSD, acc);
+        ptx::tmem_ld_wait();
 #pragma unroll
-      for (int j = 0; j < 8; ++j) split_pair<false>(x[2 * j], x[2 * j + 1], v[j], v[8 + j]);
-      v[8 + 5] = (v[8 + 5] & 0x0000FFFFu) | 0x3C000000u;  // lo block: the 1 meets b1_lo
-      ptx::tmem_st16(tBl + kSA, v);
-    }
-    if (!stage_issue([&] {
-#pragma unroll
-          for (int s = 0; s < 2; ++s)
-            ptx::mma_f16_ts(tB + kSD, tB + kSA + 8 * s, ptx::sdesc(aW + kSA1 + s * 1024, 512, 128), ID32,
-                            s > 0 ? 1u : 0u);
-          ptx::mma_f16_ts(tB + kSD, tB + kSA, ptx::sdesc(aW + kSL1, 512, 128), ID32, 1u);
-        }))
-      break;
-    // the next tile's texel gathers while layer 1 runs
-    QF q_nxt2{};
-    if (F16P && has_next) fetch_issue(L.pyr, reinterpret_cast<const uint8_t*>(L.pyr0), q_nxt, stg);
-    if (has_next2) {
-      const int64_t i2 = (c + 2 * NWG) * 128 + r;
-      q_nxt2 = load_qf<true>(L.q, i2 < L.n ? i2 : L.n - 1);
-    }
-    stage_wait();
-    // ---- layers 2, 3 (32 -> 32) and 4 (32 -> 9) -----------------------------
-    hidden_operand();
-    if (!stage_issue([&] { layer_mmas(kSA2, kSL2, 32, ID32); })) break;
-    stage_wait();
-    hidden_operand();
-    if (!stage_issue([&] { layer_mmas(kSA3, kSL3, 32, ID32); })) break;
-    stage_wait();
-    hidden_operand();
-    if (!stage_issue([&] { layer_mmas(kSA4, kSL4, 16, ID16); })) break;
-    // the next tile's filter, while the last layer runs
-    if (F16P && has_next) fetch_finish(stg, zr);
-    stage_wait();
-    // ---- proxy parameters, density or sample --------------------------------
-    float o[9];
-    {
-      uint32_t acc[16];
-      ptx::tmem_ld16(tBl + kSD, acc);
-      ptx::tmem_ld_wait();
-#pragma unroll
-      for (int j = 0; j < 9; ++j) o[j] = f32_of(acc[j]);
-    }
-    ptx::tc_fence_before();
-    if (valid) {
-      const Proxy p = activate(o);
-      if (mode == 0) {
-        const float wo[3] = {L.q.wox[i], L.q.woy[i], L.q.woz[i]};
-        pdf_out[i] = pdf_full(p, wi, wo);
-      } else {
-        float wo[3];
-        sample_dir(p, wi, u[3 * i], u[3 * i + 1], u[3 * i + 2], wo);
-        wo_out[3 * i] = wo[0];
-        wo_out[3 * i + 1] = wo[1];
-        wo_out[3 * i + 2] = wo[2];
-        if (pdf_out) pdf_out[i] = pdf_full(p, wi, wo);
+        for (int j = 0; j < 9; ++j) o[j] = f32_of(acc[j]);
+      }
+      ptx::tc_fence_before();
+      if (valid) {
+        const Proxy p = activate(o);
+        if (mode == 0) {
+          const float wo[3] = {L.q.wox[i], L.q.woy[i], L.q.woz[i]};
+          pdf_out[i] = pdf_full(p, wi, wo);
+        } else {
+          float wo[3];
+          sample_dir(p, wi, u[3 * i], u[3 * i + 1], u[3 * i + 2], wo);
+          wo_out[3 * i] = wo[0];
+          wo_out[3 * i + 1] = wo[1];
+          wo_out[3 * i + 2] = wo[2];
+          if (pdf_out) pdf_out[i] = pdf_full(p, wi, wo);
+        }
       }
     }
-    q_nxt = q_nxt2;
   }
 
   // ---- teardown (as in the evaluation kernel) --------------------------------
-  ptx::cp_async_wait_all();
   bool drained = true;
-  if (r == 0 && mma_pending) drained &= ptx::mbar_wait(bar_m, ph_m ^ 1, ptx::kDrainTimeoutNs);
+  if (r == 0 && mma_pending) drained &= ptx::mbar_wait(bar0 + 8 * wg, ph_m ^ 1, ptx::kDrainTimeoutNs);
   if (tid == 0 && w_pending) drained &= ptx::mbar_wait(bar_w, 0, ptx::kDrainTimeoutNs);
   if (bad) record_error(L.err, DEVERR_WAIT_TIMEOUT);
   if (!drained) record_error(L.err, DEVERR_DRAIN_TIMEOUT);
@@ -359,7 +357,7 @@ __global__ void __launch_bounds__(NWG * 128, 1)
   const bool all_drained = __syncthreads_and(drained ? 1 : 0) != 0;
   if (warp == 0 && all_drained) {
     ptx::tc_fence_after();
-    ptx::tmem_dealloc(tmem, 512);
+    ptx::tmem_dealloc(*tslot, 512);
   }
 }
 
@@ -428,11 +426,13 @@ int pack_sampler_blob(const float* w, uint8_t* out) {
 template <bool F16P>
 static int launch_sampler_tc(const LaunchCommon& L, const void* blob, int mode, const float* u, float* wo_out,
                              float* pdf_out, cudaStream_t s) {
-  constexpr int NWG = kSamplerNwg;
-  using S = SamplerSmem<F16P, NWG>;
+  // six chains (TMEM 6 x 72 columns) and two fetch warpgroups, 1024 threads at
+  // <= 64 registers (1920x1080, sample and density: 97 us; 5 + 2 99, 4 + 2 109)
+  constexpr int NCH = 6, NF = 2;
+  using S = SamplerSmem<NCH, NF>;
   static_assert(S::BYTES <= 227 * 1024, "shared memory");
-  static_assert(NWG * kSCols <= 512, "TMEM columns");
-  auto k = sampler_tc_kernel<F16P, NWG>;
+  static_assert(NCH * kSCols <= 512, "TMEM columns");
+  auto k = sampler_tc_kernel<F16P, NCH, NF>;
   static std::atomic<uint64_t> configured{0};
   once_per_device(configured, [&] {
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, S::BYTES);
@@ -440,9 +440,8 @@ static int launch_sampler_tc(const LaunchCommon& L, const void* blob, int mode, 
     cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
   });
   const int64_t ntiles = (L.n + 127) / 128;
-  const int64_t want = (ntiles + NWG - 1) / NWG;
-  const int grid = (int)(want < L.num_sms ? want : L.num_sms);
-  k<<<grid, NWG * 128, S::BYTES, s>>>(L, reinterpret_cast<const uint8_t*>(blob), mode, u, wo_out, pdf_out);
+  const int grid = (int)(ntiles < L.num_sms ? ntiles : L.num_sms);
+  k<<<grid, (NCH + NF) * 128, S::BYTES, s>>>(L, reinterpret_cast<const uint8_t*>(blob), mode, u, wo_out, pdf_out);
   return (int)cudaGetLastError();
 }
 

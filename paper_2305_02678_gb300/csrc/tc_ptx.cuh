@@ -296,16 +296,6 @@ __device__ __forceinline__ float2 sub2(float2 a, float2 b) {
   asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(rd) : "l"(ra), "l"(rb));
   return *reinterpret_cast<float2*>(&rd);
 }
-// 16-byte global -> shared copy through L1 (cp.async, completes into the
-// issuing thread's current group); src_size < 16 fills the rest with zeros
-// (0: nothing is read).
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, uint32_t src_size) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(src_size) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-// All but this thread's newest committed group have completed.
-__device__ __forceinline__ void cp_async_wait_1() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
 // Read-only global load that the compiler keeps where it is written (the
 // value's first use waits on it, wherever that is).
 __device__ __forceinline__ float ld_nc_pinned(const float* p) {

@@ -67,3 +67,30 @@ def test_many_chunks_per_cta_mixed_materials(gctx):
         assert torch.equal(out[idx], _pieces(m, sub, idx.numel(), sms * 128)), k
         m.destroy()
     gctx.check()
+
+
+@pytest.mark.parametrize("latent", [np.float16, np.float32])
+def test_sampler_many_tiles_per_cta(gctx, latent):
+    import torch
+    from paper_2305_02678_gb300 import binding as B
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    rng = W.rng_streams(143, 5)
+    model = W.make_model(rng[0], (14, 16, 16, 3), None)
+    mat = gctx.material(128, 128, 8, W.make_pyramid(rng[1], 128, 128, 8, dtype=latent), None, model["decoder"],
+                        sampler=W.make_mlp(rng[2], (11, 32, 32, 32, 9)))
+    n, size = sms * 128 * 20 + 33, sms * 128
+    dq = to_device(W.uniform_queries(rng[3], n, 7.0))
+    u = torch.from_numpy(rng[4].random((n, 3), dtype=np.float32)).cuda()
+
+    def sample(a, b):
+        wo, pdf = torch.empty((b - a, 3), device="cuda"), torch.empty(b - a, device="cuda")
+        B.nam_sample(gctx.h, mat.h, {k: t[a:b] for k, t in dq.items()}, b - a, u[a:b], wo, pdf,
+                     torch.cuda.current_stream())
+        return wo, pdf
+
+    wo, pdf = sample(0, n)
+    parts = [sample(a, min(a + size, n)) for a in range(0, n, size)]
+    assert torch.equal(wo, torch.cat([p[0] for p in parts]))
+    assert torch.equal(pdf, torch.cat([p[1] for p in parts]))
+    mat.destroy()
+    gctx.check()
