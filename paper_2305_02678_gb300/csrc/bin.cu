@@ -7,8 +7,8 @@
 //           histogram: same-address atomics serialise in L2);
 //   plan    exclusive scan of the counts into per-material cursors, and the
 //           chunk table of the tensor-core kernel (each material's range cut
-//           into 128-query chunks; empty slots have count 0; the number of
-//           chunks in use for the kernel to read on the device);
+//           into 128-query chunks; the number of chunks in use for the
+//           kernel to read on the device);
 //   permute each block reserves, per material, one run of slots for its
 //           segment (one global atomic per block and material) and writes
 //           each query's index to a slot of its run;
@@ -36,12 +36,21 @@ __device__ __forceinline__ uint32_t lanemask_lt() {
   return m;
 }
 
-constexpr int kSeg = 1024;  // queries per block in count and scatter
+// Queries per block in count and scatter: eight per thread, whose ids are all
+// loaded before the first is used (one memory latency per block, not one per
+// round); larger segments also mean fewer same-address atomics on the
+// per-material totals.  1920x1080, 16 materials drawn per pixel: count 18 us
+// and permute 36 us with 1024-query segments read round by round.
+constexpr int kPer = 8;
+constexpr int kSeg = kThreads * kPer;
 
 // warp-aggregated add of 1 per lane to cnt[m] in shared memory; returns the
 // value this lane's increment starts from
 __device__ __forceinline__ uint32_t warp_bump(uint32_t* cnt, int m, uint32_t act) {
-  const uint32_t same = __match_any_sync(act, m);
+  // (a warp whose lanes share one material needs no match)
+  const int first = __ffs(act) - 1;
+  const int m0 = __shfl_sync(act, m, first);
+  const uint32_t same = __all_sync(act, m == m0) ? act : __match_any_sync(act, m);
   const int leader = __ffs(same) - 1;
   uint32_t base = 0;
   if ((int)(threadIdx.x & 31) == leader) base = atomicAdd(cnt + m, (uint32_t)__popc(same));
@@ -50,79 +59,123 @@ __device__ __forceinline__ uint32_t warp_bump(uint32_t* cnt, int m, uint32_t act
 
 // A query takes part in binning unless `tile_k` is given and its 128-query
 // tile's entry there is non-negative (a tile the selection passes handle).
-__device__ __forceinline__ bool binned_query(const int32_t* tile_k, int64_t i) {
-  return tile_k == nullptr || __ldg(tile_k + (i >> 7)) < 0;
+// Loads this thread's kPer ids of the segment (-1: absent, not binned, or out
+// of range).
+__device__ __forceinline__ void load_ids(const int32_t* __restrict__ ids, int64_t seg, int64_t end, int nmat,
+                                         const int32_t* __restrict__ tile_k, int (&m)[kPer], int* err) {
+  uint32_t part = 0;  // bit j: query j of this thread takes part
+#pragma unroll
+  for (int j = 0; j < kPer; ++j) {
+    const int64_t i = seg + j * kThreads + threadIdx.x;
+    m[j] = i < end ? __ldg(ids + i) : -1;
+    if (i < end && (tile_k == nullptr || __ldg(tile_k + (i >> 7)) < 0)) part |= 1u << j;
+  }
+  bool bad = false;
+#pragma unroll
+  for (int j = 0; j < kPer; ++j) {
+    const bool in = m[j] >= 0 && m[j] < nmat, p = (part >> j) & 1u;
+    bad |= p && !in;
+    if (!p || !in) m[j] = -1;
+  }
+  if (bad && err) record_error(err, DEVERR_BOUNDS);
 }
 
 __global__ void __launch_bounds__(kThreads) bin_count_kernel(const int32_t* __restrict__ ids, int64_t n, int nmat,
                                                              const int32_t* __restrict__ tile_k,
                                                              uint32_t* __restrict__ counts, int* err) {
   extern __shared__ uint32_t cnt[];  // [nmat]
-  for (int m = threadIdx.x; m < nmat; m += blockDim.x) cnt[m] = 0;
-  __syncthreads();
   const int64_t seg = (int64_t)blockIdx.x * kSeg;
   const int64_t end = seg + kSeg < n ? seg + kSeg : n;
-  for (int64_t base = seg; base < end; base += blockDim.x) {
-    const int64_t i = base + threadIdx.x;
-    int m = -1;
-    if (i < end && binned_query(tile_k, i)) {
-      m = __ldg(ids + i);
-      if (m < 0 || m >= nmat) {
-        record_error(err, DEVERR_BOUNDS);
-        m = -1;
-      }
+  int id[kPer];
+  load_ids(ids, seg, end, nmat, tile_k, id, err);
+  for (int m = threadIdx.x; m < nmat; m += blockDim.x) cnt[m] = 0;
+  __syncthreads();
+#pragma unroll
+  for (int j = 0; j < kPer; ++j) {
+    const uint32_t act = __ballot_sync(0xffffffffu, id[j] >= 0);
+    if (id[j] < 0) continue;
+    // one add per warp of one material, else one per lane (no result needed)
+    const int first = __ffs(act) - 1;
+    if (__all_sync(act, id[j] == __shfl_sync(act, id[j], first))) {
+      if ((int)(threadIdx.x & 31) == first) atomicAdd(cnt + id[j], (uint32_t)__popc(act));
+    } else {
+      atomicAdd(cnt + id[j], 1u);
     }
-    const uint32_t act = __ballot_sync(0xffffffffu, m >= 0);
-    if (m >= 0) warp_bump(cnt, m, act);
   }
   __syncthreads();
   for (int m = threadIdx.x; m < nmat; m += blockDim.x)
     if (cnt[m]) atomicAdd(counts + m, cnt[m]);
 }
 
-// One block: cursors[m] = sum of counts before m; chunks[c] for every slot
-// c < max_chunks (a material with k queries owns ceil(k / 128) chunks);
-// *n_used = the chunks in use (the tensor-core kernel's table length).
+// inclusive scan over a warp
+template <class T>
+__device__ __forceinline__ T warp_scan(T x) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const T y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  return x;
+}
+
+// cursors[m] = sum of counts before m; chunks[c] for every slot c in use (a
+// material with k queries owns ceil(k / 128) chunks); *n_used = the chunks in
+// use (the tensor-core kernel's table length).  Every block scans the counts
+// for itself and writes its share of the table (one block: 8.7 us at
+// 1920x1080).
 __global__ void __launch_bounds__(1024) bin_plan_kernel(const uint32_t* __restrict__ counts, int nmat,
                                                         uint32_t* __restrict__ cursors, Chunk* __restrict__ chunks,
-                                                        int32_t max_chunks, int32_t* __restrict__ n_used) {
+                                                        int32_t* __restrict__ n_used) {
   extern __shared__ uint32_t sh[];
   uint32_t* qoff = sh;             // [nmat + 1] first query of each material
   uint32_t* coff = sh + nmat + 1;  // [nmat + 1] first chunk of each material
-  if (threadIdx.x == 0) {
-    uint32_t q = 0, c = 0;
-    for (int m = 0; m < nmat; ++m) {
-      qoff[m] = q;
-      coff[m] = c;
-      q += counts[m];
-      c += (counts[m] + 127) / 128;
+  __shared__ uint32_t wq[32], wc[32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint32_t carry_q = 0, carry_c = 0;
+  for (int base = 0; base < nmat; base += 1024) {
+    const int m = base + threadIdx.x;
+    const uint32_t q = m < nmat ? counts[m] : 0u, c = (q + 127) / 128;
+    const uint32_t sq = warp_scan(q), sc = warp_scan(c);
+    if (lane == 31) {
+      wq[warp] = sq;
+      wc[warp] = sc;
     }
-    qoff[nmat] = q;
-    coff[nmat] = c;
+    __syncthreads();
+    if (warp == 0) {
+      wq[lane] = warp_scan(wq[lane]);
+      wc[lane] = warp_scan(wc[lane]);
+    }
+    __syncthreads();
+    if (m < nmat) {
+      qoff[m] = carry_q + (warp ? wq[warp - 1] : 0u) + sq - q;
+      coff[m] = carry_c + (warp ? wc[warp - 1] : 0u) + sc - c;
+      if (blockIdx.x == 0) cursors[m] = qoff[m];
+    }
+    carry_q += wq[31];
+    carry_c += wc[31];
+    __syncthreads();  // wq, wc are rewritten by the next iteration
+  }
+  if (threadIdx.x == 0) {
+    qoff[nmat] = carry_q;
+    coff[nmat] = carry_c;
+    if (blockIdx.x == 0) *n_used = (int32_t)carry_c;
   }
   __syncthreads();
-  for (int m = threadIdx.x; m < nmat; m += blockDim.x) cursors[m] = qoff[m];
   const uint32_t used = coff[nmat];
-  if (threadIdx.x == 0) *n_used = (int32_t)used;
-  for (int32_t c = threadIdx.x; c < max_chunks; c += blockDim.x) {
-    Chunk ch;
-    if ((uint32_t)c < used) {
-      int lo = 0, hi = nmat - 1;  // the material whose chunk range holds c
-      while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (coff[mid] <= (uint32_t)c) lo = mid;
-        else hi = mid - 1;
-      }
-      const uint32_t k = (uint32_t)c - coff[lo];
-      ch.start = (int64_t)qoff[lo] + 128ll * k;
-      const uint32_t left = qoff[lo + 1] - (qoff[lo] + 128u * k);
-      ch.count = (int32_t)(left < 128u ? left : 128u);
-      ch.material = lo;
-    } else {
-      ch.start = 0;
-      ch.count = 0;
-      ch.material = 0;
+  for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < used; c += gridDim.x * blockDim.x) {
+    int lo = 0, hi = nmat - 1;  // the material whose chunk range holds c
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (coff[mid] <= c) lo = mid;
+      else hi = mid - 1;
     }
+    const uint32_t k = c - coff[lo];
+    const uint32_t left = qoff[lo + 1] - (qoff[lo] + 128u * k);
+    Chunk ch;
+    ch.start = (int64_t)qoff[lo] + 128ll * k;
+    ch.count = (int32_t)(left < 128u ? left : 128u);
+    ch.material = lo;
     chunks[c] = ch;
   }
 }
@@ -146,7 +199,7 @@ __global__ void __launch_bounds__(kThreads) bin_scatter_kernel(const int32_t* __
                                                                uint32_t* __restrict__ cursors,
                                                                int32_t* __restrict__ orig) {
   extern __shared__ uint32_t sh[];
-  uint32_t* cnt = sh;               // [nmat] this segment's queries per material, then a bump counter
+  uint32_t* cnt = sh;               // [nmat] this segment's queries per material
   uint32_t* run = sh + nmat;        // [nmat] first slot of the segment's run
   uint32_t* excl = sh + 2 * nmat;   // [nmat] first local position of each material
   uint32_t* stage = sh + 3 * nmat;  // [kSeg] query index of each local position
@@ -155,14 +208,15 @@ __global__ void __launch_bounds__(kThreads) bin_scatter_kernel(const int32_t* __
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t seg = (int64_t)blockIdx.x * kSeg;
   const int64_t end = seg + kSeg < n ? seg + kSeg : n;
+  int id[kPer];
+  load_ids(ids, seg, end, nmat, tile_k, id, nullptr);
   for (int m = threadIdx.x; m < nmat; m += blockDim.x) cnt[m] = 0;
   __syncthreads();
-  for (int64_t base = seg; base < end; base += blockDim.x) {
-    const int64_t i = base + threadIdx.x;
-    int m = i < end && binned_query(tile_k, i) ? __ldg(ids + i) : -1;
-    if (m >= nmat) m = -1;
-    const uint32_t act = __ballot_sync(0xffffffffu, m >= 0);
-    if (m >= 0) warp_bump(cnt, m, act);
+  uint32_t rank[kPer];  // this query's place in its material's run
+#pragma unroll
+  for (int j = 0; j < kPer; ++j) {
+    const uint32_t act = __ballot_sync(0xffffffffu, id[j] >= 0);
+    rank[j] = id[j] >= 0 ? warp_bump(cnt, id[j], act) : 0u;
   }
   __syncthreads();
   // exclusive scan of cnt over the materials: each thread sums a contiguous
@@ -170,15 +224,26 @@ __global__ void __launch_bounds__(kThreads) bin_scatter_kernel(const int32_t* __
   const int per = (nmat + kThreads - 1) / kThreads;
   const int m0 = threadIdx.x * per, m1 = m0 + per < nmat ? m0 + per : nmat;
   uint32_t mine = 0;
-  for (int m = m0; m < m1; ++m) mine += cnt[m];
-  uint32_t x = mine;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
+  bool present = false;
+  for (int m = m0; m < m1; ++m) {
+    mine += cnt[m];
+    present |= cnt[m] != 0;
   }
+  // runs reserved meanwhile
+  for (int m = threadIdx.x; m < nmat; m += blockDim.x) run[m] = cnt[m] ? atomicAdd(cursors + m, cnt[m]) : 0u;
+  const uint32_t x = warp_scan(mine);
   if (lane == 31) wsum[warp] = x;
-  __syncthreads();
+  // a segment of a few materials is written directly below: each warp's
+  // lanes of one material already take consecutive slots; staging pays off
+  // only for many (threads whose materials are present, a lower bound on the
+  // segment's materials when a thread covers several)
+  const bool one = __syncthreads_count(present) <= kDirectMaterials;
+  if (one) {
+#pragma unroll
+    for (int j = 0; j < kPer; ++j)
+      if (id[j] >= 0) orig[run[id[j]] + rank[j]] = (int32_t)(seg + j * kThreads + threadIdx.x);
+    return;
+  }
   uint32_t before = x - mine;
   for (int w = 0; w < warp; ++w) before += wsum[w];
   for (int m = m0; m < m1; ++m) {
@@ -187,48 +252,20 @@ __global__ void __launch_bounds__(kThreads) bin_scatter_kernel(const int32_t* __
   }
   uint32_t total = 0;
   for (int w = 0; w < kThreads / 32; ++w) total += wsum[w];
-  // a segment of a few materials is written directly below: each warp's
-  // lanes of one material already take consecutive slots; staging pays off
-  // only for many (threads whose materials are present, a lower bound on the
-  // segment's materials when a thread covers several)
-  bool present = false;
-  for (int m = m0; m < m1; ++m) present |= cnt[m] != 0;
-  const bool one = __syncthreads_count(present) <= kDirectMaterials;
-  for (int m = threadIdx.x; m < nmat; m += blockDim.x) {
-    run[m] = cnt[m] ? atomicAdd(cursors + m, cnt[m]) : 0u;
-    cnt[m] = 0;
-  }
   __syncthreads();
-  if (one) {
-    for (int64_t base = seg; base < end; base += blockDim.x) {
-      const int64_t i = base + threadIdx.x;
-      int m = i < end && binned_query(tile_k, i) ? __ldg(ids + i) : -1;
-      if (m >= nmat) m = -1;
-      const uint32_t act = __ballot_sync(0xffffffffu, m >= 0);
-      if (m < 0) continue;
-      const uint32_t slot = run[m] + warp_bump(cnt, m, act);
-      orig[slot] = (int32_t)i;
-    }
-    return;
-  }
-  // stage: local position = the material's first position + its bump
-  for (int64_t base = seg; base < end; base += blockDim.x) {
-    const int64_t i = base + threadIdx.x;
-    int m = i < end && binned_query(tile_k, i) ? __ldg(ids + i) : -1;
-    if (m >= nmat) m = -1;
-    const uint32_t act = __ballot_sync(0xffffffffu, m >= 0);
-    if (m < 0) continue;
-    const uint32_t lp = excl[m] + warp_bump(cnt, m, act);
-    stage[lp] = (uint32_t)i;
-    smat[lp] = m;
+  // stage: local position = the material's first position + the rank
+#pragma unroll
+  for (int j = 0; j < kPer; ++j) {
+    if (id[j] < 0) continue;
+    const uint32_t lp = excl[id[j]] + rank[j];
+    stage[lp] = (uint32_t)(seg + j * kThreads + threadIdx.x);
+    smat[lp] = id[j];
   }
   __syncthreads();
   // write: consecutive positions of one material go to consecutive slots
   for (uint32_t p = threadIdx.x; p < total; p += blockDim.x) {
     const int m = smat[p];
-    const int64_t i = stage[p];
-    const uint32_t slot = run[m] + (p - excl[m]);
-    orig[slot] = (int32_t)i;
+    orig[run[m] + (p - excl[m])] = (int32_t)stage[p];
   }
 }
 
@@ -255,65 +292,71 @@ __global__ void __launch_bounds__(kThreads) bin_scatter_kernel(const int32_t* __
 // of the counts (one block, which also writes the table's length for the
 // tensor-core kernel), and the table itself; tile_k = -1 marks the tiles
 // left to binning.
-constexpr int kTilesPerBlock = kThreads / 32;  // one tile per warp in the list pass
-constexpr int kWriteThreads = 256;             // one tile per thread in the write pass
+constexpr int kTilesPerWarp = 4;  // in the list pass; their ids are loaded together
+constexpr int kTilesPerBlock = kThreads / 32 * kTilesPerWarp;
+constexpr int kWriteThreads = 256;  // one tile per thread in the write pass
 
-// One warp per tile: the tile's distinct materials in increasing order (at
-// most kSelectPasses; tile_k = -1 beyond), and one count per pass added to
-// its material's total.
+// kTilesPerWarp tiles per warp: a tile's distinct materials in increasing
+// order (at most kSelectPasses; tile_k = -1 beyond), and one count per pass
+// added to its material's total (summed over the block first: same-address
+// adds serialise in L2).
 __global__ void __launch_bounds__(kThreads) select_tiles_kernel(const int32_t* __restrict__ ids, int64_t n,
                                                                 int nmat, int32_t* __restrict__ tile_k,
                                                                 int32_t* __restrict__ tile_mats,
                                                                 int32_t* __restrict__ mat_passes, int* err) {
+  extern __shared__ uint32_t cnt[];  // [nmat]
+  for (int m = threadIdx.x; m < nmat; m += blockDim.x) cnt[m] = 0;
+  __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t ntiles = (n + 127) / 128;
-  const int64_t t = (int64_t)blockIdx.x * kTilesPerBlock + warp;
-  if (t >= ntiles) return;  // uniform over the warp
-  const int64_t base = t * 128;
-  const int cnt = (int)(n - base < 128 ? n - base : 128);
-  int v[4];  // this lane's ids; INT_MAX once taken (or absent, or invalid)
+  const int64_t t0 = (int64_t)blockIdx.x * kTilesPerBlock + warp * kTilesPerWarp;
+  int v[kTilesPerWarp][4];  // this lane's ids; INT_MAX once taken (or absent, or invalid)
+  bool bad = false;
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int r = lane + 32 * q;
-    v[q] = INT_MAX;
-    if (r < cnt) {
-      const int m = __ldg(ids + base + r);
-      if (m < 0 || m >= nmat) record_error(err, DEVERR_BOUNDS);
-      else v[q] = m;
+  for (int u = 0; u < kTilesPerWarp; ++u)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int64_t i = (t0 + u) * 128 + lane + 32 * q;
+      v[u][q] = i < n ? __ldg(ids + i) : INT_MAX;
+    }
+#pragma unroll
+  for (int u = 0; u < kTilesPerWarp; ++u) {
+    const int64_t t = t0 + u;
+    if (t >= ntiles) break;  // uniform over the warp
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int64_t i = t * 128 + lane + 32 * q;
+      if (v[u][q] < 0 || v[u][q] >= nmat) {
+        bad |= i < n;
+        v[u][q] = INT_MAX;
+      }
+    }
+    int k = 0;
+    bool over = false;
+    for (;;) {
+      const int lm = min(min(v[u][0], v[u][1]), min(v[u][2], v[u][3]));
+      const int m = __reduce_min_sync(0xffffffffu, lm);
+      if (m == INT_MAX) break;
+      if (k == kSelectPasses) {
+        over = true;
+        break;
+      }
+      if (lane == 0) tile_mats[t * kSelectPasses + k] = m;
+      ++k;
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (v[u][q] == m) v[u][q] = INT_MAX;
+    }
+    if (lane == 0) {
+      tile_k[t] = over ? -1 : k;
+      if (!over)
+        for (int j = 0; j < k; ++j) atomicAdd(cnt + tile_mats[t * kSelectPasses + j], 1u);
     }
   }
-  int k = 0, mine = 0;  // mine: the material of this lane's pass (lane < k)
-  bool over = false;
-  for (;;) {
-    const int lm = min(min(v[0], v[1]), min(v[2], v[3]));
-    const int m = __reduce_min_sync(0xffffffffu, lm);
-    if (m == INT_MAX) break;
-    if (k == kSelectPasses) {
-      over = true;
-      break;
-    }
-    if (lane == k) mine = m;
-    if (lane == 0) tile_mats[t * kSelectPasses + k] = m;
-    ++k;
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-      if (v[q] == m) v[q] = INT_MAX;
-  }
-  if (lane == 0) tile_k[t] = over ? -1 : k;
-  // lane j counts the tile's pass j (same-address adds of one material
-  // from many tiles serialise in L2, a few thousand per frame)
-  if (!over && lane < k) atomicAdd(mat_passes + mine, 1);
-}
-
-// inclusive scan over a warp
-__device__ __forceinline__ int32_t warp_scan(int32_t x) {
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int32_t y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
-  }
-  return x;
+  if (bad) record_error(err, DEVERR_BOUNDS);
+  __syncthreads();
+  for (int m = threadIdx.x; m < nmat; m += blockDim.x)
+    if (cnt[m]) atomicAdd(mat_passes + m, (int32_t)cnt[m]);
 }
 
 // One block of 1024: the material counts become cursors (exclusive scan, in
@@ -345,21 +388,37 @@ __global__ void __launch_bounds__(1024) select_scan_kernel(int32_t* __restrict__
 // to binning has no pass.
 __global__ void __launch_bounds__(kWriteThreads) select_write_kernel(const int32_t* __restrict__ tile_k,
                                                                      const int32_t* __restrict__ tile_mats,
-                                                                     int64_t n, int32_t* __restrict__ cursors,
+                                                                     int64_t n, int nmat,
+                                                                     int32_t* __restrict__ cursors,
                                                                      Chunk* __restrict__ passes) {
+  extern __shared__ uint32_t cnt[];  // [nmat] passes of this block's tiles, then their first slot
+  for (int m = threadIdx.x; m < nmat; m += blockDim.x) cnt[m] = 0;
   const int64_t ntiles = (n + 127) / 128;
   const int64_t t = (int64_t)blockIdx.x * kWriteThreads + threadIdx.x;
-  if (t >= ntiles) return;
-  const int32_t k = __ldg(tile_k + t);
-  if (k <= 0) return;
+  const int32_t k = t < ntiles ? __ldg(tile_k + t) : 0;
+  int32_t mat[kSelectPasses];
+  uint32_t rank[kSelectPasses];
+#pragma unroll
+  for (int j = 0; j < kSelectPasses; ++j) mat[j] = j < k ? __ldg(tile_mats + t * kSelectPasses + j) : -1;
+  __syncthreads();
+#pragma unroll
+  for (int j = 0; j < kSelectPasses; ++j) {
+    const uint32_t act = __ballot_sync(0xffffffffu, mat[j] >= 0);
+    rank[j] = mat[j] >= 0 ? warp_bump(cnt, mat[j], act) : 0u;
+  }
+  __syncthreads();
+  for (int m = threadIdx.x; m < nmat; m += blockDim.x)
+    if (cnt[m]) cnt[m] = (uint32_t)atomicAdd(cursors + m, (int32_t)cnt[m]);
+  __syncthreads();
   const int64_t base = t * 128;
-  const int cnt = (int)(n - base < 128 ? n - base : 128);
-  for (int j = 0; j < k; ++j) {
+#pragma unroll
+  for (int j = 0; j < kSelectPasses; ++j) {
+    if (mat[j] < 0) continue;
     Chunk ch;
     ch.start = base;
-    ch.count = cnt;
-    ch.material = __ldg(tile_mats + t * kSelectPasses + j);
-    passes[atomicAdd(cursors + ch.material, 1)] = ch;
+    ch.count = (int)(n - base < 128 ? n - base : 128);
+    ch.material = mat[j];
+    passes[cnt[mat[j]] + rank[j]] = ch;
   }
 }
 
@@ -393,7 +452,8 @@ static int bin_eval(const BinArgs& a, const int32_t* tile_k, cudaStream_t s) {
   if (e) return e;
   const int gseg = (int)((n + kSeg - 1) / kSeg);
   bin_count_kernel<<<gseg, kThreads, a.nmat * sizeof(uint32_t), s>>>(a.ids, n, a.nmat, tile_k, counts, a.L.err);
-  bin_plan_kernel<<<1, 1024, 2 * (a.nmat + 1) * sizeof(uint32_t), s>>>(counts, a.nmat, cursors, chunks, maxc, n_used);
+  const int gplan = (maxc + 1023) / 1024 < 16 ? (maxc + 1023) / 1024 : 16;
+  bin_plan_kernel<<<gplan, 1024, 2 * (a.nmat + 1) * sizeof(uint32_t), s>>>(counts, a.nmat, cursors, chunks, n_used);
   const int scatter_smem = (3 * a.nmat + (kStage + 1) * kSeg) * (int)sizeof(uint32_t);
   static std::atomic<uint64_t> scatter_attr{0};
   once_per_device(scatter_attr, [] {
@@ -459,10 +519,11 @@ int launch_select_eval(const SelectArgs& a, void* stream) {
   Chunk* passes = (Chunk*)(p + l.passes);
   int e = (int)cudaMemsetAsync(counts, 0, (size_t)nmat * 4, s);
   if (e) return e;
-  select_tiles_kernel<<<(int)l.nb, kThreads, 0, s>>>(a.ids, n, nmat, tile_k, tile_mats, counts, a.L.err);
+  const int mat_smem = nmat * (int)sizeof(uint32_t);
+  select_tiles_kernel<<<(int)l.nb, kThreads, mat_smem, s>>>(a.ids, n, nmat, tile_k, tile_mats, counts, a.L.err);
   select_scan_kernel<<<1, 1024, 0, s>>>(counts, nmat, total);
-  select_write_kernel<<<(int)((l.ntiles + kWriteThreads - 1) / kWriteThreads), kWriteThreads, 0, s>>>(
-      tile_k, tile_mats, n, counts, passes);
+  select_write_kernel<<<(int)((l.ntiles + kWriteThreads - 1) / kWriteThreads), kWriteThreads, mat_smem, s>>>(
+      tile_k, tile_mats, n, nmat, counts, passes);
   e = (int)cudaGetLastError();
   if (e) return e;
   LaunchCommon L = a.L;

@@ -94,3 +94,37 @@ def test_sampler_many_tiles_per_cta(gctx, latent):
     assert torch.equal(pdf, torch.cat([p[1] for p in parts]))
     mat.destroy()
     gctx.check()
+
+
+@pytest.mark.parametrize("nmat,n", [(3, 2048), (700, 2049), (4096, 300007)])
+@pytest.mark.parametrize("coherent", [False, True])
+def test_binning_segments_and_bad_ids(gctx, nmat, n, coherent):
+    """Material counts up to the limit, partly filled segments, runs of one
+    material, and ids outside the range at both ends of int32."""
+    import torch
+    from paper_2305_02678_gb300 import binding as B
+    from paper_2305_02678_gb300 import NamError
+    rng = W.rng_streams(144, 6)
+    two = [gctx.material(32, 32, 6, W.make_pyramid(rng[k], 32, 32, 6, dtype=np.float16), None,
+                         W.make_model(rng[2 + k], (14, 16, 16, 3), None)["decoder"]) for k in range(2)]
+    handles = [two[k % 2].h for k in range(nmat)]
+    dq = to_device(W.uniform_queries(rng[4], n, 5.0))
+    ids = rng[5].integers(0, nmat, n).astype(np.int32)
+    if coherent:
+        ids = np.repeat(ids, 200)[:n].copy()
+    bad = rng[5].integers(0, n, 9)
+    ids[bad] = np.resize(np.array([-1, nmat, -2 ** 31, 2 ** 31 - 1], np.int64), 9).astype(np.int32)
+    ref = torch.stack([m.eval(dq) for m in two])
+    ok = (ids >= 0) & (ids < nmat)
+    want = torch.full((n, 3), -7.0, device="cuda")
+    idx = torch.from_numpy(np.nonzero(ok)[0]).cuda()
+    want[idx] = ref[torch.from_numpy(ids[ok] % 2).long().cuda(), idx]
+    for call in (B.nam_eval_binned, B.nam_eval_select):
+        out = torch.full((n, 3), -7.0, device="cuda")
+        call(gctx.h, handles, dq, torch.from_numpy(ids).cuda(), n, out, torch.cuda.current_stream())
+        assert torch.equal(out, want)
+        with pytest.raises(NamError):
+            gctx.check()
+    for m in two:
+        m.destroy()
+    gctx.check()
