@@ -16,11 +16,12 @@ def __getattr__(name):
     # this package before the library exists); a missing library raises
     # ImportError there -- there is no fallback.
     import importlib
-    if name in ("B", "binding"):
-        return importlib.import_module(__name__ + ".binding")
-    if name == "NamError":
-        return importlib.import_module(__name__ + ".binding").NamError
-    raise AttributeError(name)
+    if name not in ("B", "binding", "NamError"):
+        raise AttributeError(name)
+    mod = importlib.import_module(__name__ + ".binding")
+    # found here from now on, without this function
+    globals().update(B=mod, NamError=mod.NamError)
+    return globals()[name]
 
 
 def flatten_frame(frame):
@@ -134,11 +135,12 @@ class Material:
         import torch
 
         from . import binding as B
-        n = int(q["u"].shape[0])
+        u = q["u"]
+        n = int(u.shape[0])
         if out is None:
-            out = torch.empty((n, 3), dtype=torch.float32, device=q["u"].device)
+            out = torch.empty((n, 3), dtype=torch.float32, device=u.device)
         if stream is None:
-            stream = torch.cuda.current_stream(q["u"].device)
+            stream = B.current_stream(u.device)
         B.nam_eval(self.ctx.h, self.h, q, n, out, stream, flags)
         return out
 
@@ -147,11 +149,12 @@ class Material:
         import torch
 
         from . import binding as B
-        n = int(q["u"].shape[0])
-        rgb = torch.empty((n, 3), dtype=torch.float32, device=q["u"].device)
-        alb = torch.empty((n, 3), dtype=torch.float32, device=q["u"].device)
+        u = q["u"]
+        n = int(u.shape[0])
+        rgb = torch.empty((n, 3), dtype=torch.float32, device=u.device)
+        alb = torch.empty((n, 3), dtype=torch.float32, device=u.device)
         if stream is None:
-            stream = torch.cuda.current_stream(q["u"].device)
+            stream = B.current_stream(u.device)
         B.nam_eval_albedo(self.ctx.h, self.h, q, n, rgb, alb, stream, flags)
         return rgb, alb
 
