@@ -1,51 +1,78 @@
 // Reverse mode of the FP32 evaluation, the log-space L1 loss and Adam
 // (training of the decoder and the latent texture, Sec. 5).
 //
-// Backward kernel: a CTA of 512 threads takes tiles of 128 queries.  Two
-// lane mappings share the tile:
-//  - a quad of four adjacent lanes per query, for the per-query work: the
-//    latent fetch, the frame MLP (lane p owns frame hidden units p + 4e, the
-//    six outputs are summed over the quad), the frame construction and its
-//    backward (redundant in the quad, ALU only), dL/dx (lane p owns x
-//    entries 4p..4p+3) and the pyramid scatter (lane p takes bilinear tap p;
+// Backward kernel: two groups of eight compute warps each take tiles of 64
+// queries, one group's waits under the other's work; the MMAs are issued by
+// threads of the compute warps (issuing warps of their own would cost every
+// thread 32 of its 128 registers: 453 us against 411).  The forward is recomputed in FP32 on the FMA
+// pipes, in a fixed order of operations (a ReLU sign that a rounding flips
+// moves a texel's gradient by far more than the rounding); everything behind
+// the signs, which is two thirds of the work, runs on the tensor cores as
+// bf16 MMAs on three-way splits (x = x_h + x_m + x_l, eight significant bits
+// each; six products, FP32 accumulation, small products first), which have
+// FP32's range and lose less than its rounding.
+//  - a quad of four adjacent lanes per query: the latent fetch, the frame MLP
+//    (lane p owns frame hidden units p + 4e, the six outputs are summed over
+//    the quad), the frame construction and its backward (redundant in the
+//    quad, ALU only) and the pyramid scatter (lane p takes bilinear tap p;
 //    taps that coincide, as at the coarsest levels, are merged so that each
 //    distinct texel of a query takes one update);
-//  - a half-warp per four queries for the decoder layers: lane l owns hidden
-//    units l + 16 jj of all four queries, a 4 x (H/16) register block, so
-//    that every shared-memory operand feeds four FMAs per query block.
-//  Activations and deltas go to shared-memory rows; the lanes that read them
-//  are in the writer's warp, so a __syncwarp orders them.
-//  Training step variant (LOSS): the decoder blocks also finish the forward
-//  (y = Wo h2 + bo, summed over the half-warp), evaluate the log-space L1
-//  loss against the target and start the backward from its gradient, so a
-//  training step needs no separate forward or loss pass.  With the albedo
-//  head (ALB: six outputs, RGB then albedo) the fused loss adds the albedo's
-//  L2 error against one-sample albedo estimates (the paper's albedo
-//  inference), and the output layer's gradient blocks span eight rows.
-//  Phase B (thread = 4x4 block of one weight matrix): each owner sums the
-//  outer products delta[q][rows] * act[q][cols] over the tile in registers
-//  (two 16-byte shared loads per 16 FMAs), the column-0 owners also sum the
-//  bias deltas.  The registers are added to the global gradient with one
-//  atomic per parameter per CTA after the CTA's last tile.
-//  Same-address atomics serialise in L2, and every query whose lod reaches
-//  the coarsest levels lands on a handful of texels there: the gradient of
-//  the coarsest levels is summed in shared memory first (per warp for the
-//  tiniest ones, per CTA for the next) and added to the global buffer once
-//  per CTA.
+//  - a half-warp per four queries for the decoder's forward: lane l owns
+//    hidden units l + 16 jj of all four queries, a 4 x (H/16) register block,
+//    so that every shared-memory operand feeds four FMAs per query block; the
+//    output layer's gradient, three columns wide, is summed in these lanes;
+//  - MMAs per tile: d1 = D2 W2 (queries in the rows), dx = D1 W1, and, with
+//    the same operands read the other way (queries along K), C2 = D2^T [H1 |
+//    X 1], C1 = D1^T [X 1] and CF = [DHF | DR]^T [X 1 | HF], which hold every
+//    weight and bias gradient of the other layers; they are read back each
+//    tile and summed in registers (the accumulator cuts off instead of rounding:
+//    a sum over all tiles in it would drift), one atomic per parameter and
+//    CTA at the end.  (An infinite delta may give NaN where a product of FP32
+//    values would give an infinity.)
+// Operand arrays: [term][unit / 8][query][unit % 8] bf16, which is K-major for
+// the products over units and MN-major for those over queries.
+// What bounds it: the latency of the tile's chain of stages (16 warps a CTA,
+// which shared memory and registers allow no more of; the forward on the FMA
+// pipes is a fifth of a tile's time, the fetch and the scatter a sixth each).
+// H = 64 with the fused loss, 262,144 queries, 1024^2 pyramid: 290 us, against
+// 378 us with every product on the FMA pipes; 131,072 queries with the latents
+// given: 133 us (163).  Smaller batches and decoders, against that kernel:
+// H = 64, 10,000 queries 38 us (44); H = 16, 262,144 queries 187 us (207).
+// Training step variant (LOSS): the decoder blocks also finish the forward
+// (y = Wo h2 + bo, summed over the half-warp), evaluate the log-space L1
+// loss against the target and start the backward from its gradient, so a
+// training step needs no separate forward or loss pass.  With the albedo
+// head (ALB: six outputs, RGB then albedo) the fused loss adds the albedo's
+// L2 error against one-sample albedo estimates (the paper's albedo
+// inference).
+// Same-address atomics serialise in L2, and every query whose lod reaches
+// the coarsest levels lands on a handful of texels there: the gradient of
+// the coarsest levels is summed in shared memory first (per warp for the
+// tiniest ones, per CTA for the next) and added to the global buffer once
+// per CTA.
 #include <cuda_runtime.h>
 
 #include "common.cuh"
+#include "tc_ptx.cuh"
 
 namespace nam {
 
-constexpr int kBwdQ = 128;             // queries per tile
-constexpr int kBwdThreads = 4 * kBwdQ;  // a quad per query
+constexpr int kBwdQ = 64;             // queries per tile, one tile per group
+constexpr int kBwdGroup = 4 * kBwdQ;  // threads of a group: a quad per query
+constexpr int kBwdThreads = 2 * kBwdGroup;
+constexpr int kBlk = kBwdQ * 16;      // bytes of an operand block (eight units of the queries)
 
 template <int H, bool ALB = false>
 struct BwdSmem {
   static constexpr int NO = ALB ? 6 : 3;  // decoder outputs
   static constexpr int DW = ALB ? 8 : 4;  // DY row length
-  static constexpr int S = H + 4;  // padded row stride: rows l + 16 jj of a half-warp hit distinct banks
+  static constexpr int S = H + 4;  // padded row stride of W2 and H1: rows l + 16 jj of a half-warp hit distinct banks
+  // operand terms: A holds first D2 (H / 8 blocks), then D1, DHF (2 blocks)
+  // and DR (1); B holds H1, X (2 blocks, with the 1) and HF (2).  An MMA's A
+  // has 128 rows, a group's 64 (or 24) of them in its half of the TMEM
+  // lanes: it reads up to 8 KB before and 16 KB past a term's start, rows
+  // whose results are not used, inside this struct.
+  static constexpr int TA = (H / 8 + 3) * kBlk, TB = (H / 8 + 4) * kBlk;
   // parameters
   float fW1[16 * 8], fb1[16], fW2[6 * 16], fb2[8];
   float W1[H][20];   // W1[j][0..13], zero padding
@@ -53,24 +80,55 @@ struct BwdSmem {
   float W2[H][S];    // W2[j][k]
   float b2[H];
   float Wo[NO * H], bo[8];
-  float lred[16];  // per-warp loss partials
-  // per-query vectors of the current tile (deltas at pre-activations)
-  float Z[kBwdQ][8];     // frame MLP input (z)
-  float HF[kBwdQ][16];   // frame hidden activations
-  float DHF[kBwdQ][16];  // delta at the frame hidden pre-activations
-  float R[kBwdQ][8];     // frame MLP output r = (n_raw, t_raw)
-  float DR[kBwdQ][8];    // delta at r, zero padding
-  float X[kBwdQ][16];    // decoder input x (14), zero padding
-  float DX[kBwdQ][16];   // dL/dx
-  float D1[kBwdQ][S];    // delta at decoder layer-1 pre-activations
-  float H1[kBwdQ][S];    // decoder layer-1 activations
-  float D2[kBwdQ][S];    // delta at layer-2 pre-activations
-  float H2[kBwdQ][S];    // layer-2 activations
-  float DY[kBwdQ][DW];   // delta at the outputs (after the cosine factor), zero padding;
-                         // with the fused loss first the targets and the cosine
-                         // factor: (t_r, t_g, t_b, cf), or with ALB (t_r, t_g, t_b,
-                         // albedo t_r, t_g, t_b, 0, cf)
+  float lred[16];       // per-warp loss partials
+  float gwo[NO * H + 8];  // output layer's gradient of the CTA
+  uint32_t tslot, pad[3];
+  uint64_t bars[8];  // per group: d1, C2, dx, C1
+  // per group, of the current tile (deltas at pre-activations)
+  struct Group {
+    uint32_t mask1[8][16];  // per warp and (jj * 4 + qq): layer-1 signs of its two half-warps
+    float R[kBwdQ][8];      // frame MLP output r = (n_raw, t_raw)
+    float X[kBwdQ][16];     // decoder input x (14), zero padding; then dL/dx
+    float DY[kBwdQ][DW];    // delta at the outputs (after the cosine factor), zero padding;
+                            // with the fused loss first the targets and the cosine
+                            // factor: (t_r, t_g, t_b, cf), or with ALB (t_r, t_g, t_b,
+                            // albedo t_r, t_g, t_b, 0, cf)
+    alignas(128) uint8_t A[3 * TA];  // before D2: layer-1 activations H1[q][S] in FP32
+    uint8_t B[3 * TB];
+  } g[2];
+  uint8_t W2T[3 * H * H * 2];   // MMA B operand of d1: rows k, K = j
+  uint8_t W1T[3 * 16 * H * 2];  // MMA B operand of dx: rows c, K = j
 };
+
+// the three bf16 terms of x (its next eight significant bits each), as bits
+__device__ __forceinline__ void split3_one(float x, uint16_t& h, uint16_t& m, uint16_t& l) {
+  const uint32_t b = __float_as_uint(x);
+  const float r = x - __uint_as_float(b & 0xFFFF0000u);
+  const uint32_t br = __float_as_uint(r);
+  const float q = r - __uint_as_float(br & 0xFFFF0000u);
+  h = (uint16_t)(b >> 16);
+  m = (uint16_t)(br >> 16);
+  l = (uint16_t)(__float_as_uint(q) >> 16);
+}
+// U values (consecutive units) of one query to their rows of the three terms;
+// p: the first unit's place in term 0, TS: bytes of a term
+template <int U, int TS>
+__device__ __forceinline__ void put_terms(uint8_t* p, const float (&v)[U]) {
+  uint32_t w[3][U / 2];
+#pragma unroll
+  for (int j = 0; j < U / 2; ++j) ptx::split3(v[2 * j], v[2 * j + 1], w[0][j], w[1][j], w[2][j]);
+#pragma unroll
+  for (int t = 0; t < 3; ++t) {
+    if constexpr (U == 4) {
+      *reinterpret_cast<uint2*>(p + t * TS) = make_uint2(w[t][0], w[t][1]);
+    } else {
+#pragma unroll
+      for (int b = 0; b < U / 8; ++b)
+        *reinterpret_cast<uint4*>(p + t * TS + b * kBlk) =
+            make_uint4(w[t][4 * b], w[t][4 * b + 1], w[t][4 * b + 2], w[t][4 * b + 3]);
+    }
+  }
+}
 
 // Log-space L1 loss of one output element g against its target y (Sec. 5.2
 // names an L1 loss in log space; read as |log(1 + max(g, 0)) - log(1 + y)|
@@ -101,14 +159,103 @@ __device__ __forceinline__ float dot4(const float4 a, const float4 b, float s) {
   return fmaf(a.w, b.w, s);
 }
 
+// The latent of a quad's query: lane p filters channels 2p and 2p + 1 (a texel
+// is one 32-byte sector of the four lanes' loads).  quad_taps starts the
+// loads, quad_filter sums in fetch_latent's order of operations.  f0: u, v,
+// lod, xi in lanes 0..3.
+struct QuadTaps {
+  float2 x[8];
+  float w[8];
+};
+__device__ __forceinline__ void quad_taps(const BackwardArgs& A, float f0, int p, QuadTaps& T) {
+  const float u = __shfl_sync(0xffffffffu, f0, 0, 4), v = __shfl_sync(0xffffffffu, f0, 1, 4);
+  const float lod = __shfl_sync(0xffffffffu, f0, 2, 4), xi = __shfl_sync(0xffffffffu, f0, 3, 4);
+  const LevelPick lp = pick_levels(A.pyr, lod);
+  const bool stoch = A.pyr.filter == NAM_FILTER_STOCHASTIC;
+  auto level = [&](int l, float wgt, bool load, float2* x, float* w) {
+    const int W = A.pyr.w[l];
+    int x0, x1, y0, y1;
+    float fx, fy;
+    tap_axis(A.pyr, u, W, x0, x1, fx);
+    tap_axis(A.pyr, v, A.pyr.h[l], y0, y1, fy);
+    const uint32_t base = (uint32_t)A.pyr.off[l];
+    const uint32_t r0 = base + (uint32_t)y0 * (uint32_t)W, r1 = base + (uint32_t)y1 * (uint32_t)W;
+    const uint32_t idx[4] = {r0 + x0, r0 + x1, r1 + x0, r1 + x1};
+    const float gx = 1.0f - fx, gy = 1.0f - fy;
+    w[0] = gx * gy * wgt;
+    w[1] = fx * gy * wgt;
+    w[2] = gx * fy * wgt;
+    w[3] = fx * fy * wgt;
+    const float2* t = reinterpret_cast<const float2*>(A.pyramid) + p;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) x[k] = load ? __ldg(t + 4 * (size_t)idx[k]) : make_float2(0.0f, 0.0f);
+  };
+  level(stoch && xi < lp.t ? lp.l1 : lp.l0, stoch ? 1.0f : 1.0f - lp.t, true, T.x, T.w);
+  // (a level of weight 0 is not read and adds zeros)
+  level(lp.l1, stoch ? 0.0f : lp.t, !stoch && lp.t != 0.0f, T.x + 4, T.w + 4);
+}
+__device__ __forceinline__ void quad_gather(float2 a, float z[8]) {
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    z[2 * k] = __shfl_sync(0xffffffffu, a.x, k, 4);
+    z[2 * k + 1] = __shfl_sync(0xffffffffu, a.y, k, 4);
+  }
+}
+__device__ __forceinline__ void quad_filter(const QuadTaps& T, float z[8]) {
+  float2 acc = make_float2(0.0f, 0.0f);
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    acc.x = fmaf(T.w[k], T.x[k].x, acc.x);
+    acc.y = fmaf(T.w[k], T.x[k].y, acc.y);
+  }
+  quad_gather(acc, z);
+}
+
+// One query's fields, spread over its quad: lane p holds (u, v, lod, xi)[p],
+// wi[p], wo[p], and target or output gradient [p] and [3 + p] (p < 3).
+struct QuadFields {
+  float f0, f1, f2, g0, g1;
+};
+template <bool LOSS, bool ALB>
+__device__ __forceinline__ QuadFields quad_fields(const BackwardArgs& A, int64_t i, bool valid, int p) {
+  QuadFields f{};
+  const float* a = p == 0 ? A.q.u : p == 1 ? A.q.v : p == 2 ? A.q.lod : A.q.xi;
+  if (!A.z_in && a) f.f0 = __ldg(a + i);
+  if (p < 3) {
+    f.f1 = __ldg((p == 0 ? A.q.wix : p == 1 ? A.q.wiy : A.q.wiz) + i);
+    f.f2 = __ldg((p == 0 ? A.q.wox : p == 1 ? A.q.woy : A.q.woz) + i);
+    if (valid) {
+      if (LOSS) {
+        f.g0 = __ldg(A.target + 3 * i + p);
+        if (ALB) f.g1 = __ldg(A.target_albedo + 3 * i + p);
+      } else {
+        f.g0 = __ldg(A.grad_rgb + (ALB ? 6 : 3) * i + p);
+        if (ALB) f.g1 = __ldg(A.grad_rgb + 6 * i + 3 + p);
+      }
+    }
+  }
+  return f;
+}
+
 template <int H, bool FRAME, bool F16, bool LOSS, bool ALB>
 __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const BackwardArgs A) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
+  extern __shared__ __align__(128) unsigned char smem_raw[];
   using Sm = BwdSmem<H, ALB>;
   Sm& S = *reinterpret_cast<Sm*>(smem_raw);
-  constexpr int NO = Sm::NO, DW = Sm::DW;
+  constexpr int NO = Sm::NO, DW = Sm::DW, TA = Sm::TA, TB = Sm::TB;
   constexpr int JB = H / 16;  // hidden units per lane in the decoder blocks
+  constexpr int U = H / 4;    // units per lane where a row is shared by four
+  constexpr int N2 = H + 16;  // columns of C2
+  // TMEM columns of a group
+  constexpr int cD1 = 0, cDX = 64, cC2 = 80, cC1 = 160, cCF = 176, cGroup = 208;
   const int t = threadIdx.x;
+  const int lane = t & 31, warp = __shfl_sync(0xffffffffu, t >> 5, 0);
+  // groups: compute warps 4k and 4k + 1 (TMEM lanes 0..63), 4k + 2 and 4k + 3
+  // (lanes 64..127)
+  const int grp = (warp >> 1) & 1;
+  typename Sm::Group& G = S.g[grp];
+  const uint32_t bar0 = ptx::smem_u32(S.bars) + 32 * grp;
+  const int bid = 4 * grp;  // named barriers bid + 1 .. bid + 4
   // ---- parameters -> shared ---------------------------------------------------
   {
     const float* p = A.params;
@@ -134,79 +281,169 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const Backward
     p += NO * H;
     if (t < 8) S.bo[t] = t < NO ? p[t] : 0.0f;
   }
+  // MMA B operands of the delta products
+  {
+    const float* W1 = A.params + (FRAME ? 246 : 0);
+    const float* W2 = W1 + 14 * H + H;
+    for (int i = t; i < H * H; i += kBwdThreads) {
+      const int j = i / H, k = i % H;  // W2[j][k] -> row k, K index j
+      uint16_t w[3];
+      split3_one(W2[i], w[0], w[1], w[2]);
+#pragma unroll
+      for (int e = 0; e < 3; ++e)
+        *reinterpret_cast<uint16_t*>(S.W2T + e * H * H * 2 + (j / 8) * (H * 16) + k * 16 + (j % 8) * 2) = w[e];
+    }
+    for (int i = t; i < H * 16; i += kBwdThreads) {
+      const int j = i / 16, c = i % 16;
+      uint16_t w[3];
+      split3_one(c < 14 ? W1[j * 14 + c] : 0.0f, w[0], w[1], w[2]);
+#pragma unroll
+      for (int e = 0; e < 3; ++e)
+        *reinterpret_cast<uint16_t*>(S.W1T + e * 16 * H * 2 + (j / 8) * 256 + c * 16 + (j % 8) * 2) = w[e];
+    }
+    for (int i = t; i < NO * H + 8; i += kBwdThreads) S.gwo[i] = 0.0f;
+  }
+  if (t == 0) {
+    // C1 and CF are issued by two warps
+    for (int k = 0; k < 8; ++k) ptx::mbar_init(ptx::smem_u32(&S.bars[k]), (k & 3) == 3 ? 2 : 1);
+    ptx::fence_mbar_init();
+  }
+  if (warp == 0) {
+    ptx::tmem_alloc(ptx::smem_u32(&S.tslot), 512);
+    ptx::tmem_relinquish();
+  }
   // coarse-level accumulators after the tile: [16 warps][tiny_n][8], [cta_n][8]
   float* wacc = reinterpret_cast<float*>(smem_raw + sizeof(Sm));
   float* cacc = wacc + 16 * 8 * A.tiny_n;
   for (int i = t; i < 8 * (16 * A.tiny_n + A.cta_n); i += kBwdThreads) wacc[i] = 0.0f;
   float* my_wacc = wacc + (t >> 5) * 8 * A.tiny_n;
 
-  // ---- phase-B ownership: one 4x4 block of one gradient matrix ------------------
-  // blocks: dW2 (H/4)^2, dW1 H/4 x 4 (14 columns padded to 16), dWo
-  // DW/4 x H/4 (3 rows padded to 4, or 6 padded to 8), dWf1 4 x 2, dWf2 2 x 4
-  // (6 rows padded to 8)
-  constexpr int NB2 = (H / 4) * (H / 4), NB1 = H, NBO = (DW / 4) * (H / 4);
-  int role = -1, r0 = 0, c0 = 0;
-  const float* dp = nullptr;
-  const float* ap = nullptr;
-  int dstride = 0, astride = 0;
-  {
-    int b = t;
-    if (b < NB2) {
-      role = 0; r0 = 4 * (b / (H / 4)); c0 = 4 * (b % (H / 4));
-      dp = &S.D2[0][r0]; dstride = Sm::S; ap = &S.H1[0][c0]; astride = Sm::S;
-    } else if ((b -= NB2) < NB1) {
-      role = 1; r0 = 4 * (b >> 2); c0 = 4 * (b & 3);
-      dp = &S.D1[0][r0]; dstride = Sm::S; ap = &S.X[0][c0]; astride = 16;
-    } else if ((b -= NB1) < NBO) {
-      role = 2; r0 = 4 * (b / (H / 4)); c0 = 4 * (b % (H / 4));
-      dp = &S.DY[0][r0]; dstride = DW; ap = &S.H2[0][c0]; astride = Sm::S;
-    } else if (FRAME && (b -= NBO) < 8) {
-      role = 3; r0 = 4 * (b >> 1); c0 = 4 * (b & 1);
-      dp = &S.DHF[0][r0]; dstride = 16; ap = &S.Z[0][c0]; astride = 8;
-    } else if (FRAME && (b -= 8) < 8) {
-      role = 4; r0 = 4 * (b >> 2); c0 = 4 * (b & 3);
-      dp = &S.DR[0][r0]; dstride = 8; ap = &S.HF[0][c0]; astride = 16;
-    }
-  }
-  float acc[16], accb[4];
-#pragma unroll
-  for (int i = 0; i < 16; ++i) acc[i] = 0.0f;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) accb[i] = 0.0f;
+  ptx::fence_proxy_async();
+  ptx::tc_fence_before();
   __syncthreads();
+  ptx::tc_fence_after();
+  const uint32_t tmem = S.tslot + cGroup * grp;
+  const int64_t ntiles = (A.n + kBwdQ - 1) / kBwdQ;
+  bool bad = false;
+
+  // A stage's products, one thread: six of term pairs, the small ones first.
+  // a, b: the descriptors of the first term's first step
+  auto products = [&](uint32_t d, uint64_t a, uint32_t ta, uint32_t astep, uint64_t b, uint32_t tb, uint32_t bstep,
+                      int steps, uint32_t id) {
+    const int at[6] = {2, 1, 0, 1, 0, 0}, bt[6] = {0, 1, 2, 0, 1, 0};
+#pragma unroll
+    for (int e = 0; e < 6; ++e)
+#pragma unroll
+      for (int s = 0; s < steps; ++s)
+        ptx::mma_f16(d, ptx::sdesc_at(a, at[e] * ta + s * astep, 0), ptx::sdesc_at(b, bt[e] * tb + s * bstep, 0), id,
+                     e + s > 0 ? 1u : 0u);
+  };
+  // operands: the second group's rows are 64..127 of an MMA
+  const uint32_t aA = ptx::smem_u32(G.A), aB = ptx::smem_u32(G.B);
+  const uint32_t aK = aA - grp * 64 * 16, aM = aA - grp * 8 * kBlk;
+  constexpr uint32_t kMN = (1u << 15) | (1u << 16);  // both operands MN-major
+  const int64_t tile0 = blockIdx.x + (int64_t)grp * gridDim.x, tstep = 2 * (int64_t)gridDim.x;
+  // lw: this warp in its group.  Gradients of this thread's part of C2, C1 and
+  // CF: row grow of the group's half of the TMEM lanes, a quarter of the columns
+  const int lw = ((warp >> 2) << 1) | (warp & 1), lt = 32 * lw + lane;
+  const int grow = 32 * (lw & 1) + lane, gq = lw >> 1;
+  const uint32_t tl = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
+  const bool use2 = 32 * (lw & 1) < H, usef = FRAME && (lw & 1) == 0;
+  float acc2[N2 / 4], acc1[4], accf[8], gwo[NO][JB], gbo[NO];
+#pragma unroll
+  for (int i = 0; i < N2 / 4; ++i) acc2[i] = 0.0f;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) acc1[i] = 0.0f;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) accf[i] = 0.0f;
+#pragma unroll
+  for (int c = 0; c < NO; ++c) {
+    gbo[c] = 0.0f;
+#pragma unroll
+    for (int jj = 0; jj < JB; ++jj) gwo[c][jj] = 0.0f;
+  }
+  // the weight gradients of the tile before: add C2, C1 and CF to the registers
+  auto collect = [&]() {
+    ptx::tc_fence_after();
+    if (use2) {
+#pragma unroll
+      for (int c0 = 0; c0 < N2 / 4; c0 += 4) {
+        uint32_t v[4];
+        ptx::tmem_ld4(tl + cC2 + gq * (N2 / 4) + c0, v);
+        ptx::tmem_ld_wait();
+#pragma unroll
+        for (int e = 0; e < 4; ++e) acc2[c0 + e] += __uint_as_float(v[e]);
+      }
+      uint32_t v[4];
+      ptx::tmem_ld4(tl + cC1 + 4 * gq, v);
+      ptx::tmem_ld_wait();
+#pragma unroll
+      for (int e = 0; e < 4; ++e) acc1[e] += __uint_as_float(v[e]);
+    }
+    if (usef) {
+      uint32_t v[8];
+      ptx::tmem_ld8(tl + cCF + 8 * gq, v);
+      ptx::tmem_ld_wait();
+#pragma unroll
+      for (int e = 0; e < 8; ++e) accf[e] += __uint_as_float(v[e]);
+    }
+  };
+  uint32_t ph = 0;  // parity of this tile's MMAs
 
   float lsum = 0.0f;  // fused loss: this lane's share of the sum
-  const int ql = t >> 2, p = t & 3;         // quad: query ql, lane p
-  const int hl = t & 15, qb = (t >> 4) * 4;  // half-warp: queries qb..qb+3, units hl + 16 jj
+  const int ql = lt >> 2, p = lt & 3;         // quad: query ql, lane p
+  const int hl = lt & 15, qb = (lt >> 4) * 4;  // half-warp: queries qb..qb+3, units hl + 16 jj
   const bool cosine = (A.flags & NAM_OUT_COSINE) != 0;
-  const int64_t ntiles = (A.n + kBwdQ - 1) / kBwdQ;
-  for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+  uint32_t issued = 0;  // tiles whose MMAs were issued (the same in the whole group)
+  bool stop = false;    // a wait ran out
+  // the fields of the next tile are loaded a tile ahead (its texels as well
+  // would cost more in spilled registers than their latency)
+  auto row_of = [&](int64_t tile, bool& valid) -> int64_t {
+    const int64_t start = tile * kBwdQ;
+    valid = ql < A.n - start;
+    return start + (valid ? ql : 0);
+  };
+  QuadFields nxt{};
+  if (tile0 < ntiles) {
+    bool v;
+    const int64_t i = row_of(tile0, v);
+    nxt = quad_fields<LOSS, ALB>(A, i, v, p);
+  }
+  for (int64_t tile = tile0; tile < ntiles; tile += tstep, ph ^= 1u) {
     const int64_t start = tile * kBwdQ;
     const int count = (int)((A.n - start) < kBwdQ ? (A.n - start) : kBwdQ);
-    const bool valid = ql < count;
-    const int64_t i = start + (valid ? ql : 0);
-    // =================== phase A ===========================================
+    bool valid;
+    const int64_t i = row_of(tile, valid);
+    const QuadFields cur = nxt;
+    if (tile + tstep < ntiles) {
+      bool v;
+      const int64_t j = row_of(tile + tstep, v);
+      nxt = quad_fields<LOSS, ALB>(A, j, v, p);
+    }
     // ---- quad: latent, frame MLP, frame, decoder input ----------------------
+    float hf[4] = {0.0f, 0.0f, 0.0f, 0.0f};  // frame hidden units p + 4e
     {
       float z[8];
       if (A.z_in) {
         // encoder phase (Sec. 5.1): the latent is given, the texture bypassed
-        const float4 a = reinterpret_cast<const float4*>(A.z_in + 8 * i)[0];
-        const float4 b = reinterpret_cast<const float4*>(A.z_in + 8 * i)[1];
-        z[0] = a.x; z[1] = a.y; z[2] = a.z; z[3] = a.w; z[4] = b.x; z[5] = b.y; z[6] = b.z; z[7] = b.w;
+        quad_gather(reinterpret_cast<const float2*>(A.z_in + 8 * i)[p], z);
       } else {
-        const float xi = A.q.xi ? A.q.xi[i] : 0.0f;
-        fetch_latent<F16>(A.pyr, A.pyramid, A.q.u[i], A.q.v[i], A.q.lod[i], xi, z);
+        QuadTaps T;
+        quad_taps(A, cur.f0, p, T);
+        quad_filter(T, z);
       }
-      const float wi[3] = {A.q.wix[i], A.q.wiy[i], A.q.wiz[i]};
-      const float wo[3] = {A.q.wox[i], A.q.woy[i], A.q.woz[i]};
+      float wi[3], wo[3];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        wi[c] = __shfl_sync(0xffffffffu, cur.f1, c, 4);
+        wo[c] = __shfl_sync(0xffffffffu, cur.f2, c, 4);
+      }
       float x[14];
 #pragma unroll
       for (int c = 0; c < 8; ++c) x[c] = z[c];
       if (FRAME) {
         // lane p owns frame hidden units p + 4e (rows 8 floats apart in four
         // distinct bank groups)
-        float hf[4];
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
           const float4* row = reinterpret_cast<const float4*>(&S.fW1[(p + 4 * e) * 8]);
@@ -215,7 +452,6 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const Backward
           s = dot4(a, make_float4(z[0], z[1], z[2], z[3]), s);
           s = dot4(b, make_float4(z[4], z[5], z[6], z[7]), s);
           hf[e] = fmaxf(s, 0.0f);
-          S.HF[ql][p + 4 * e] = hf[e];
         }
         float r[6];
 #pragma unroll
@@ -229,50 +465,57 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const Backward
         to_local(F, wi[0], wi[1], wi[2], x + 8);
         to_local(F, wo[0], wo[1], wo[2], x + 11);
         if (p == 0) {
-          reinterpret_cast<float4*>(&S.R[ql][0])[0] = make_float4(r[0], r[1], r[2], r[3]);
-          reinterpret_cast<float4*>(&S.R[ql][0])[1] = make_float4(r[4], r[5], 0.0f, 0.0f);
+          reinterpret_cast<float4*>(&G.R[ql][0])[0] = make_float4(r[0], r[1], r[2], r[3]);
+          reinterpret_cast<float4*>(&G.R[ql][0])[1] = make_float4(r[4], r[5], 0.0f, 0.0f);
         }
       } else {
         x[8] = wi[0]; x[9] = wi[1]; x[10] = wi[2];
         x[11] = wo[0]; x[12] = wo[1]; x[13] = wo[2];
       }
       if (p == 0) {
-        float4* X4 = reinterpret_cast<float4*>(&S.X[ql][0]);
+        float4* X4 = reinterpret_cast<float4*>(&G.X[ql][0]);
         X4[0] = make_float4(x[0], x[1], x[2], x[3]);
         X4[1] = make_float4(x[4], x[5], x[6], x[7]);
         X4[2] = make_float4(x[8], x[9], x[10], x[11]);
         X4[3] = make_float4(x[12], x[13], 0.0f, 0.0f);
-        reinterpret_cast<float4*>(&S.Z[ql][0])[0] = make_float4(z[0], z[1], z[2], z[3]);
-        reinterpret_cast<float4*>(&S.Z[ql][0])[1] = make_float4(z[4], z[5], z[6], z[7]);
-        const float cf = cosine ? fmaxf(wi[2], 0.0f) : 1.0f;
-        float4* dy4 = reinterpret_cast<float4*>(&S.DY[ql][0]);
-        if (LOSS) {
-          const float* tg = A.target + 3 * i;
-          if (ALB) {
-            const float* ta = A.target_albedo + 3 * i;
-            dy4[0] = valid ? make_float4(tg[0], tg[1], tg[2], ta[0]) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            dy4[1] = valid ? make_float4(ta[1], ta[2], 0.0f, cf) : make_float4(0.0f, 0.0f, 0.0f, cf);
-          } else {
-            dy4[0] = valid ? make_float4(tg[0], tg[1], tg[2], cf) : make_float4(0.0f, 0.0f, 0.0f, cf);
-          }
-        } else if constexpr (ALB) {
-          // dL/d(output) of the caller, [n][6]; the cosine factor scales the RGB only
-          float dy[6];
-#pragma unroll
-          for (int c = 0; c < 6; ++c) dy[c] = valid ? A.grad_rgb[6 * i + c] * (c < 3 ? cf : 1.0f) : 0.0f;
-          dy4[0] = make_float4(dy[0], dy[1], dy[2], dy[3]);
-          dy4[1] = make_float4(dy[4], dy[5], 0.0f, 0.0f);
-        } else {
-          float dy[3];
-#pragma unroll
-          for (int c = 0; c < 3; ++c) dy[c] = valid ? A.grad_rgb[3 * i + c] * cf : 0.0f;
-          dy4[0] = make_float4(dy[0], dy[1], dy[2], 0.0f);
-        }
+      }
+      // DY: the targets and the cosine factor, or the caller's dL/d(output)
+      // times that factor (which scales the RGB only)
+      const float cf = cosine ? fmaxf(wi[2], 0.0f) : 1.0f;
+      if (p < 3) {
+        G.DY[ql][p] = LOSS ? cur.g0 : cur.g0 * cf;
+        if (ALB) G.DY[ql][3 + p] = cur.g1;
+      } else {
+        G.DY[ql][DW - 1] = LOSS ? cf : 0.0f;
+        if (ALB) G.DY[ql][6] = 0.0f;
       }
     }
+    // the MMAs of the tile before have read A and B: their sums to registers
+    if (tile != tile0) {
+      bad |= !ptx::mbar_wait(bar0 + 24, ph ^ 1u, A.timeout_ns);
+      collect();
+    }
     __syncwarp();
+    // X (with the 1 that meets the bias deltas) and HF as MMA operands
+    if (p < 2) {
+      const float4 a = reinterpret_cast<const float4*>(&G.X[ql][0])[2 * p];
+      const float4 b = reinterpret_cast<const float4*>(&G.X[ql][0])[2 * p + 1];
+      const float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, p ? 1.0f : b.z, b.w};
+      put_terms<8, TB>(G.B + (H / 8 + p) * kBlk + ql * 16, v);
+    }
+    if (FRAME) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        uint16_t w[3];
+        split3_one(hf[e], w[0], w[1], w[2]);
+        uint8_t* o = G.B + (H / 8 + 2 + (e >> 1)) * kBlk + ql * 16 + ((p + 4 * e) & 7) * 2;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) *reinterpret_cast<uint16_t*>(o + k * TB) = w[k];
+      }
+    }
     // ---- half-warp blocks: decoder forward and backward ---------------------
-    uint32_t mask1 = 0;  // bit jj * 4 + qq: layer-1 unit hl + 16 jj of query qb + qq is active
+    float (*H1)[Sm::S] = reinterpret_cast<float (*)[Sm::S]>(G.A);
+    uint32_t sgn2 = 0;  // lane jj * 4 + qq: layer-2 signs of unit hl + 16 jj, query qq of either half-warp
     {
       float a[4][JB];
       // layer 1 (the forward value of y is not needed: dL/dy comes in)
@@ -284,7 +527,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const Backward
       for (int c4 = 0; c4 < 4; ++c4) {
         float4 xv[4];
 #pragma unroll
-        for (int qq = 0; qq < 4; ++qq) xv[qq] = reinterpret_cast<const float4*>(&S.X[qb + qq][0])[c4];
+        for (int qq = 0; qq < 4; ++qq) xv[qq] = reinterpret_cast<const float4*>(&G.X[qb + qq][0])[c4];
 #pragma unroll
         for (int jj = 0; jj < JB; ++jj) {
           const float4 w = reinterpret_cast<const float4*>(&S.W1[hl + 16 * jj][0])[c4];
@@ -296,10 +539,24 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const Backward
       for (int jj = 0; jj < JB; ++jj)
 #pragma unroll
         for (int qq = 0; qq < 4; ++qq) {
-          S.H1[qb + qq][hl + 16 * jj] = fmaxf(a[qq][jj], 0.0f);
-          if (a[qq][jj] > 0.0f) mask1 |= 1u << (jj * 4 + qq);
+          H1[qb + qq][hl + 16 * jj] = fmaxf(a[qq][jj], 0.0f);
+          const uint32_t act = __ballot_sync(0xffffffffu, a[qq][jj] > 0.0f);
+          if (lane == jj * 4 + qq) G.mask1[lw][lane] = act;
         }
       __syncwarp();
+      // H1 as MMA operand: a quarter of a row per lane (eight rows side by
+      // side in each quarter-warp: no bank conflicts)
+      {
+        const float* row = &H1[8 * lw + (lane & 7)][U * (lane >> 3)];
+        float v[U];
+#pragma unroll
+        for (int k = 0; k < U; k += 4) {
+          const float4 x = *reinterpret_cast<const float4*>(row + k);
+          v[k] = x.x; v[k + 1] = x.y; v[k + 2] = x.z; v[k + 3] = x.w;
+        }
+        const int u0 = U * (lane >> 3);
+        put_terms<U, TB>(G.B + (u0 / 8) * kBlk + (8 * lw + (lane & 7)) * 16 + (u0 % 8) * 2, v);
+      }
       // layer 2
 #pragma unroll
       for (int jj = 0; jj < JB; ++jj)
@@ -309,7 +566,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const Backward
       for (int m = 0; m < H / 4; ++m) {
         float4 hv[4];
 #pragma unroll
-        for (int qq = 0; qq < 4; ++qq) hv[qq] = reinterpret_cast<const float4*>(&S.H1[qb + qq][0])[m];
+        for (int qq = 0; qq < 4; ++qq) hv[qq] = reinterpret_cast<const float4*>(&H1[qb + qq][0])[m];
 #pragma unroll
         for (int jj = 0; jj < JB; ++jj) {
           const float4 w = reinterpret_cast<const float4*>(&S.W2[hl + 16 * jj][0])[m];
@@ -319,8 +576,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const Backward
       }
       if (LOSS) {
         // output y = Wo relu(a) + bo of the four queries, summed over the
-        // half-warp; lane (mq, mc) = (hl / 4, hl % 4) takes element mc of
-        // query qb + mq: loss and dL/dy (times the cosine factor) into DY
+        // half-warp; a lane then takes element mc of query qb + mq: loss and dL/dy (times the cosine factor) into DY
         if constexpr (ALB) {
           float y[4][NO];
 #pragma unroll
@@ -359,7 +615,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const Backward
           float tv[DW];  // targets; the cosine factor last
 #pragma unroll
           for (int c4 = 0; c4 < DW / 4; ++c4) {
-            const float4 v = reinterpret_cast<const float4*>(&S.DY[qb + mq][0])[c4];
+            const float4 v = reinterpret_cast<const float4*>(&G.DY[qb + mq][0])[c4];
             tv[4 * c4] = v.x; tv[4 * c4 + 1] = v.y; tv[4 * c4 + 2] = v.z; tv[4 * c4 + 3] = v.w;
           }
           const float cf = tv[DW - 1];
@@ -386,7 +642,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const Backward
               if (vq) lsum += r * r;
               d = 2.0f * r * A.loss_inv;
             }
-            S.DY[qb + mq][e] = vq ? d : 0.0f;
+            G.DY[qb + mq][e] = vq ? d : 0.0f;
           }
           __syncwarp();
         } else {
@@ -406,20 +662,29 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const Backward
               for (int c = 0; c < 3; ++c) y[qq][c] = fmaf(o[c], h, y[qq][c]);
             }
           }
+          // pairs, fours and so on, a lane keeping the queries of its own low
+          // bits: lane hl ends with the sums of query hl & 3
+          float y2[2][3], ys[3];
 #pragma unroll
-          for (int off = 1; off < 16; off <<= 1)
+          for (int k = 0; k < 2; ++k)
 #pragma unroll
-            for (int qq = 0; qq < 4; ++qq)
+            for (int c = 0; c < 3; ++c) {
+              const bool o = hl & 1;
+              y2[k][c] = (o ? y[2 * k + 1][c] : y[2 * k][c]) +
+                         __shfl_xor_sync(0xffffffffu, o ? y[2 * k][c] : y[2 * k + 1][c], 1);
+            }
 #pragma unroll
-              for (int c = 0; c < 3; ++c) y[qq][c] += __shfl_xor_sync(0xffffffffu, y[qq][c], off);
-          const int mq = hl >> 2, mc = hl & 3;
-          float ym = 0.0f;
+          for (int c = 0; c < 3; ++c) {
+            const bool o = hl & 2;
+            ys[c] = (o ? y2[1][c] : y2[0][c]) + __shfl_xor_sync(0xffffffffu, o ? y2[0][c] : y2[1][c], 2);
+          }
 #pragma unroll
-          for (int qq = 0; qq < 4; ++qq)
+          for (int off = 4; off < 16; off <<= 1)
 #pragma unroll
-            for (int c = 0; c < 3; ++c)
-              if (qq == mq && c == mc) ym = y[qq][c];
-          const float4 tv = *reinterpret_cast<const float4*>(&S.DY[qb + mq][0]);
+            for (int c = 0; c < 3; ++c) ys[c] += __shfl_xor_sync(0xffffffffu, ys[c], off);
+          const int mq = hl & 3, mc = hl >> 2;
+          const float ym = mc == 0 ? ys[0] : mc == 1 ? ys[1] : ys[2];
+          const float4 tv = *reinterpret_cast<const float4*>(&G.DY[qb + mq][0]);
           __syncwarp();
           if (mc < 3) {
             const float g = (ym + S.bo[mc]) * tv.w;
@@ -427,102 +692,155 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const Backward
             const float l = log_l1(g, mc == 0 ? tv.x : mc == 1 ? tv.y : tv.z, &gr);
             const bool vq = qb + mq < count;
             if (vq) lsum += l;
-            S.DY[qb + mq][mc] = vq ? gr * A.loss_inv * tv.w : 0.0f;
+            G.DY[qb + mq][mc] = vq ? gr * A.loss_inv * tv.w : 0.0f;
           } else {
-            S.DY[qb + mq][3] = 0.0f;
+            G.DY[qb + mq][3] = 0.0f;
           }
           __syncwarp();
         }
       }
-      // layer-2 delta d2 = (Wo^T dy) where the unit is active
-      if constexpr (ALB) {
+      // output layer's gradient and the layer-2 signs
+      {
         float dyv[4][NO];
 #pragma unroll
         for (int qq = 0; qq < 4; ++qq)
 #pragma unroll
-          for (int c = 0; c < NO; ++c) dyv[qq][c] = S.DY[qb + qq][c];
+          for (int c = 0; c < NO; ++c) {
+            dyv[qq][c] = G.DY[qb + qq][c];
+            gbo[c] += dyv[qq][c];
+          }
 #pragma unroll
-        for (int jj = 0; jj < JB; ++jj) {
-          const int j = hl + 16 * jj;
-          float o[NO];
-#pragma unroll
-          for (int c = 0; c < NO; ++c) o[c] = S.Wo[c * H + j];
+        for (int jj = 0; jj < JB; ++jj)
 #pragma unroll
           for (int qq = 0; qq < 4; ++qq) {
-            const float s = a[qq][jj];
-            float d = o[NO - 1] * dyv[qq][NO - 1];
+            const float h = fmaxf(a[qq][jj], 0.0f);
 #pragma unroll
-            for (int c = NO - 2; c >= 0; --c) d = fmaf(o[c], dyv[qq][c], d);
-            S.H2[qb + qq][j] = fmaxf(s, 0.0f);
-            S.D2[qb + qq][j] = s > 0.0f ? d : 0.0f;
+            for (int c = 0; c < NO; ++c) gwo[c][jj] = fmaf(dyv[qq][c], h, gwo[c][jj]);
+            const uint32_t act = __ballot_sync(0xffffffffu, a[qq][jj] > 0.0f);
+            if (lane == jj * 4 + qq) sgn2 = act;
           }
-        }
-      } else {
-        float4 dyv[4];
-#pragma unroll
-        for (int qq = 0; qq < 4; ++qq) dyv[qq] = *reinterpret_cast<const float4*>(&S.DY[qb + qq][0]);
-#pragma unroll
-        for (int jj = 0; jj < JB; ++jj) {
-          const int j = hl + 16 * jj;
-          const float o0 = S.Wo[j], o1 = S.Wo[H + j], o2 = S.Wo[2 * H + j];
-#pragma unroll
-          for (int qq = 0; qq < 4; ++qq) {
-            const float s = a[qq][jj];
-            S.H2[qb + qq][j] = fmaxf(s, 0.0f);
-            S.D2[qb + qq][j] = s > 0.0f ? fmaf(o0, dyv[qq].x, fmaf(o1, dyv[qq].y, o2 * dyv[qq].z)) : 0.0f;
-          }
-        }
       }
-      __syncwarp();
-      // layer-1 delta d1 = (W2^T d2) where the unit is active; W2 is read by
-      // column (unit k of lane hl is column hl + 16 kk)
-#pragma unroll
-      for (int kk = 0; kk < JB; ++kk)
-#pragma unroll
-        for (int qq = 0; qq < 4; ++qq) a[qq][kk] = 0.0f;
-#pragma unroll 2
-      for (int m = 0; m < H / 4; ++m) {
-        float4 dv[4];
-#pragma unroll
-        for (int qq = 0; qq < 4; ++qq) dv[qq] = reinterpret_cast<const float4*>(&S.D2[qb + qq][0])[m];
-#pragma unroll
-        for (int kk = 0; kk < JB; ++kk) {
-          const float4 w = make_float4(S.W2[4 * m][hl + 16 * kk], S.W2[4 * m + 1][hl + 16 * kk],
-                                       S.W2[4 * m + 2][hl + 16 * kk], S.W2[4 * m + 3][hl + 16 * kk]);
-#pragma unroll
-          for (int qq = 0; qq < 4; ++qq) a[qq][kk] = dot4(w, dv[qq], a[qq][kk]);
-        }
-      }
-#pragma unroll
-      for (int kk = 0; kk < JB; ++kk)
-#pragma unroll
-        for (int qq = 0; qq < 4; ++qq)
-          S.D1[qb + qq][hl + 16 * kk] = ((mask1 >> (kk * 4 + qq)) & 1u) ? a[qq][kk] : 0.0f;
     }
-    __syncwarp();
-    // ---- quad: dL/dx, frame backward, pyramid scatter ------------------------
+    // every warp has read its H1 rows: A takes D2
+    if (ptx::bar_red_or(bid + 4, kBwdGroup, bad)) {
+      stop = true;
+      break;
+    }
+    // ---- layer-2 delta d2 = (Wo^T dy) where the unit is active ---------------
     {
-      // dx[4p .. 4p+3] = sum_k W1[k][4p ..] d1[k]
-      float4 dxp = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-#pragma unroll 4
-      for (int k4 = 0; k4 < H / 4; ++k4) {
-        const float4 d = reinterpret_cast<const float4*>(&S.D1[ql][0])[k4];
-        const float dk[4] = {d.x, d.y, d.z, d.w};
+      const int row = lane & 7, q = 8 * lw + row, u0 = U * (lane >> 3);
+      const uint32_t bits = __shfl_sync(0xffffffffu, sgn2, (u0 / 16) * 4 + (row & 3)) >> (16 * (row >> 2) + u0 % 16);
+      float dy[NO], v[U];
+#pragma unroll
+      for (int c = 0; c < NO; ++c) dy[c] = G.DY[q][c];
+#pragma unroll
+      for (int k = 0; k < U; k += 4) {
+        float o[NO][4];
+#pragma unroll
+        for (int c = 0; c < NO; ++c) {
+          const float4 w = *reinterpret_cast<const float4*>(&S.Wo[c * H + u0 + k]);
+          o[c][0] = w.x; o[c][1] = w.y; o[c][2] = w.z; o[c][3] = w.w;
+        }
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-          const float4 w = reinterpret_cast<const float4*>(&S.W1[4 * k4 + e][0])[p];
-          dxp.x = fmaf(w.x, dk[e], dxp.x);
-          dxp.y = fmaf(w.y, dk[e], dxp.y);
-          dxp.z = fmaf(w.z, dk[e], dxp.z);
-          dxp.w = fmaf(w.w, dk[e], dxp.w);
+          float d = o[NO - 1][e] * dy[NO - 1];
+#pragma unroll
+          for (int c = NO - 2; c >= 0; --c) d = fmaf(o[c][e], dy[c], d);
+          v[k + e] = (bits >> (k + e)) & 1u ? d : 0.0f;
         }
       }
-      reinterpret_cast<float4*>(&S.DX[ql][0])[p] = dxp;
+      put_terms<U, TA>(G.A + (u0 / 8) * kBlk + q * 16 + (u0 % 8) * 2, v);
+    }
+    ptx::fence_proxy_async();
+    ptx::tc_fence_before();
+    ++issued;
+    // D2 written: d1 = D2 W2 (warp 0), C2 = D2^T [H1 | X 1] (warp 7)
+    if (lw == 0) {
+      ptx::bar_sync(bid + 1, kBwdGroup);
+      if (ptx::elect()) {
+        ptx::tc_fence_after();
+        products(tmem + cD1, ptx::sdesc(aK, kBlk, 128), TA, 2 * kBlk, ptx::sdesc(ptx::smem_u32(S.W2T), H * 16, 128),
+                 H * H * 2, 2 * H * 16, H / 16, ptx::idesc_bf16(128, H));
+        ptx::mma_commit(bar0);
+      }
       __syncwarp();
+    } else if (lw == 7) {
+      ptx::bar_sync(bid + 1, kBwdGroup);
+      if (ptx::elect()) {
+        ptx::tc_fence_after();
+        products(tmem + cC2, ptx::sdesc(aM, 128, kBlk), TA, 256, ptx::sdesc(aB, 128, kBlk), TB, 256, kBwdQ / 16,
+                 ptx::idesc_bf16(128, N2) | kMN);
+        ptx::mma_commit(bar0 + 8);
+      }
+      __syncwarp();
+    } else {
+      ptx::bar_arrive(bid + 1, kBwdGroup);
+    }
+    // ---- layer-1 delta d1 = (W2^T d2) where the unit is active ---------------
+    {
+      bad |= !ptx::mbar_wait(bar0, ph, A.timeout_ns);
+      ptx::tc_fence_after();
+      const int u0 = U * gq;
+      const uint32_t bits = G.mask1[grow >> 3][(u0 / 16) * 4 + (grow & 3)] >> (16 * ((grow >> 2) & 1) + u0 % 16);
+      uint32_t d[U];
+#pragma unroll
+      for (int k = 0; k < U; k += 4) ptx::tmem_ld4(tl + cD1 + u0 + k, *reinterpret_cast<uint32_t(*)[4]>(&d[k]));
+      ptx::tmem_ld_wait();
+      float v[U];
+#pragma unroll
+      for (int k = 0; k < U; ++k) v[k] = (bits >> k) & 1u ? __uint_as_float(d[k]) : 0.0f;
+      bad |= !ptx::mbar_wait(bar0 + 8, ph, A.timeout_ns);  // C2 has read D2
+      put_terms<U, TA>(G.A + (u0 / 8) * kBlk + grow * 16 + (u0 % 8) * 2, v);
+    }
+    ptx::fence_proxy_async();
+    ptx::tc_fence_before();
+    // D1 written: dx = D1 W1 (warp 2), C1 = D1^T [X 1] (warp 6)
+    if (lw == 2) {
+      ptx::bar_sync(bid + 2, kBwdGroup);
+      if (ptx::elect()) {
+        ptx::tc_fence_after();
+        products(tmem + cDX, ptx::sdesc(aK, kBlk, 128), TA, 2 * kBlk, ptx::sdesc(ptx::smem_u32(S.W1T), 256, 128),
+                 16 * H * 2, 512, H / 16, ptx::idesc_bf16(128, 16));
+        ptx::mma_commit(bar0 + 16);
+      }
+      __syncwarp();
+    } else if (lw == 6) {
+      ptx::bar_sync(bid + 2, kBwdGroup);
+      if (ptx::elect()) {
+        ptx::tc_fence_after();
+        products(tmem + cC1, ptx::sdesc(aM, 128, kBlk), TA, 256, ptx::sdesc(aB + (H / 8) * kBlk, 128, kBlk), TB, 256,
+                 kBwdQ / 16, ptx::idesc_bf16(128, 16) | kMN);
+        ptx::mma_commit(bar0 + 24);
+      }
+      __syncwarp();
+    } else {
+      ptx::bar_arrive(bid + 2, kBwdGroup);
+    }
+    // ---- dL/dx to its rows ----------------------------------------------------
+    if (gq == 0) {
+      bad |= !ptx::mbar_wait(bar0 + 16, ph, A.timeout_ns);
+      ptx::tc_fence_after();
+      uint32_t d[16];
+      ptx::tmem_ld16(tl + cDX, d);
+      ptx::tmem_ld_wait();
+#pragma unroll
+      for (int c4 = 0; c4 < 4; ++c4)
+        *reinterpret_cast<uint4*>(&G.X[grow][4 * c4]) =
+            make_uint4(d[4 * c4], d[4 * c4 + 1], d[4 * c4 + 2], d[4 * c4 + 3]);
+      ptx::tc_fence_before();
+    }
+    if (ptx::bar_red_or(bid + 4, kBwdGroup, bad)) {
+      // (the other half of C1's and CF's barrier)
+      if (lw == 5 && ptx::elect()) ptx::mma_commit(bar0 + 24);
+      stop = true;
+      break;
+    }
+    // ---- quad: frame backward, pyramid scatter --------------------------------
+    {
       float dx[16];
 #pragma unroll
       for (int c4 = 0; c4 < 4; ++c4) {
-        const float4 d = reinterpret_cast<const float4*>(&S.DX[ql][0])[c4];
+        const float4 d = reinterpret_cast<const float4*>(&G.X[ql][0])[c4];
         dx[4 * c4] = d.x; dx[4 * c4 + 1] = d.y; dx[4 * c4 + 2] = d.z; dx[4 * c4 + 3] = d.w;
       }
       float dz[8];
@@ -531,8 +849,8 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const Backward
       if (FRAME) {
         float r[6];
         {
-          const float4 r0 = reinterpret_cast<const float4*>(&S.R[ql][0])[0];
-          const float4 r1 = reinterpret_cast<const float4*>(&S.R[ql][0])[1];
+          const float4 r0 = reinterpret_cast<const float4*>(&G.R[ql][0])[0];
+          const float4 r1 = reinterpret_cast<const float4*>(&G.R[ql][0])[1];
           r[0] = r0.x; r[1] = r0.y; r[2] = r0.z; r[3] = r0.w; r[4] = r1.x; r[5] = r1.y;
         }
         const Frame F = build_frame(r);
@@ -548,8 +866,12 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const Backward
         const float c1_ = F.n[2] * F.t[0] - F.n[0] * F.t[2];
         const float c2_ = F.n[0] * F.t[1] - F.n[1] * F.t[0];
         const float cl = sqrtf(c0_ * c0_ + c1_ * c1_ + c2_ * c2_);
-        const float wi[3] = {A.q.wix[i], A.q.wiy[i], A.q.wiz[i]};
-        const float wo[3] = {A.q.wox[i], A.q.woy[i], A.q.woz[i]};
+        float wi[3], wo[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          wi[c] = __shfl_sync(0xffffffffu, cur.f1, c, 4);
+          wo[c] = __shfl_sync(0xffffffffu, cur.f2, c, 4);
+        }
         // x' = T w: dT row k += dx'_k w
         float dt[3], db[3], dn[3];
 #pragma unroll
@@ -560,9 +882,10 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const Backward
         }
         // b = c / |c|, c = n x t
         const float bdb = F.b[0] * db[0] + F.b[1] * db[1] + F.b[2] * db[2];
+        const float icl = 1.0f / cl;
         float gc[3];
 #pragma unroll
-        for (int k = 0; k < 3; ++k) gc[k] = (db[k] - F.b[k] * bdb) / cl;
+        for (int k = 0; k < 3; ++k) gc[k] = (db[k] - F.b[k] * bdb) * icl;
         dn[0] += F.t[1] * gc[2] - F.t[2] * gc[1];
         dn[1] += F.t[2] * gc[0] - F.t[0] * gc[2];
         dn[2] += F.t[0] * gc[1] - F.t[1] * gc[0];
@@ -572,9 +895,10 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const Backward
         float dr[6] = {0, 0, 0, 0, 0, 0};
         if (!tdeg) {
           const float tdt = F.t[0] * dt[0] + F.t[1] * dt[1] + F.t[2] * dt[2];
+          const float itpl = 1.0f / tpl;
           float dtp[3];
 #pragma unroll
-          for (int k = 0; k < 3; ++k) dtp[k] = (dt[k] - F.t[k] * tdt) / tpl;
+          for (int k = 0; k < 3; ++k) dtp[k] = (dt[k] - F.t[k] * tdt) * itpl;
           const float ndtp = F.n[0] * dtp[0] + F.n[1] * dtp[1] + F.n[2] * dtp[2];
 #pragma unroll
           for (int k = 0; k < 3; ++k) {
@@ -584,8 +908,9 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const Backward
         }
         if (!ndeg) {
           const float ndn = F.n[0] * dn[0] + F.n[1] * dn[1] + F.n[2] * dn[2];
+          const float inl = 1.0f / nl;
 #pragma unroll
-          for (int k = 0; k < 3; ++k) dr[k] += (dn[k] - F.n[k] * ndn) / nl;
+          for (int k = 0; k < 3; ++k) dr[k] += (dn[k] - F.n[k] * ndn) * inl;
         }
         if (!valid) {
 #pragma unroll
@@ -598,12 +923,16 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const Backward
           float g = 0.0f;
 #pragma unroll
           for (int j = 0; j < 6; ++j) g = fmaf(S.fW2[j * 16 + p + 4 * e], dr[j], g);
-          dhf[e] = S.HF[ql][p + 4 * e] > 0.0f ? g : 0.0f;
-          S.DHF[ql][p + 4 * e] = dhf[e];
+          dhf[e] = hf[e] > 0.0f ? g : 0.0f;
+          uint16_t w[3];
+          split3_one(dhf[e], w[0], w[1], w[2]);
+          uint8_t* o = G.A + (H / 8 + (e >> 1)) * kBlk + ql * 16 + ((p + 4 * e) & 7) * 2;
+#pragma unroll
+          for (int k = 0; k < 3; ++k) *reinterpret_cast<uint16_t*>(o + k * TA) = w[k];
         }
         if (p == 0) {
-          reinterpret_cast<float4*>(&S.DR[ql][0])[0] = make_float4(dr[0], dr[1], dr[2], dr[3]);
-          reinterpret_cast<float4*>(&S.DR[ql][0])[1] = make_float4(dr[4], dr[5], 0.0f, 0.0f);
+          const float v[8] = {dr[0], dr[1], dr[2], dr[3], dr[4], dr[5], 0.0f, 0.0f};
+          put_terms<8, TA>(G.A + (H / 8 + 2) * kBlk + ql * 16, v);
         }
         float gz[8];
 #pragma unroll
@@ -620,6 +949,25 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const Backward
 #pragma unroll
         for (int c = 0; c < 8; ++c) dz[c] += quad_sum(gz[c]);
       }
+      // DHF, DR written: CF = [DHF | DR]^T [X 1 | HF] (warp 5), which runs
+      // while the texels take their gradients
+      ptx::fence_proxy_async();
+      ptx::tc_fence_before();
+      if (lw == 5) {
+        ptx::bar_sync(bid + 3, kBwdGroup);
+        if (ptx::elect()) {
+          ptx::tc_fence_after();
+          if (FRAME)
+            products(tmem + cCF, ptx::sdesc(aM + (H / 8) * kBlk, 128, kBlk), TA, 256,
+                     ptx::sdesc(aB + (H / 8) * kBlk, 128, kBlk), TB, 256, kBwdQ / 16, ptx::idesc_bf16(128, 32) | kMN);
+          ptx::mma_commit(bar0 + 24);
+        }
+        __syncwarp();
+      } else {
+        ptx::bar_arrive(bid + 3, kBwdGroup);
+      }
+      const float u = __shfl_sync(0xffffffffu, cur.f0, 0, 4), v = __shfl_sync(0xffffffffu, cur.f0, 1, 4);
+      const float lod = __shfl_sync(0xffffffffu, cur.f0, 2, 4), xi = __shfl_sync(0xffffffffu, cur.f0, 3, 4);
       if (A.dz_out) {
         // encoder phase: dL/dz goes to the encoder's backward
         if (valid && p == 0) {
@@ -628,8 +976,6 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const Backward
         }
       } else if (valid && A.grad_pyramid) {
         // pyramid scatter: z = sum_k w_k texel_k  =>  dtexel_k += w_k dz
-        const float u = A.q.u[i], v = A.q.v[i], lod = A.q.lod[i];
-        const float xi = A.q.xi ? A.q.xi[i] : 0.0f;
         LevelPick lp = pick_levels(A.pyr, lod);
         int lv[2];
         float lw[2];
@@ -684,68 +1030,100 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const Backward
         }
       }
     }
-    __syncthreads();
-    // =================== phase B ===========================================
-    if (role >= 0) {
-#pragma unroll 2
-      for (int qq = 0; qq < count; ++qq) {
-        const float4 d = *reinterpret_cast<const float4*>(dp + qq * dstride);
-        const float4 a = *reinterpret_cast<const float4*>(ap + qq * astride);
-        const float dv[4] = {d.x, d.y, d.z, d.w};
-        const float av[4] = {a.x, a.y, a.z, a.w};
-#pragma unroll
-        for (int rr = 0; rr < 4; ++rr) {
-#pragma unroll
-          for (int cc = 0; cc < 4; ++cc) acc[4 * rr + cc] = fmaf(dv[rr], av[cc], acc[4 * rr + cc]);
-          accb[rr] += dv[rr];
-        }
-      }
-    }
-    __syncthreads();
   }
   // ---- flush: one atomic per parameter and coarse texel channel per CTA -------
-  // (the last tile ended with a barrier)
+  if (stop) {
+    bad = true;
+  } else if (tile0 < ntiles) {
+    bad |= !ptx::mbar_wait(bar0 + 24, ph ^ 1u, A.timeout_ns);
+    collect();
+  }
   if (LOSS) {
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, off);
-    if ((t & 31) == 0) S.lred[t >> 5] = lsum;
-    __syncthreads();
-    if (t == 0) {
+    if (lane == 0) S.lred[warp] = lsum;
+  }
+#pragma unroll
+  for (int c = 0; c < NO; ++c) {
+#pragma unroll
+    for (int jj = 0; jj < JB; ++jj) atomicAdd(&S.gwo[c * H + hl + 16 * jj], gwo[c][jj]);
+    if (hl == 0) atomicAdd(&S.gwo[NO * H + c], gbo[c]);
+  }
+  if (!__syncthreads_or(bad)) {
+    if (LOSS && t == 0) {
       float tot = 0.0f;
       for (int w = 0; w < 16; ++w) tot += S.lred[w];
       atomicAdd(A.loss_acc, tot * A.loss_inv);
     }
-  }
-  for (int k = t; k < 8 * A.tiny_n; k += kBwdThreads) {
-    float c = 0.0f;
-    for (int w = 0; w < 16; ++w) c += wacc[w * 8 * A.tiny_n + k];
-    if (c != 0.0f) atomicAdd(A.grad_pyramid + A.tiny_tex0 * 8 + k, c);
-  }
-  for (int k = t; k < 8 * A.cta_n; k += kBwdThreads) {
-    const float c = cacc[k];
-    if (c != 0.0f) atomicAdd(A.grad_pyramid + A.cta_tex0 * 8 + k, c);
-  }
-  if (role < 0) return;
-  float* g = A.grad_params;
-  const int o = FRAME ? 246 : 0;
-  const int oW1 = o, ob1 = o + 14 * H, oW2 = ob1 + H, ob2 = oW2 + H * H, oWo = ob2 + H, obo = oWo + NO * H;
-  // (weight offset, row stride, valid rows, valid columns, bias offset)
-  int wo_ = 0, ws = 0, nr = 0, nc = 0, bo_ = 0;
-  switch (role) {
-    case 0: wo_ = oW2; ws = H; nr = H; nc = H; bo_ = ob2; break;
-    case 1: wo_ = oW1; ws = 14; nr = H; nc = 14; bo_ = ob1; break;
-    case 2: wo_ = oWo; ws = H; nr = NO; nc = H; bo_ = obo; break;
-    case 3: wo_ = 0; ws = 8; nr = 16; nc = 8; bo_ = 128; break;
-    default: wo_ = 144; ws = 16; nr = 6; nc = 16; bo_ = 240; break;
-  }
+    for (int k = t; k < 8 * A.tiny_n; k += kBwdThreads) {
+      float c = 0.0f;
+      for (int w = 0; w < 16; ++w) c += wacc[w * 8 * A.tiny_n + k];
+      if (c != 0.0f) atomicAdd(A.grad_pyramid + A.tiny_tex0 * 8 + k, c);
+    }
+    for (int k = t; k < 8 * A.cta_n; k += kBwdThreads) {
+      const float c = cacc[k];
+      if (c != 0.0f) atomicAdd(A.grad_pyramid + A.cta_tex0 * 8 + k, c);
+    }
+    // Both groups' sums of C2, C1 and CF meet in shared memory (odd row
+    // lengths: no bank conflicts; the first group's operands are done with),
+    // so that the atomics run along the parameters and once per CTA (straight
+    // from the registers, a row per lane, they took 20 us more).
+    constexpr int R2 = N2 + 1, R1 = 17, RF = 33;
+    float* s2 = reinterpret_cast<float*>(S.g[0].A);
+    float* s1 = s2 + H * R2;
+    float* sf = s1 + H * R1;
+    static_assert((H * (R2 + R1) + 22 * RF) * 4 <= 3 * TA, "the sums do not fit");
 #pragma unroll
-  for (int rr = 0; rr < 4; ++rr) {
-    const int row = r0 + rr;
-    if (row >= nr) continue;
+    for (int k = 0; k < 2; ++k) {
+      if (grp == k) {
+        auto put = [&](float* d, float v) { *d = k ? *d + v : v; };
+        if (grow < H) {
 #pragma unroll
-    for (int cc = 0; cc < 4; ++cc)
-      if (c0 + cc < nc) atomicAdd(&g[wo_ + row * ws + c0 + cc], acc[4 * rr + cc]);
-    if (c0 == 0) atomicAdd(&g[bo_ + row], accb[rr]);
+          for (int c = 0; c < N2 / 4; ++c) put(s2 + grow * R2 + gq * (N2 / 4) + c, acc2[c]);
+#pragma unroll
+          for (int c = 0; c < 4; ++c) put(s1 + grow * R1 + gq * 4 + c, acc1[c]);
+        }
+        if (FRAME && grow < 22) {
+#pragma unroll
+          for (int c = 0; c < 8; ++c) put(sf + grow * RF + gq * 8 + c, accf[c]);
+        }
+      }
+      __syncthreads();
+    }
+    float* g = A.grad_params;
+    constexpr int o = FRAME ? 246 : 0;
+    constexpr int ob1 = o + 14 * H, oW2 = ob1 + H, ob2 = oW2 + H * H, oWo = ob2 + H;
+    if (FRAME) {
+      // rows: DHF, DR; columns: X (the 1 in column 14), HF
+      for (int k = t; k < 246; k += kBwdThreads)
+        atomicAdd(&g[k], k < 128   ? sf[(k >> 3) * RF + (k & 7)]
+                         : k < 144 ? sf[(k - 128) * RF + 14]
+                         : k < 240 ? sf[(16 + (k - 144) / 16) * RF + 16 + (k - 144) % 16]
+                                   : sf[(k - 224) * RF + 14]);
+    }
+    for (int k = t; k < 14 * H; k += kBwdThreads) atomicAdd(&g[o + k], s1[k / 14 * R1 + k % 14]);
+    for (int k = t; k < H; k += kBwdThreads) {
+      atomicAdd(&g[ob1 + k], s1[k * R1 + 14]);
+      atomicAdd(&g[ob2 + k], s2[k * R2 + H + 14]);
+    }
+    for (int k = t; k < H * H; k += kBwdThreads) atomicAdd(&g[oW2 + k], s2[k / H * R2 + k % H]);
+    for (int k = t; k < NO * H + NO; k += kBwdThreads) atomicAdd(&g[oWo + k], S.gwo[k]);  // weights, then the bias
+  }
+
+  // ---- teardown ----------------------------------------------------------------
+  // MMAs in flight after a wait gave up are waited for with the fixed drain
+  // limit, and TMEM is freed only if they completed.
+  bool drained = true;
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+    if (issued > 0) drained &= ptx::mbar_wait(bar0 + 8 * k, (issued - 1) & 1u, ptx::kDrainTimeoutNs);
+  if (bad) record_error(A.err, DEVERR_WAIT_TIMEOUT);
+  if (!drained) record_error(A.err, DEVERR_DRAIN_TIMEOUT);
+  ptx::tc_fence_before();
+  const bool all_drained = __syncthreads_and(drained ? 1 : 0) != 0;
+  if (warp == 0 && all_drained) {
+    ptx::tc_fence_after();
+    ptx::tmem_dealloc(S.tslot, 512);
   }
 }
 

@@ -68,17 +68,6 @@ struct F32Smem {
   static constexpr int BYTES = TSLOT_OFF + 16;
 };
 
-// (a, b) -> the three bf16 pairs of the cut-off split (a in the low half)
-__device__ __forceinline__ void split3(float a, float b, uint32_t& h, uint32_t& m, uint32_t& l) {
-  auto top = [](float x) { return __uint_as_float(__float_as_uint(x) & 0xFFFF0000u); };
-  auto pack = [](float x, float y) { return __byte_perm(__float_as_uint(x), __float_as_uint(y), 0x7632); };
-  h = pack(a, b);
-  const float2 r = ptx::sub2(make_float2(a, b), make_float2(top(a), top(b)));
-  m = pack(r.x, r.y);
-  const float2 q = ptx::sub2(r, make_float2(top(r.x), top(r.y)));
-  l = pack(q.x, q.y);
-}
-
 // One query with the weights in global memory: for the rows whose inputs are
 // not finite (an infinity has no split), with the per-thread kernel's results.
 template <int H, int NH, int FK, bool F16P>
@@ -344,7 +333,7 @@ __global__ void __launch_bounds__((NCH + NF) * 128, 1)
       for (int k0 = 0; k0 < KX; k0 += 16) {
         uint32_t h[8], m[8], l[8];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) split3(x[k0 + 2 * j], x[k0 + 2 * j + 1], h[j], m[j], l[j]);
+        for (int j = 0; j < 8; ++j) ptx::split3(x[k0 + 2 * j], x[k0 + 2 * j + 1], h[j], m[j], l[j]);
         ptx::tmem_st8(tX + lane + k0 / 2, h);
         ptx::tmem_st8(tX + lane + KX / 2 + k0 / 2, m);
         ptx::tmem_st8(tX + lane + KX + k0 / 2, l);
@@ -364,7 +353,7 @@ __global__ void __launch_bounds__((NCH + NF) * 128, 1)
           uint32_t h[8], m[8], l[8];
 #pragma unroll
           for (int j = 0; j < 8; ++j)
-            split3(fmaxf(f32_of(acc[2 * j]), 0.0f), fmaxf(f32_of(acc[2 * j + 1]), 0.0f), h[j], m[j], l[j]);
+            ptx::split3(fmaxf(f32_of(acc[2 * j]), 0.0f), fmaxf(f32_of(acc[2 * j + 1]), 0.0f), h[j], m[j], l[j]);
           ptx::tmem_st8(tX + lane + c0 / 2, h);
           ptx::tmem_st8(tX + lane + H / 2 + c0 / 2, m);
           ptx::tmem_st8(tX + lane + H + c0 / 2, l);

@@ -201,6 +201,8 @@ struct BackwardArgs {
   float* grad_pyramid;     // may be null
   uint32_t flags;
   int num_sms;
+  int* err;                // the context's device error word
+  uint64_t timeout_ns;     // limit of every wait
   // set by the launcher: the gradient of texels [tiny_tex0, texels) is summed
   // in per-warp shared copies, that of [cta_tex0, tiny_tex0) in one shared
   // copy per CTA, before it reaches the global buffer

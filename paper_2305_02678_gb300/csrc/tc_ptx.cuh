@@ -296,6 +296,18 @@ __device__ __forceinline__ float2 sub2(float2 a, float2 b) {
   asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(rd) : "l"(ra), "l"(rb));
   return *reinterpret_cast<float2*>(&rd);
 }
+// (a, b) -> the three bf16 pairs (a in the low half) of x = x_h + x_m + x_l:
+// each term the next eight significant bits of x, cut off, so that the sum is
+// x itself.
+__device__ __forceinline__ void split3(float a, float b, uint32_t& h, uint32_t& m, uint32_t& l) {
+  auto top = [](float x) { return __uint_as_float(__float_as_uint(x) & 0xFFFF0000u); };
+  auto pack = [](float x, float y) { return __byte_perm(__float_as_uint(x), __float_as_uint(y), 0x7632); };
+  h = pack(a, b);
+  const float2 r = sub2(make_float2(a, b), make_float2(top(a), top(b)));
+  m = pack(r.x, r.y);
+  const float2 q = sub2(r, make_float2(top(r.x), top(r.y)));
+  l = pack(q.x, q.y);
+}
 // Read-only global load that the compiler keeps where it is written (the
 // value's first use waits on it, wherever that is).
 __device__ __forceinline__ float ld_nc_pinned(const float* p) {
@@ -359,6 +371,13 @@ __device__ __forceinline__ bool bar_red_or(uint32_t id, uint32_t nthreads, bool 
       : "r"((uint32_t)v), "r"(id), "r"(nthreads)
       : "memory");
   return r != 0;
+}
+// Named barrier `id` over `nthreads` threads: waiting, and arriving only.
+__device__ __forceinline__ void bar_sync(uint32_t id, uint32_t nthreads) {
+  asm volatile("barrier.cta.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
+}
+__device__ __forceinline__ void bar_arrive(uint32_t id, uint32_t nthreads) {
+  asm volatile("barrier.cta.arrive %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
 __device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
   asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d)

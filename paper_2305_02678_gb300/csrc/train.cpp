@@ -61,6 +61,8 @@ static void fill_bwd(nam_ctx* ctx, nam_material m, const nam_queries* q, int64_t
   a->grad_pyramid = grad_pyramid;
   a->flags = flags;
   a->num_sms = ctx->num_sms;
+  a->err = ctx->err_word;
+  a->timeout_ns = ctx->timeout_ns;
 }
 
 extern "C" nam_status nam_backward(nam_ctx* ctx, nam_material m, const nam_queries* q, int64_t n,

@@ -97,6 +97,8 @@ extern "C" nam_status nam_train_step_noalloc(nam_ctx* ctx, nam_material m, const
   a.grad_pyramid = m->grad + m->pyr_off;
   a.flags = flags;
   a.num_sms = ctx->num_sms;
+  a.err = ctx->err_word;
+  a.timeout_ns = ctx->timeout_ns;
   if (!e) e = launch_backward(a, s);
   const int64_t np = m->n_params, po = m->pyr_off, nt = m->pyr.texels * 8;
   if (!e)
