@@ -50,6 +50,7 @@
 // the coarsest levels is summed in shared memory first (per warp for the
 // tiniest ones, per CTA for the next) and added to the global buffer once
 // per CTA.
+#include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
 #include "common.cuh"
@@ -109,6 +110,18 @@ __device__ __forceinline__ void split3_one(float x, uint16_t& h, uint16_t& m, ui
   h = (uint16_t)(b >> 16);
   m = (uint16_t)(br >> 16);
   l = (uint16_t)(__float_as_uint(q) >> 16);
+}
+// the same of a weight, rounded to nearest: terms of either sign, so that what
+// the six products leave out (middle times last, last times last) has no sign
+// of its own, and a little (4e-8) larger, for the accumulator, which cuts off:
+// dL/dz came out 1.6e-7 too small without either
+__device__ __forceinline__ void split3_weight(float x, uint16_t& h, uint16_t& m, uint16_t& l) {
+  const __nv_bfloat16 a = __float2bfloat16_rn(x);
+  const float r = x - __bfloat162float(a);
+  const __nv_bfloat16 b = __float2bfloat16_rn(r);
+  h = __bfloat16_as_ushort(a);
+  m = __bfloat16_as_ushort(b);
+  l = __bfloat16_as_ushort(__float2bfloat16_rn(fmaf(x, 4e-8f, r - __bfloat162float(b))));
 }
 // U values (consecutive units) of one query to their rows of the three terms;
 // p: the first unit's place in term 0, TS: bytes of a term
@@ -288,7 +301,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const Backward
     for (int i = t; i < H * H; i += kBwdThreads) {
       const int j = i / H, k = i % H;  // W2[j][k] -> row k, K index j
       uint16_t w[3];
-      split3_one(W2[i], w[0], w[1], w[2]);
+      split3_weight(W2[i], w[0], w[1], w[2]);
 #pragma unroll
       for (int e = 0; e < 3; ++e)
         *reinterpret_cast<uint16_t*>(S.W2T + e * H * H * 2 + (j / 8) * (H * 16) + k * 16 + (j % 8) * 2) = w[e];
@@ -296,7 +309,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const Backward
     for (int i = t; i < H * 16; i += kBwdThreads) {
       const int j = i / 16, c = i % 16;
       uint16_t w[3];
-      split3_one(c < 14 ? W1[j * 14 + c] : 0.0f, w[0], w[1], w[2]);
+      split3_weight(c < 14 ? W1[j * 14 + c] : 0.0f, w[0], w[1], w[2]);
 #pragma unroll
       for (int e = 0; e < 3; ++e)
         *reinterpret_cast<uint16_t*>(S.W1T + e * 16 * H * 2 + (j / 8) * 256 + c * 16 + (j % 8) * 2) = w[e];
