@@ -5,236 +5,301 @@
 // per texel to initialise the texture.
 //
 // Forward (encode_kernel): one thread per row, weights in shared memory.
-// Backward (encoder_backward_kernel): a CTA of 128 threads takes tiles of 128
-// rows; phase A (thread = row) recomputes the forward and back-propagates
-// dL/dz to the hidden pre-activations, keeping the layer inputs and deltas of
-// the tile in shared memory; phase B (thread = 4x4 block of one weight
-// matrix) sums the outer products over the tile in registers; one atomic per
-// parameter per CTA at the end.
+// Backward (encoder_backward_kernel): a warp takes 32 rows; with a lane per row
+// it recomputes the forward and back-propagates dL/dz, and between the layers,
+// with a lane per block of a weight matrix, it sums that layer's outer products
+// over the rows in registers.  Warps wait for none but themselves; their sums
+// meet in shared memory, one atomic per parameter and CTA at the end.
+// Both are bound by the latency of a row's chain of packed FMAs and shared
+// loads at eight warps per SM, which the registers of fully unrolled layers
+// leave (more warps with spilled registers were slower).  131,072 rows, four
+// inputs: forward 19 us (a dot product per unit, 16 padded inputs: 32),
+// backward 40 us (with tiles of 128 rows per CTA and barriers between a row
+// phase and a block phase: 71).
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "nam_internal.h"
+#include "tc_ptx.cuh"
 
 namespace nam {
 namespace {
 
 constexpr int kE = 32;        // hidden width
 constexpr int kKMax = 16;     // inputs, padded
-constexpr int kTile = 128;    // rows per backward tile
+constexpr int kBwdThreads = 128;
+constexpr int kBwdCtas = 2;   // per SM
 
-// weights in shared memory, rows padded to 16-byte multiples
+// Weights in shared memory, an input's weights side by side, so that one
+// broadcast load feeds two packed FMAs on neighbouring units and the unit sums
+// stay in registers (a dot product per unit took a load for every four FMAs).
+// KP: inputs, padded to a multiple of four.
+template <int KP>
 struct EncW {
-  float W1[kE][kKMax];  // zero beyond K
+  float W1T[KP][kE];  // zero beyond K
   float b1[kE];
-  float W2[kE][kE];
+  float W2T[kE][kE];
   float b2[kE];
-  float W3[8][kE];
   float b3[8];
 };
 
-__device__ void load_encoder(EncW& S, const float* __restrict__ p, int K, int t, int nt) {
-  for (int i = t; i < kE * kKMax; i += nt) {
-    const int j = i / kKMax, c = i % kKMax;
-    S.W1[j][c] = c < K ? p[j * K + c] : 0.0f;
+template <int KP>
+__device__ void load_encoder(EncW<KP>& S, const float* __restrict__ p, int K, int t, int nt) {
+  for (int i = t; i < kE * KP; i += nt) {
+    const int j = i % kE, c = i / kE;
+    S.W1T[c][j] = c < K ? p[j * K + c] : 0.0f;
   }
   p += kE * K;
   for (int i = t; i < kE; i += nt) S.b1[i] = p[i];
   p += kE;
-  for (int i = t; i < kE * kE; i += nt) S.W2[i / kE][i % kE] = p[i];
+  for (int i = t; i < kE * kE; i += nt) S.W2T[i % kE][i / kE] = p[i];
   p += kE * kE;
   for (int i = t; i < kE; i += nt) S.b2[i] = p[i];
-  p += kE;
-  for (int i = t; i < 8 * kE; i += nt) S.W3[i / kE][i % kE] = p[i];
-  p += 8 * kE;
+  p += kE + 8 * kE;
   for (int i = t; i < 8; i += nt) S.b3[i] = p[i];
 }
 
-__device__ __forceinline__ void load_row(const float* __restrict__ attrs, int K, int64_t i, float k[kKMax]) {
+template <int KP>
+__device__ __forceinline__ void load_row(const float* __restrict__ attrs, int K, int64_t i, float k[KP]) {
 #pragma unroll
-  for (int c = 0; c < kKMax; ++c) k[c] = c < K ? attrs[i * K + c] : 0.0f;
+  for (int c = 0; c < KP; ++c) k[c] = c < K ? attrs[i * K + c] : 0.0f;
 }
 
-// h1 = ReLU(W1 k + b1) into registers, h2 = ReLU(W2 h1 + b2) into the
-// caller's shared-memory row; pre-activation signs in masks
-__device__ __forceinline__ void hidden(const EncW& S, const float k[kKMax], float h1[kE], float* h2row,
-                                       uint32_t& m1, uint32_t& m2) {
-  m1 = m2 = 0;
+// acc[0..U) += w[0..U) x, w in shared memory
+template <int U>
+__device__ __forceinline__ void axpy(float2 (&acc)[U / 2], const float* w, float x) {
+  const float2 xx = make_float2(x, x);
 #pragma unroll
-  for (int j = 0; j < kE; ++j) {
-    float s = S.b1[j];
-#pragma unroll
-    for (int c = 0; c < kKMax; ++c) s = fmaf(S.W1[j][c], k[c], s);
-    h1[j] = fmaxf(s, 0.0f);
-    if (s > 0.0f) m1 |= 1u << j;
-  }
-#pragma unroll 1
-  for (int j = 0; j < kE; ++j) {
-    float s = S.b2[j];
-#pragma unroll
-    for (int c = 0; c < kE; ++c) s = fmaf(S.W2[j][c], h1[c], s);
-    h2row[j] = fmaxf(s, 0.0f);
-    if (s > 0.0f) m2 |= 1u << j;
+  for (int u = 0; u < U; u += 4) {
+    const float4 v = *reinterpret_cast<const float4*>(w + u);
+    acc[u / 2] = ptx::fma2(make_float2(v.x, v.y), xx, acc[u / 2]);
+    acc[u / 2 + 1] = ptx::fma2(make_float2(v.z, v.w), xx, acc[u / 2 + 1]);
   }
 }
+template <int U>
+__device__ __forceinline__ void start(float2 (&acc)[U / 2], const float* b) {
+#pragma unroll
+  for (int u = 0; u < U; u += 2) acc[u / 2] = *reinterpret_cast<const float2*>(b + u);
+}
+__device__ __forceinline__ uint32_t relu(float2 (&a)[kE / 2]) {
+  uint32_t m = 0;
+#pragma unroll
+  for (int u = 0; u < kE / 2; ++u) {
+    if (a[u].x > 0.0f) m |= 1u << (2 * u);
+    if (a[u].y > 0.0f) m |= 2u << (2 * u);
+    a[u] = make_float2(fmaxf(a[u].x, 0.0f), fmaxf(a[u].y, 0.0f));
+  }
+  return m;
+}
+__device__ __forceinline__ float unit(const float2 (&a)[kE / 2], int j) { return j & 1 ? a[j / 2].y : a[j / 2].x; }
 
-constexpr int kFwdThreads = 256;
+// h1 = ReLU(W1 k + b1), h2 = ReLU(W2 h1 + b2); pre-activation signs in masks
+template <int KP>
+__device__ __forceinline__ void hidden(const EncW<KP>& S, const float k[KP], float2 (&h1)[kE / 2],
+                                       float2 (&h2)[kE / 2], uint32_t& m1, uint32_t& m2) {
+  start<kE>(h1, S.b1);
+#pragma unroll
+  for (int c = 0; c < KP; ++c) axpy<kE>(h1, S.W1T[c], k[c]);
+  m1 = relu(h1);
+  start<kE>(h2, S.b2);
+#pragma unroll
+  for (int c = 0; c < kE; ++c) axpy<kE>(h2, S.W2T[c], unit(h1, c));
+  m2 = relu(h2);
+}
 
-__global__ void __launch_bounds__(kFwdThreads) encode_kernel(const float* __restrict__ W, int K,
+constexpr int kFwdThreads = 128;
+constexpr int kFwdCtas = 2;  // per SM
+
+template <int KP>
+__global__ void __launch_bounds__(kFwdThreads, kFwdCtas) encode_kernel(const float* __restrict__ W, int K,
                                                              const float* __restrict__ attrs, int64_t n,
                                                              float* __restrict__ z_out) {
-  __shared__ __align__(16) EncW S;
-  __shared__ float H2[kFwdThreads][kE + 1];  // odd stride: a thread's row, conflict-free
+  __shared__ __align__(16) EncW<KP> S;
+  __shared__ __align__(16) float W3T[kE][8];
   load_encoder(S, W, K, threadIdx.x, blockDim.x);
+  const float* W3 = W + kE * (K + 1) + kE * (kE + 1);
+  for (int i = threadIdx.x; i < 8 * kE; i += blockDim.x) W3T[i % kE][i / kE] = W3[i];
   __syncthreads();
-  float* h2 = H2[threadIdx.x];
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    float k[kKMax], h1[kE];
+    float k[KP];
+    float2 h1[kE / 2], h2[kE / 2], z[4];
     uint32_t m1, m2;
-    load_row(attrs, K, i, k);
+    load_row<KP>(attrs, K, i, k);
     hidden(S, k, h1, h2, m1, m2);
-    float z[8];
+    start<8>(z, S.b3);
 #pragma unroll
-    for (int c = 0; c < 8; ++c) z[c] = S.b3[c];
-#pragma unroll 4
-    for (int j = 0; j < kE; ++j) {
-      const float h = h2[j];
-#pragma unroll
-      for (int c = 0; c < 8; ++c) z[c] = fmaf(S.W3[c][j], h, z[c]);
-    }
+    for (int j = 0; j < kE; ++j) axpy<8>(z, W3T[j], unit(h2, j));
     float4* o = reinterpret_cast<float4*>(z_out + i * 8);
-    o[0] = make_float4(z[0], z[1], z[2], z[3]);
-    o[1] = make_float4(z[4], z[5], z[6], z[7]);
+    o[0] = make_float4(z[0].x, z[0].y, z[1].x, z[1].y);
+    o[1] = make_float4(z[2].x, z[2].y, z[3].x, z[3].y);
   }
 }
 
+template <int KP>
 struct EncBwdSmem {
-  EncW w;
-  static constexpr int S = kE + 4;  // padded row stride
-  float X[kTile][kKMax];            // inputs k
-  float H1[kTile][S], D1[kTile][S];
-  float H2[kTile][S], D2[kTile][S];
-  float DZ[kTile][8];
+  EncW<KP> w;
+  float W2[kE][kE], W3[8][kE];
+  // per warp, of its 32 rows (odd multiples of 16 bytes apart: no bank
+  // conflicts): a layer's deltas, its inputs, dL/dz
+  struct Warp {
+    float D[32][kE + 4], X[32][kE + 4], DZ[32][8];
+  } r[kBwdThreads / 32];
 };
 
-__global__ void __launch_bounds__(kTile) encoder_backward_kernel(const float* __restrict__ W, int K,
+template <int KP>
+__global__ void __launch_bounds__(kBwdThreads, kBwdCtas) encoder_backward_kernel(const float* __restrict__ W, int K,
                                                                  const float* __restrict__ attrs,
                                                                  const float* __restrict__ dz, int64_t n,
                                                                  float* __restrict__ grad) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  EncBwdSmem& S = *reinterpret_cast<EncBwdSmem*>(smem_raw);
-  const int t = threadIdx.x;
-  load_encoder(S.w, W, K, t, kTile);
-  // phase-B ownership: 4x4 blocks of dW3 [8][32] (16), dW2 [32][32] (64),
-  // dW1 [32][16] (32, columns beyond K dropped at the flush)
-  int role = -1, r0 = 0, c0 = 0;
-  const float* dp = nullptr;
-  const float* ap = nullptr;
-  int dstride = 0, astride = 0;
+  using Sm = EncBwdSmem<KP>;
+  Sm& S = *reinterpret_cast<Sm*>(smem_raw);
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  load_encoder(S.w, W, K, t, kBwdThreads);
   {
-    int b = t;
-    if (b < 16) {
-      role = 0; r0 = 4 * (b >> 3); c0 = 4 * (b & 7);
-      dp = &S.DZ[0][r0]; dstride = 8; ap = &S.H2[0][c0]; astride = EncBwdSmem::S;
-    } else if ((b -= 16) < 64) {
-      role = 1; r0 = 4 * (b >> 3); c0 = 4 * (b & 7);
-      dp = &S.D2[0][r0]; dstride = EncBwdSmem::S; ap = &S.H1[0][c0]; astride = EncBwdSmem::S;
-    } else if ((b -= 64) < 32) {
-      role = 2; r0 = 4 * (b >> 2); c0 = 4 * (b & 3);
-      dp = &S.D1[0][r0]; dstride = EncBwdSmem::S; ap = &S.X[0][c0]; astride = kKMax;
-    }
+    const float* W2 = W + kE * (K + 1);
+    for (int i = t; i < kE * kE; i += kBwdThreads) S.W2[i / kE][i % kE] = W2[i];
+    for (int i = t; i < 8 * kE; i += kBwdThreads) S.W3[i / kE][i % kE] = W2[kE * (kE + 1) + i];
   }
-  float acc[16], accb[4];
-#pragma unroll
-  for (int e = 0; e < 16; ++e) acc[e] = 0.0f;
-#pragma unroll
-  for (int e = 0; e < 4; ++e) accb[e] = 0.0f;
   __syncthreads();
-  const int64_t ntiles = (n + kTile - 1) / kTile;
-  for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    const int64_t start = tile * kTile;
-    const int count = (int)((n - start) < kTile ? (n - start) : kTile);
-    // ---- phase A: thread = row -----------------------------------------------
-    if (t < count) {
-      const int64_t i = start + t;
-      float k[kKMax], h1[kE];
-      uint32_t m1, m2;
-      load_row(attrs, K, i, k);
-      hidden(S.w, k, h1, S.H2[t], m1, m2);
-      float g[8];
-      {
-        const float4 a = reinterpret_cast<const float4*>(dz + i * 8)[0];
-        const float4 b = reinterpret_cast<const float4*>(dz + i * 8)[1];
-        g[0] = a.x; g[1] = a.y; g[2] = a.z; g[3] = a.w; g[4] = b.x; g[5] = b.y; g[6] = b.z; g[7] = b.w;
-      }
+  typename Sm::Warp& R = S.r[warp];
+  // this lane's gradients: dW3 rows 2r.., columns 4c..; dW2 rows 8r..,
+  // columns 4c..; dW1 row `lane`; biases of unit `lane` (b3: lane % 8)
+  const int r = lane >> 3, c = lane & 7;
+  float2 acc3[4], acc2[16], acc1[KP / 2];
+  float ab1 = 0.0f, ab2 = 0.0f, ab3 = 0.0f;
 #pragma unroll
-      for (int c4 = 0; c4 < kKMax / 4; ++c4)
-        reinterpret_cast<float4*>(&S.X[t][0])[c4] = make_float4(k[4 * c4], k[4 * c4 + 1], k[4 * c4 + 2], k[4 * c4 + 3]);
+  for (int e = 0; e < 4; ++e) acc3[e] = make_float2(0.0f, 0.0f);
 #pragma unroll
-      for (int j4 = 0; j4 < kE / 4; ++j4)
-        reinterpret_cast<float4*>(&S.H1[t][0])[j4] = make_float4(h1[4 * j4], h1[4 * j4 + 1], h1[4 * j4 + 2], h1[4 * j4 + 3]);
-      reinterpret_cast<float4*>(&S.DZ[t][0])[0] = make_float4(g[0], g[1], g[2], g[3]);
-      reinterpret_cast<float4*>(&S.DZ[t][0])[1] = make_float4(g[4], g[5], g[6], g[7]);
-      // d2 = (W3^T dz) where layer 2 is active
-#pragma unroll 1
-      for (int j = 0; j < kE; ++j) {
-        float s = 0.0f;
+  for (int e = 0; e < 16; ++e) acc2[e] = make_float2(0.0f, 0.0f);
 #pragma unroll
-        for (int c = 0; c < 8; ++c) s = fmaf(S.w.W3[c][j], g[c], s);
-        S.D2[t][j] = ((m2 >> j) & 1u) ? s : 0.0f;
-      }
-      // d1 = (W2^T d2) where layer 1 is active (accumulated in h1's registers)
+  for (int e = 0; e < KP / 2; ++e) acc1[e] = make_float2(0.0f, 0.0f);
+  auto store = [&](float* row, const float2 (&v)[kE / 2]) {
 #pragma unroll
-      for (int c = 0; c < kE; ++c) h1[c] = 0.0f;
-#pragma unroll 2
-      for (int j = 0; j < kE; ++j) {
-        const float d = S.D2[t][j];
+    for (int j = 0; j < kE / 2; j += 2)
+      reinterpret_cast<float4*>(row)[j / 2] = make_float4(v[j].x, v[j].y, v[j + 1].x, v[j + 1].y);
+  };
+  auto keep = [&](float2 (&v)[kE / 2], uint32_t m) {
 #pragma unroll
-        for (int c = 0; c < kE; ++c) h1[c] = fmaf(S.w.W2[j][c], d, h1[c]);
-      }
-#pragma unroll
-      for (int j4 = 0; j4 < kE / 4; ++j4) {
-        float v[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) v[e] = ((m1 >> (4 * j4 + e)) & 1u) ? h1[4 * j4 + e] : 0.0f;
-        reinterpret_cast<float4*>(&S.D1[t][0])[j4] = make_float4(v[0], v[1], v[2], v[3]);
-      }
+    for (int u = 0; u < kE / 2; ++u)
+      v[u] = make_float2((m >> (2 * u)) & 1u ? v[u].x : 0.0f, (m >> (2 * u + 1)) & 1u ? v[u].y : 0.0f);
+  };
+  // acc[2 rr .. 2 rr + 1] += d a
+  auto outer = [&](float2* acc, int rr, float d, const float4& a) {
+    const float2 dd = make_float2(d, d);
+    acc[2 * rr] = ptx::fma2(dd, make_float2(a.x, a.y), acc[2 * rr]);
+    acc[2 * rr + 1] = ptx::fma2(dd, make_float2(a.z, a.w), acc[2 * rr + 1]);
+  };
+  const int64_t ntiles = (n + 31) / 32;
+  for (int64_t tile = blockIdx.x + (int64_t)warp * gridDim.x; tile < ntiles;
+       tile += (int64_t)gridDim.x * (kBwdThreads / 32)) {
+    const int64_t start_row = tile * 32;
+    const int count = (int)((n - start_row) < 32 ? (n - start_row) : 32);
+    const int64_t i = start_row + (lane < count ? lane : 0);
+    // ---- lane = row: forward -------------------------------------------------
+    float k[KP];
+    float2 h1[kE / 2], h2[kE / 2];
+    uint32_t m1, m2;
+    load_row<KP>(attrs, K, i, k);
+    const float4 ga = reinterpret_cast<const float4*>(dz + i * 8)[0];
+    const float4 gb = reinterpret_cast<const float4*>(dz + i * 8)[1];
+    hidden(S.w, k, h1, h2, m1, m2);
+    store(R.X[lane], h2);
+    reinterpret_cast<float4*>(R.DZ[lane])[0] = ga;
+    reinterpret_cast<float4*>(R.DZ[lane])[1] = gb;
+    __syncwarp();
+    // ---- lane = block of dW3 -------------------------------------------------
+#pragma unroll 4
+    for (int q = 0; q < count; ++q) {
+      const float2 d = *reinterpret_cast<const float2*>(&R.DZ[q][2 * r]);
+      const float4 a = *reinterpret_cast<const float4*>(&R.X[q][4 * c]);
+      outer(acc3, 0, d.x, a);
+      outer(acc3, 1, d.y, a);
+      ab3 += R.DZ[q][c];
     }
-    __syncthreads();
-    // ---- phase B: thread = 4x4 gradient block ---------------------------------
-    if (role >= 0) {
-#pragma unroll 2
-      for (int qq = 0; qq < count; ++qq) {
-        const float4 d = *reinterpret_cast<const float4*>(dp + qq * dstride);
-        const float4 a = *reinterpret_cast<const float4*>(ap + qq * astride);
-        const float dv[4] = {d.x, d.y, d.z, d.w};
-        const float av[4] = {a.x, a.y, a.z, a.w};
+    // ---- lane = row: d2 = (W3^T dz) where layer 2 is active -------------------
+    {
+      const float g[8] = {ga.x, ga.y, ga.z, ga.w, gb.x, gb.y, gb.z, gb.w};
 #pragma unroll
-        for (int rr = 0; rr < 4; ++rr) {
+      for (int u = 0; u < kE / 2; ++u) h2[u] = make_float2(0.0f, 0.0f);
 #pragma unroll
-          for (int cc = 0; cc < 4; ++cc) acc[4 * rr + cc] = fmaf(dv[rr], av[cc], acc[4 * rr + cc]);
-          accb[rr] += dv[rr];
-        }
-      }
+      for (int e = 0; e < 8; ++e) axpy<kE>(h2, S.W3[e], g[e]);
+      keep(h2, m2);
     }
-    __syncthreads();
-  }
-  if (role < 0) return;
-  // (weight offset, row stride, valid rows, valid columns, bias offset)
-  const int oW1 = 0, ob1 = kE * K, oW2 = ob1 + kE, ob2 = oW2 + kE * kE, oW3 = ob2 + kE, ob3 = oW3 + 8 * kE;
-  int wo = 0, ws = 0, nc = 0, bo = 0;
-  switch (role) {
-    case 0: wo = oW3; ws = kE; nc = kE; bo = ob3; break;
-    case 1: wo = oW2; ws = kE; nc = kE; bo = ob2; break;
-    default: wo = oW1; ws = K; nc = K; bo = ob1; break;
-  }
+    __syncwarp();
+    store(R.D[lane], h2);
+    store(R.X[lane], h1);
+    __syncwarp();
+    // ---- lane = block of dW2 -------------------------------------------------
+#pragma unroll 2
+    for (int q = 0; q < count; ++q) {
+      const float4 d0 = *reinterpret_cast<const float4*>(&R.D[q][8 * r]);
+      const float4 d1 = *reinterpret_cast<const float4*>(&R.D[q][8 * r + 4]);
+      const float4 a = *reinterpret_cast<const float4*>(&R.X[q][4 * c]);
+      outer(acc2, 0, d0.x, a); outer(acc2, 1, d0.y, a); outer(acc2, 2, d0.z, a); outer(acc2, 3, d0.w, a);
+      outer(acc2, 4, d1.x, a); outer(acc2, 5, d1.y, a); outer(acc2, 6, d1.z, a); outer(acc2, 7, d1.w, a);
+      ab2 += R.D[q][lane];
+    }
+    // ---- lane = row: d1 = (W2^T d2) where layer 1 is active -------------------
 #pragma unroll
-  for (int rr = 0; rr < 4; ++rr) {
-    const int row = r0 + rr;
+    for (int u = 0; u < kE / 2; ++u) h1[u] = make_float2(0.0f, 0.0f);
 #pragma unroll
-    for (int cc = 0; cc < 4; ++cc)
-      if (c0 + cc < nc) atomicAdd(&grad[wo + row * ws + c0 + cc], acc[4 * rr + cc]);
-    if (c0 == 0) atomicAdd(&grad[bo + row], accb[rr]);
+    for (int j = 0; j < kE; ++j) axpy<kE>(h1, S.W2[j], unit(h2, j));
+    keep(h1, m1);
+    __syncwarp();
+    store(R.D[lane], h1);
+#pragma unroll
+    for (int e = 0; e < KP / 4; ++e)
+      reinterpret_cast<float4*>(R.X[lane])[e] = make_float4(k[4 * e], k[4 * e + 1], k[4 * e + 2], k[4 * e + 3]);
+    __syncwarp();
+    // ---- lane = row of dW1 ---------------------------------------------------
+#pragma unroll 4
+    for (int q = 0; q < count; ++q) {
+      const float d = R.D[q][lane];
+#pragma unroll
+      for (int e = 0; e < KP / 4; ++e) outer(acc1, e, d, *reinterpret_cast<const float4*>(&R.X[q][4 * e]));
+      ab1 += d;
+    }
+    __syncwarp();
   }
+  // ---- the warps' sums meet in shared memory: one atomic per parameter and CTA
+  const int ob1 = kE * K, oW2 = ob1 + kE, ob2 = oW2 + kE * kE, oW3 = ob2 + kE, ob3 = oW3 + 8 * kE, np = ob3 + 8;
+  static_assert((kE * (KP + 1) + kE * (kE + 1) + 8 * (kE + 1)) * 4 <= (int)sizeof(typename Sm::Warp), "");
+  float* o = reinterpret_cast<float*>(&R);
+#pragma unroll
+  for (int e = 0; e < KP; ++e)
+    if (e < K) o[lane * K + e] = e & 1 ? acc1[e / 2].y : acc1[e / 2].x;
+  o[ob1 + lane] = ab1;
+  o[ob2 + lane] = ab2;
+  if (lane < 8) o[ob3 + lane] = ab3;
+#pragma unroll
+  for (int rr = 0; rr < 8; ++rr)
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      o[oW2 + (8 * r + rr) * kE + 4 * c + e] = e & 1 ? acc2[2 * rr + e / 2].y : acc2[2 * rr + e / 2].x;
+#pragma unroll
+  for (int rr = 0; rr < 2; ++rr)
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      o[oW3 + (2 * r + rr) * kE + 4 * c + e] = e & 1 ? acc3[2 * rr + e / 2].y : acc3[2 * rr + e / 2].x;
+  __syncthreads();
+  for (int i = t; i < np; i += kBwdThreads) {
+    float v = 0.0f;
+#pragma unroll
+    for (int w = 0; w < kBwdThreads / 32; ++w) v += reinterpret_cast<const float*>(&S.r[w])[i];
+    atomicAdd(&grad[i], v);
+  }
+}
+
+// the kernels for K inputs padded to 4, 8, 12 or 16 (padding to 16 always
+// would be three quarters of the first layer's work for four inputs)
+template <class F>
+void by_inputs(int K, F&& f) {
+  if (K <= 4) f(std::integral_constant<int, 4>());
+  else if (K <= 8) f(std::integral_constant<int, 8>());
+  else if (K <= 12) f(std::integral_constant<int, 12>());
+  else f(std::integral_constant<int, 16>());
 }
 
 }  // namespace
@@ -243,9 +308,11 @@ int launch_encode(const float* W, int K, const float* attrs, int64_t n, float* z
   if (n == 0) return 0;
   if (K < 1 || K > kKMax) return (int)cudaErrorInvalidValue;
   int64_t blocks = (n + kFwdThreads - 1) / kFwdThreads;
-  const int64_t cap = (int64_t)num_sms * 8;
+  const int64_t cap = (int64_t)num_sms * kFwdCtas;
   if (blocks > cap) blocks = cap;
-  encode_kernel<<<(int)blocks, kFwdThreads, 0, (cudaStream_t)stream>>>(W, K, attrs, n, z_out);
+  by_inputs(K, [&](auto kp) {
+    encode_kernel<kp><<<(int)blocks, kFwdThreads, 0, (cudaStream_t)stream>>>(W, K, attrs, n, z_out);
+  });
   return (int)cudaGetLastError();
 }
 
@@ -253,15 +320,16 @@ int launch_encoder_backward(const float* W, int K, const float* attrs, const flo
                             int num_sms, void* stream) {
   if (n == 0) return 0;
   if (K < 1 || K > kKMax) return (int)cudaErrorInvalidValue;
-  const int smem = (int)sizeof(EncBwdSmem);
-  static std::atomic<uint64_t> attr_done{0};
-  once_per_device(attr_done, [&] {
-    cudaFuncSetAttribute(encoder_backward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  });
-  const int64_t tiles = (n + kTile - 1) / kTile;
-  int64_t grid = (int64_t)num_sms * 2;
+  const int64_t tiles = (n + 31) / 32;  // one per warp
+  int64_t grid = (int64_t)num_sms * kBwdCtas;
   if (grid > tiles) grid = tiles;
-  encoder_backward_kernel<<<(int)grid, kTile, smem, (cudaStream_t)stream>>>(W, K, attrs, dz, n, grad);
+  by_inputs(K, [&](auto kp) {
+    auto k = encoder_backward_kernel<kp>;
+    const int smem = (int)sizeof(EncBwdSmem<kp>);
+    static std::atomic<uint64_t> attr_done{0};
+    once_per_device(attr_done, [&] { cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem); });
+    k<<<(int)grid, kBwdThreads, smem, (cudaStream_t)stream>>>(W, K, attrs, dz, n, grad);
+  });
   return (int)cudaGetLastError();
 }
 
