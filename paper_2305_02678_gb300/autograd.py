@@ -15,6 +15,7 @@ the optimiser update.
 from __future__ import annotations
 
 import torch
+import torch.autograd.forward_ad as fwd_ad
 
 from . import binding as B
 
@@ -103,9 +104,61 @@ class NeuralMaterial(torch.nn.Module):
                                         B.NAM_OUT_COSINE if cosine else 0)
 
 
+def _log_l1_ops(rgb, target):
+    d = torch.log1p(torch.relu(rgb)) - torch.log1p(target)
+    return (d.abs() + 0.01 * torch.relu(-rgb)).mean()
+
+
+class _LogL1(torch.autograd.Function):
+    """_log_l1_ops of contiguous FP32 CUDA tensors in one pass: the forward
+    also writes the derivative for a unit gradient.  A derivative that is
+    itself to be differentiated is taken through the tensor operations."""
+
+    @staticmethod
+    def forward(ctx, rgb, target):
+        loss = torch.empty((), dtype=torch.float32, device=rgb.device)
+        work = torch.empty(304, dtype=torch.float64, device=rgb.device)
+        unit = torch.empty_like(rgb) if ctx.needs_input_grad[0] else None
+        B._check(B.lib().nam_internal_log_l1(rgb.data_ptr(), target.data_ptr(), rgb.numel(), B.ptr(unit),
+                                             loss.data_ptr(), work.data_ptr(), B.current_stream(rgb.device)),
+                 "log_l1_loss")
+        if unit is not None:
+            ctx.save_for_backward(unit)
+            ctx.inputs = rgb, target, rgb._version, target._version
+        return loss
+
+    @staticmethod
+    def backward(ctx, grad):
+        if torch.is_grad_enabled():
+            rgb, target, *versions = ctx.inputs
+            if [rgb._version, target._version] != versions:
+                raise RuntimeError("log_l1_loss: an input needed for a second derivative was modified in place")
+            loss = _log_l1_ops(rgb, target)
+            return torch.autograd.grad(loss, rgb, grad, create_graph=True)[0], None
+        unit, = ctx.saved_tensors
+        return unit * grad, None
+
+
+def _one_pass(rgb, target):
+    """Whether _LogL1 takes these inputs: plain contiguous FP32 CUDA tensors
+    outside of anything that has to see the single tensor operations (vmap
+    and the other function transforms, forward-mode duals, tracing, modes)."""
+    return (type(rgb) is torch.Tensor and type(target) in (torch.Tensor, torch.nn.Parameter)
+            and rgb.is_cuda and rgb.dtype == torch.float32 and target.dtype == torch.float32
+            and rgb.device == target.device and rgb.shape == target.shape and rgb.numel() > 0
+            and not target.requires_grad and rgb.is_contiguous() and target.is_contiguous()
+            and not (rgb.is_neg() or target.is_neg())
+            and rgb.device.index == torch.cuda.current_device()
+            and not torch.jit.is_tracing() and not torch.compiler.is_compiling()
+            and not torch._C._are_functorch_transforms_active()
+            and torch._C._len_torch_dispatch_stack() == 0 and torch._C._len_torch_function_stack() == 0
+            and fwd_ad.unpack_dual(rgb).tangent is None and fwd_ad.unpack_dual(target).tangent is None)
+
+
 def log_l1_loss(rgb, target):
     """Mean over the batch and channels of |log(1 + max(g, 0)) - log(1 + y)|
     plus 0.01 * max(-g, 0): the paper's L1 loss in log space (Sec. 5), with a
     small linear penalty so that negative outputs still receive a gradient."""
-    d = torch.log1p(torch.relu(rgb)) - torch.log1p(target)
-    return (d.abs() + 0.01 * torch.relu(-rgb)).mean()
+    if _one_pass(rgb, target):
+        return _LogL1.apply(rgb, target)
+    return _log_l1_ops(rgb, target)
