@@ -101,13 +101,16 @@ typedef struct nam_material_s* nam_material;
 
 enum { NAM_LATENT_F32 = 0, NAM_LATENT_F16 = 1 };
 /* Arithmetic of the MLPs.
- * F32: plain FP32 FMA on CUDA cores, one query per thread.
+ * F32: FP32 results; a trainable material's as plain FP32 FMA on CUDA cores,
+ * one query per thread; otherwise the decoder's wide layers on tensor cores,
+ * with operands split into three bf16 terms (FP32's range and accuracy: the
+ * error against exact arithmetic is no larger than the per-thread form's).
  * F16: parameters quantised to binary16 at creation (post-training
  * quantisation, Sec. 5.2), MLP layers on tensor cores with FP16 operands and
  * FP32 accumulation.  The operands the result is most sensitive to (the
- * latent, the transformed directions, the frame MLP's hidden layer, the last
- * hidden layer; every hidden layer for hidden width < 64) enter as two FP16
- * halves, so the error against FP16 weights with exact activations stays
+ * latent, the transformed directions, the frame MLP's hidden layer; every
+ * hidden layer for hidden width < 64) enter as two FP16 halves, and the
+ * output layer reads the last hidden layer in FP32, so the error against FP16 weights with exact activations stays
  * within 2e-3.
  * FP8 (beyond the paper): as F16, except that the hidden -> hidden decoder
  * layers have E4M3 weights with a power-of-two per-layer scale (the smallest

@@ -1,7 +1,8 @@
 // Plain FP32 evaluation: one query per thread, MLP weights staged in shared
 // memory, FP32 FMA on CUDA cores.  This is the "divergent" per-thread form
-// of the decoder (Sec. 7.1: whole network per thread, unrolled FMAs) and the
-// FP32 reference point the reduced-precision tensor-core path is compared to.
+// of the decoder (Sec. 7.1: whole network per thread, unrolled FMAs), for
+// materials whose masters may change between launches (others:
+// eval_f32_tc.cu) and for the activation range of nam_fp8_calibrate.
 // With the albedo head the kernel also writes the albedo triplet.
 #include <cuda_runtime.h>
 

@@ -5,7 +5,8 @@
 // backward, each of a few microseconds of device time behind as much or more
 // of host time; here it is two launches (the second adds up the blocks' sums,
 // in a fixed order), and a scaling of the derivative when the gradient comes
-// back.  150,000 values: the 22 launches took 72 us of device time, these 7.
+// back.  A training iteration of 50,000 queries through autograd: 370 us, with
+// the tensor operations 636.
 #include <cuda_runtime.h>
 
 #include "nam_ctx.h"
