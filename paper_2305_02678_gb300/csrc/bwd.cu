@@ -34,10 +34,10 @@
 // What bounds it: the latency of the tile's chain of stages (16 warps a CTA,
 // which shared memory and registers allow no more of; the forward on the FMA
 // pipes is a fifth of a tile's time, the fetch and the scatter a sixth each).
-// H = 64 with the fused loss, 262,144 queries, 1024^2 pyramid: 290 us, against
+// H = 64 with the fused loss, 262,144 queries, 1024^2 pyramid: 281 us, against
 // 378 us with every product on the FMA pipes; 131,072 queries with the latents
-// given: 133 us (163).  Smaller batches and decoders, against that kernel:
-// H = 64, 10,000 queries 38 us (44); H = 16, 262,144 queries 187 us (207).
+// given: 131 us (163).  Smaller batches and decoders, against that kernel:
+// H = 64, 10,000 queries 37 us (44); H = 16, 262,144 queries 188 us (207).
 // Training step variant (LOSS): the decoder blocks also finish the forward
 // (y = Wo h2 + bo, summed over the half-warp), evaluate the log-space L1
 // loss against the target and start the backward from its gradient, so a
@@ -67,7 +67,7 @@ template <int H, bool ALB = false>
 struct BwdSmem {
   static constexpr int NO = ALB ? 6 : 3;  // decoder outputs
   static constexpr int DW = ALB ? 8 : 4;  // DY row length
-  static constexpr int S = H + 4;  // padded row stride of W2 and H1: rows l + 16 jj of a half-warp hit distinct banks
+  static constexpr int S = H + 4;  // padded row stride of H1
   // operand terms: A holds first D2 (H / 8 blocks), then D1, DHF (2 blocks)
   // and DR (1); B holds H1, X (2 blocks, with the 1) and HF (2).  An MMA's A
   // has 128 rows, a group's 64 (or 24) of them in its half of the TMEM
@@ -76,9 +76,14 @@ struct BwdSmem {
   static constexpr int TA = (H / 8 + 3) * kBlk, TB = (H / 8 + 4) * kBlk;
   // parameters
   float fW1[16 * 8], fb1[16], fW2[6 * 16], fb2[8];
-  float W1[H][20];   // W1[j][0..13], zero padding
+  // W1 (14 inputs, zero padding) and W2 of the forward's packed FMAs: row 16 p
+  // + l holds (w[l + 32 p][k], w[l + 32 p + 16][k]) for every k, or for H = 16
+  // w[l][k]; 16 bytes of padding: the rows of a half-warp hit distinct banks
+  static constexpr int P = H >= 32 ? 2 : 1;
+  static constexpr int S1 = 16 * P + 4, S2 = H * P + 4;
+  float W1[H / P][S1];
   float b1[H];
-  float W2[H][S];    // W2[j][k]
+  float W2[H / P][S2];
   float b2[H];
   float Wo[NO * H], bo[8];
   float lred[16];       // per-warp loss partials
@@ -224,6 +229,38 @@ __device__ __forceinline__ void quad_filter(const QuadTaps& T, float z[8]) {
   quad_gather(acc, z);
 }
 
+// a[qq][jj] += w[unit jj][4 m ..] . x[qq], in the order of dot4.  P = 2: units
+// jj and jj + 1 side by side in packed FMAs (half the FMA instructions, and
+// moves that double x; the kernel 290 -> 281 us).  w: this lane's first row, the
+// next units' 16 rows of W floats on.
+template <int JB, int P, int W>
+__device__ __forceinline__ void fma_block(float (&a)[4][JB], const float* w, const float4 (&x)[4], int m) {
+  if constexpr (P == 2) {
+#pragma unroll
+    for (int jj = 0; jj < JB; jj += 2) {
+      const float4 w0 = reinterpret_cast<const float4*>(w + 8 * jj * W)[2 * m];
+      const float4 w1 = reinterpret_cast<const float4*>(w + 8 * jj * W)[2 * m + 1];
+#pragma unroll
+      for (int qq = 0; qq < 4; ++qq) {
+        float2 s = make_float2(a[qq][jj], a[qq][jj + 1]);
+        s = ptx::fma2(make_float2(w0.x, w0.y), make_float2(x[qq].x, x[qq].x), s);
+        s = ptx::fma2(make_float2(w0.z, w0.w), make_float2(x[qq].y, x[qq].y), s);
+        s = ptx::fma2(make_float2(w1.x, w1.y), make_float2(x[qq].z, x[qq].z), s);
+        s = ptx::fma2(make_float2(w1.z, w1.w), make_float2(x[qq].w, x[qq].w), s);
+        a[qq][jj] = s.x;
+        a[qq][jj + 1] = s.y;
+      }
+    }
+  } else {
+#pragma unroll
+    for (int jj = 0; jj < JB; ++jj) {
+      const float4 v = reinterpret_cast<const float4*>(w + 16 * jj * W)[m];
+#pragma unroll
+      for (int qq = 0; qq < 4; ++qq) a[qq][jj] = dot4(v, x[qq], a[qq][jj]);
+    }
+  }
+}
+
 // One query's fields, spread over its quad: lane p holds (u, v, lod, xi)[p],
 // wi[p], wo[p], and target or output gradient [p] and [3 + p] (p < 3).
 struct QuadFields {
@@ -255,7 +292,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const Backward
   extern __shared__ __align__(128) unsigned char smem_raw[];
   using Sm = BwdSmem<H, ALB>;
   Sm& S = *reinterpret_cast<Sm*>(smem_raw);
-  constexpr int NO = Sm::NO, DW = Sm::DW, TA = Sm::TA, TB = Sm::TB;
+  constexpr int NO = Sm::NO, DW = Sm::DW, TA = Sm::TA, TB = Sm::TB, P = Sm::P;
   constexpr int JB = H / 16;  // hidden units per lane in the decoder blocks
   constexpr int U = H / 4;    // units per lane where a row is shared by four
   constexpr int N2 = H + 16;  // columns of C2
@@ -279,14 +316,16 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const Backward
       if (t < 8) S.fb2[t] = t < 6 ? p[240 + t] : 0.0f;
       p += 246;
     }
-    for (int i = t; i < H * 20; i += kBwdThreads) {
-      const int j = i / 20, k = i % 20;
-      S.W1[j][k] = k < 14 ? p[j * 14 + k] : 0.0f;
+    auto row = [](int j) { return P == 2 ? (j >> 5) * 16 + (j & 15) : j; };
+    auto col = [](int j, int k) { return P == 2 ? 2 * k + ((j >> 4) & 1) : k; };
+    for (int i = t; i < H * 16; i += kBwdThreads) {
+      const int j = i / 16, k = i % 16;
+      S.W1[row(j)][col(j, k)] = k < 14 ? p[j * 14 + k] : 0.0f;
     }
     p += 14 * H;
     for (int i = t; i < H; i += kBwdThreads) S.b1[i] = p[i];
     p += H;
-    for (int i = t; i < H * H; i += kBwdThreads) S.W2[i / H][i % H] = p[i];
+    for (int i = t; i < H * H; i += kBwdThreads) S.W2[row(i / H)][col(i / H, i % H)] = p[i];
     p += H * H;
     for (int i = t; i < H; i += kBwdThreads) S.b2[i] = p[i];
     p += H;
@@ -541,12 +580,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const Backward
         float4 xv[4];
 #pragma unroll
         for (int qq = 0; qq < 4; ++qq) xv[qq] = reinterpret_cast<const float4*>(&G.X[qb + qq][0])[c4];
-#pragma unroll
-        for (int jj = 0; jj < JB; ++jj) {
-          const float4 w = reinterpret_cast<const float4*>(&S.W1[hl + 16 * jj][0])[c4];
-#pragma unroll
-          for (int qq = 0; qq < 4; ++qq) a[qq][jj] = dot4(w, xv[qq], a[qq][jj]);
-        }
+        fma_block<JB, P, Sm::S1>(a, &S.W1[hl][0], xv, c4);
       }
 #pragma unroll
       for (int jj = 0; jj < JB; ++jj)
@@ -580,12 +614,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const Backward
         float4 hv[4];
 #pragma unroll
         for (int qq = 0; qq < 4; ++qq) hv[qq] = reinterpret_cast<const float4*>(&H1[qb + qq][0])[m];
-#pragma unroll
-        for (int jj = 0; jj < JB; ++jj) {
-          const float4 w = reinterpret_cast<const float4*>(&S.W2[hl + 16 * jj][0])[m];
-#pragma unroll
-          for (int qq = 0; qq < 4; ++qq) a[qq][jj] = dot4(w, hv[qq], a[qq][jj]);
-        }
+        fma_block<JB, P, Sm::S2>(a, &S.W2[hl][0], hv, m);
       }
       if (LOSS) {
         // output y = Wo relu(a) + bo of the four queries, summed over the
