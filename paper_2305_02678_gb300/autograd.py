@@ -143,13 +143,13 @@ def _one_pass(rgb, target):
     """Whether _LogL1 takes these inputs: plain contiguous FP32 CUDA tensors
     outside of anything that has to see the single tensor operations (vmap
     and the other function transforms, forward-mode duals, tracing, modes)."""
-    return (type(rgb) is torch.Tensor and type(target) in (torch.Tensor, torch.nn.Parameter)
+    return (not torch.compiler.is_compiling() and not torch.jit.is_tracing()
+            and type(rgb) is torch.Tensor and type(target) in (torch.Tensor, torch.nn.Parameter)
             and rgb.is_cuda and rgb.dtype == torch.float32 and target.dtype == torch.float32
             and rgb.device == target.device and rgb.shape == target.shape and rgb.numel() > 0
             and not target.requires_grad and rgb.is_contiguous() and target.is_contiguous()
             and not (rgb.is_neg() or target.is_neg())
             and rgb.device.index == torch.cuda.current_device()
-            and not torch.jit.is_tracing() and not torch.compiler.is_compiling()
             and not torch._C._are_functorch_transforms_active()
             and torch._C._len_torch_dispatch_stack() == 0 and torch._C._len_torch_function_stack() == 0
             and fwd_ad.unpack_dual(rgb).tangent is None and fwd_ad.unpack_dual(target).tangent is None)
