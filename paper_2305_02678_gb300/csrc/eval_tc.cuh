@@ -1020,12 +1020,17 @@ __global__ void __launch_bounds__((NCH + NF) * 128, 1) eval_f16_kernel(const __g
 // ---------------------------------------------------------------------------
 // One material: five chains (TMEM 5 x (H + 32) <= 480 of 512 columns) and two
 // fetch warpgroups, 896 threads at <= 72 registers (1920x1080, H = 64: 90 us;
-// three fetch warpgroups at 64 registers 96, four chains 97).  Mixed
-// materials, whose fetch also follows the binning permutation: four and
-// three (a material per pixel at 1920x1080: 250 us; 5 + 2 263, 5 + 3 277).
+// three fetch warpgroups at 64 registers 96, four chains 97).  Four and three
+// where the fetch is the longer side: mixed materials, whose fetch also follows
+// the binning permutation (a material per pixel at 1920x1080: 250 us; 5 + 2
+// 263, 5 + 3 277); FP32 texels, two loads and sectors of HBM traffic each
+// (1.5 M queries, 2048^2, H = 16 .. 64: 81 .. 105 us, 5 + 2 95 .. 124; not FP8
+// with three hidden layers, 126 against 120); and H = 16 in FP16, whose chains
+// are short (52 .. 64 us, 5 + 2 60 .. 74; H = 32 with a frame 70 against 66).
 template <int H, int FK, int NH, bool F16P, bool MULTI, bool P8>
 static int launch_f16_one(const LaunchCommon& L, cudaStream_t s) {
-  constexpr int NCH = MULTI ? 4 : 5, NF = MULTI ? 3 : 2;
+  constexpr bool kFetch3 = MULTI || (F16P ? H == 16 && !P8 : !(P8 && NH == 3));
+  constexpr int NCH = kFetch3 ? 4 : 5, NF = kFetch3 ? 3 : 2;
   using S = F16Smem<H, FK, NH, F16P, MULTI, NCH, NF>;
   static_assert(S::BYTES <= 227 * 1024, "shared memory");
   static_assert(NCH * F16Cols<H>::COLS <= 512, "TMEM columns");
