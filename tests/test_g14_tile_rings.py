@@ -21,6 +21,9 @@ def _pieces(mat, dq, n, size):
     (2, 64, 2, (8, 16, 6), 0, np.float16),
     (1, 32, 2, (8, 12), 0, np.float16),
     (1, 16, 2, None, 1, np.float32),
+    (1, 16, 2, (8, 16, 6), 0, np.float16),
+    (1, 64, 2, (8, 16, 6), 0, np.float32),
+    (2, 64, 3, (8, 12), 0, np.float32),
     (0, 64, 2, (8, 16, 6), 0, np.float16),
     (0, 64, 3, (8, 12), 1, np.float32),
     (0, 32, 2, None, 0, np.float32),
