@@ -568,12 +568,14 @@ __global__ void __launch_bounds__((NCH + NF) * 128, 1) eval_f16_kernel(const __g
     ptx::tc_fence_after();
   };
 
-  // the leader gives up its weight slot (the lock is held for a few
-  // instructions only; without it the slot stays taken and waits run out)
+  // the leader gives up its weight slot; the barrier before has every thread of
+  // the warpgroup done with the slot's weights.  An atomic decrement without
+  // the lock: it cannot fail, so no slot stays taken by a warpgroup that has
+  // stopped using it.
   auto release_slot = [&]() {
-    if (my_slot >= 0 && smem_lock(slot_lock, ptx::globaltimer(), L.timeout_ns)) {
-      slot_users[my_slot] = slot_users[my_slot] - 1;
-      smem_unlock(slot_lock);
+    if (my_slot >= 0) {
+      __threadfence_block();
+      atomicSub(const_cast<int*>(slot_users + my_slot), 1);
       my_slot = -1;
     }
   };
@@ -647,7 +649,7 @@ __global__ void __launch_bounds__((NCH + NF) * 128, 1) eval_f16_kernel(const __g
             for (int k = 0; k < S::SLOTS && sl < 0; ++k)
               if (slot_mat[k] == cur.mat) {
                 sl = k;
-                slot_users[k] = slot_users[k] + 1;
+                atomicAdd(const_cast<int*>(slot_users + k), 1);  // (a release takes no lock)
                 gen = slot_loads[k];
               }
             for (int k = 0; k < S::SLOTS && sl < 0; ++k)
@@ -662,7 +664,8 @@ __global__ void __launch_bounds__((NCH + NF) * 128, 1) eval_f16_kernel(const __g
             smem_unlock(slot_lock);
             if (sl >= 0) break;
             __nanosleep(256);
-            ok = smem_lock(slot_lock, t0, L.timeout_ns);
+            // (smem_lock reads the clock only when the lock is taken)
+            ok = ptx::globaltimer() - t0 <= L.timeout_ns && smem_lock(slot_lock, t0, L.timeout_ns);
           }
           if (load) {
             const uint32_t bar = bar_w + 8 * sl;
@@ -991,10 +994,7 @@ __global__ void __launch_bounds__((NCH + NF) * 128, 1) eval_f16_kernel(const __g
   // MMAs and bulk copies still in flight after a wait gave up are waited for
   // with the fixed drain limit, and TMEM is freed only if they all completed.
   // A warpgroup leaving its loop gives up its weight slot.
-  if (MULTI && r == 0 && my_slot >= 0 && smem_lock(slot_lock, ptx::globaltimer(), L.timeout_ns)) {
-    slot_users[my_slot] = slot_users[my_slot] - 1;
-    smem_unlock(slot_lock);
-  }
+  if (MULTI && r == 0 && my_slot >= 0) atomicSub(const_cast<int*>(slot_users + my_slot), 1);
   bool drained = true;
   if (r == 0 && mma_pending) drained &= ptx::mbar_wait(bar0 + 8 * wg, ph_m ^ 1, ptx::kDrainTimeoutNs);
   if (!MULTI && tid == 0 && w_pending) drained &= ptx::mbar_wait(bar_w, 0, ptx::kDrainTimeoutNs);
