@@ -988,13 +988,18 @@ __global__ void __launch_bounds__((NCH + NF) * 128, 1) eval_f16_kernel(const __g
     }
     ptx::tc_fence_before();
   }
+  if constexpr (MULTI) {
+    // every thread is past its last reads of the slot's weights (the output
+    // layer takes them from shared memory) before another chain may load over
+    // them; all threads of a warpgroup leave the loop together
+    ptx::bar_sync(bar_id, 128);
+    if (r == 0) release_slot();
+  }
   }  // chain warpgroups
 
   // ---- teardown -------------------------------------------------------------
   // MMAs and bulk copies still in flight after a wait gave up are waited for
   // with the fixed drain limit, and TMEM is freed only if they all completed.
-  // A warpgroup leaving its loop gives up its weight slot.
-  if (MULTI && r == 0 && my_slot >= 0) atomicSub(const_cast<int*>(slot_users + my_slot), 1);
   bool drained = true;
   if (r == 0 && mma_pending) drained &= ptx::mbar_wait(bar0 + 8 * wg, ph_m ^ 1, ptx::kDrainTimeoutNs);
   if (!MULTI && tid == 0 && w_pending) drained &= ptx::mbar_wait(bar_w, 0, ptx::kDrainTimeoutNs);

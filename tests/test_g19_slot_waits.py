@@ -44,3 +44,27 @@ def test_short_wait_limit_reports_timeout(entry):
         for k, m in enumerate(mats):
             idx = torch.nonzero(ids == k)[:, 0]
             assert torch.equal(out[idx], m.eval({f: t[idx].contiguous() for f, t in dq.items()})), k
+
+
+@pytest.mark.parametrize("tiles", [1, 5, 6, 9])
+def test_last_tiles_of_a_cta_keep_their_weights(gctx, tiles):
+    """CTAs whose chains finish on a few tiles each, of more materials than
+    slots: a chain that is done gives its slot to one that still needs it."""
+    import torch
+    from paper_2305_02678_gb300 import binding as B
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    rng = W.rng_streams(192, 14)
+    mats = _materials(gctx, rng, 6)
+    n = sms * tiles * 128
+    dq = to_device(W.uniform_queries(rng[12], n, 6.0))
+    ids = rng[13].integers(0, 6, sms * tiles)
+    ref = torch.stack([m.eval(dq) for m in mats])
+    want = ref[torch.from_numpy(np.repeat(ids, 128)).cuda(), torch.arange(n, device="cuda")]
+    items = [(128 * k, 128, int(i)) for k, i in enumerate(ids)]  # in tile order: neighbours differ
+    for _ in range(20):
+        out = torch.empty((n, 3), device="cuda")
+        B.nam_eval_multi(gctx.h, [m.h for m in mats], dq, items, out, torch.cuda.current_stream())
+        assert torch.equal(out, want)
+    for m in mats:
+        m.destroy()
+    gctx.check()
