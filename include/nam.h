@@ -464,7 +464,9 @@ nam_status nam_scene_render_paths(nam_ctx* ctx, const nam_scene* scene, const na
  * NULL; a misaligned pointer is refused with NAM_ERR_INVALID_ARG).  Weight
  * gradients are reduced per CTA then added with one atomic per parameter and
  * CTA; pyramid gradients are scattered with atomics (tap weight x dL/dz).
- * ReLU'(0) = 0.  No gradient flows through the degenerate-frame fallbacks. */
+ * ReLU'(0) = 0.  No gradient flows through the degenerate-frame fallbacks.
+ * After a device-side wait that ran out (nam_check_device_error) the buffers
+ * hold a part of the sums. */
 nam_status nam_backward(nam_ctx* ctx, nam_material m, const nam_queries* q, int64_t n,
                         const float* grad_rgb, float* grad_params, float* grad_pyramid,
                         void* stream, uint32_t flags);
@@ -482,7 +484,12 @@ typedef struct {
  * two more apply Adam.  target_rgb is device [n][3]; *loss_out (host)
  * receives L of this step's forward (the call synchronises the stream to
  * read it).  Optimiser moments live in the material; the first call
- * allocates the material's 256-byte loss accumulator. */
+ * allocates the material's 256-byte loss accumulator.
+ * If a device-side wait of the backward runs past wait_timeout_ns, the step is
+ * not applied: masters, moments and pyramid stay as they were and the material's
+ * gradient is cleared.  A call with loss_out then returns NAM_ERR_TIMEOUT and
+ * leaves *loss_out alone; one without reports it through
+ * nam_check_device_error.  So do the other training steps below. */
 nam_status nam_train_step(nam_ctx* ctx, nam_material m, const nam_queries* q, const float* target_rgb,
                           int64_t n, const nam_adam* opt, float* loss_out, void* stream, uint32_t flags);
 

@@ -448,6 +448,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const Backward
   const bool cosine = (A.flags & NAM_OUT_COSINE) != 0;
   uint32_t issued = 0;  // tiles whose MMAs were issued (the same in the whole group)
   bool stop = false;    // a wait ran out
+  int64_t left = ntiles;  // the tile it ran out in
   // the fields of the next tile are loaded a tile ahead (its texels as well
   // would cost more in spilled registers than their latency)
   auto row_of = [&](int64_t tile, bool& valid) -> int64_t {
@@ -766,6 +767,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const Backward
     // every warp has read its H1 rows: A takes D2
     if (ptx::bar_red_or(bid + 4, kBwdGroup, bad)) {
       stop = true;
+      left = tile;
       break;
     }
     // ---- layer-2 delta d2 = (Wo^T dy) where the unit is active ---------------
@@ -875,6 +877,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const Backward
       // (the other half of C1's and CF's barrier)
       if (lw == 5 && ptx::elect()) ptx::mma_commit(bar0 + 24);
       stop = true;
+      left = tile;
       break;
     }
     // ---- quad: frame backward, pyramid scatter --------------------------------
@@ -1076,6 +1079,13 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const Backward
   // ---- flush: one atomic per parameter and coarse texel channel per CTA -------
   if (stop) {
     bad = true;
+    // the encoder's backward reads every row of dz: none is left from before
+    if (A.dz_out)
+      for (; left < ntiles; left += tstep) {
+        bool valid;
+        const int64_t i = row_of(left, valid);
+        if (valid) reinterpret_cast<float2*>(A.dz_out + 8 * i)[p] = make_float2(0.0f, 0.0f);
+      }
   } else if (tile0 < ntiles) {
     bad |= !ptx::mbar_wait(bar0 + 24, ph ^ 1u, A.timeout_ns);
     collect();
@@ -1159,7 +1169,10 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const Backward
 #pragma unroll
   for (int k = 0; k < 4; ++k)
     if (issued > 0) drained &= ptx::mbar_wait(bar0 + 8 * k, (issued - 1) & 1u, ptx::kDrainTimeoutNs);
-  if (bad) record_error(A.err, DEVERR_WAIT_TIMEOUT);
+  if (bad) {
+    record_error(A.err, DEVERR_WAIT_TIMEOUT);
+    if (A.failed) atomicExch(A.failed, 1);
+  }
   if (!drained) record_error(A.err, DEVERR_DRAIN_TIMEOUT);
   ptx::tc_fence_before();
   const bool all_drained = __syncthreads_and(drained ? 1 : 0) != 0;
@@ -1274,6 +1287,7 @@ struct AdamStep {
   float lr, b1, b2, eps, c1, c2;
 };
 
+// (a step whose backward failed only clears the gradient, a part of its sum)
 __device__ __forceinline__ void adam_one(float& p, float& g, float& m, float& v, const AdamStep& a) {
   const float gi = g;
   m = a.b1 * m + (1.0f - a.b1) * gi;
@@ -1283,9 +1297,12 @@ __device__ __forceinline__ void adam_one(float& p, float& g, float& m, float& v,
 }
 
 __global__ void adam_kernel(float* __restrict__ p, float* __restrict__ g, float* __restrict__ m, float* __restrict__ v,
-                            int64_t count, const AdamStep a) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x)
-    adam_one(p[i], g[i], m[i], v[i], a);
+                            int64_t count, const AdamStep a, const int* __restrict__ failed) {
+  const bool skip = failed && *failed;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x) {
+    if (skip) g[i] = 0.0f;
+    else adam_one(p[i], g[i], m[i], v[i], a);
+  }
 }
 
 // 16-byte vector form of the same per-element update, bound by HBM: four
@@ -1293,7 +1310,13 @@ __global__ void adam_kernel(float* __restrict__ p, float* __restrict__ g, float*
 // reached the texel (262,144 queries, training step with a 2048^2 pyramid 557
 // -> 544 us, 1024^2 357 -> 355, 256^2, where all are reached, the same).
 __global__ void adam4_kernel(float4* __restrict__ p, float4* __restrict__ g, float4* __restrict__ m,
-                             float4* __restrict__ v, int64_t count4, const AdamStep a) {
+                             float4* __restrict__ v, int64_t count4, const AdamStep a,
+                             const int* __restrict__ failed) {
+  if (failed && *failed) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count4; i += (int64_t)gridDim.x * blockDim.x)
+      g[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    return;
+  }
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count4; i += (int64_t)gridDim.x * blockDim.x) {
     float4 P = p[i], G = g[i], M = m[i], V = v[i];
     const bool clear = (__float_as_uint(G.x) | __float_as_uint(G.y) | __float_as_uint(G.z) | __float_as_uint(G.w)) != 0;
@@ -1309,7 +1332,7 @@ __global__ void adam4_kernel(float4* __restrict__ p, float4* __restrict__ g, flo
 }
 
 int launch_adam(float* p, const float* g, float* m, float* v, int64_t count, float lr, float b1, float b2, float eps,
-                int step, void* stream) {
+                int step, const int* failed, void* stream) {
   if (count == 0) return 0;
   cudaStream_t s = (cudaStream_t)stream;
   const AdamStep a{lr, b1, b2, eps, 1.0f - powf(b1, (float)step), 1.0f - powf(b2, (float)step)};
@@ -1322,7 +1345,7 @@ int launch_adam(float* p, const float* g, float* m, float* v, int64_t count, flo
       int grid = (int)((count4 + 255) / 256);
       if (grid > 8192) grid = 8192;
       adam4_kernel<<<grid, 256, 0, s>>>(reinterpret_cast<float4*>(p), reinterpret_cast<float4*>(gm),
-                                        reinterpret_cast<float4*>(m), reinterpret_cast<float4*>(v), count4, a);
+                                        reinterpret_cast<float4*>(m), reinterpret_cast<float4*>(v), count4, a, failed);
     }
     head = 4 * count4;
   }
@@ -1330,7 +1353,7 @@ int launch_adam(float* p, const float* g, float* m, float* v, int64_t count, flo
   if (rest > 0) {
     int grid = (int)((rest + 255) / 256);
     if (grid > 4096) grid = 4096;
-    adam_kernel<<<grid, 256, 0, s>>>(p + head, gm + head, m + head, v + head, rest, a);
+    adam_kernel<<<grid, 256, 0, s>>>(p + head, gm + head, m + head, v + head, rest, a, failed);
   }
   return (int)cudaGetLastError();
 }

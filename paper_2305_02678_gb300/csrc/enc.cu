@@ -151,7 +151,9 @@ template <int KP>
 __global__ void __launch_bounds__(kBwdThreads, kBwdCtas) encoder_backward_kernel(const float* __restrict__ W, int K,
                                                                  const float* __restrict__ attrs,
                                                                  const float* __restrict__ dz, int64_t n,
-                                                                 float* __restrict__ grad) {
+                                                                 float* __restrict__ grad,
+                                                                 const int* __restrict__ failed) {
+  if (failed && *failed) return;  // dz is not this batch's
   extern __shared__ __align__(16) unsigned char smem_raw[];
   using Sm = EncBwdSmem<KP>;
   Sm& S = *reinterpret_cast<Sm*>(smem_raw);
@@ -317,7 +319,7 @@ int launch_encode(const float* W, int K, const float* attrs, int64_t n, float* z
 }
 
 int launch_encoder_backward(const float* W, int K, const float* attrs, const float* dz, int64_t n, float* grad,
-                            int num_sms, void* stream) {
+                            int num_sms, const int* failed, void* stream) {
   if (n == 0) return 0;
   if (K < 1 || K > kKMax) return (int)cudaErrorInvalidValue;
   const int64_t tiles = (n + 31) / 32;  // one per warp
@@ -328,7 +330,7 @@ int launch_encoder_backward(const float* W, int K, const float* attrs, const flo
     const int smem = (int)sizeof(EncBwdSmem<kp>);
     static std::atomic<uint64_t> attr_done{0};
     once_per_device(attr_done, [&] { cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem); });
-    k<<<(int)grid, kBwdThreads, smem, (cudaStream_t)stream>>>(W, K, attrs, dz, n, grad);
+    k<<<(int)grid, kBwdThreads, smem, (cudaStream_t)stream>>>(W, K, attrs, dz, n, grad, failed);
   });
   return (int)cudaGetLastError();
 }

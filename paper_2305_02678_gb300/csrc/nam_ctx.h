@@ -30,7 +30,7 @@ struct nam_material_s {
   float* adam_m = nullptr;    // trainable: [pyr_off + texels*8]
   float* adam_v = nullptr;
   float* grad = nullptr;      // trainable: gradient buffer, same layout
-  void* train_scratch = nullptr;  // trainable: the training step's loss accumulator
+  void* train_scratch = nullptr;  // trainable: the training step's StepResult
   size_t train_scratch_bytes = 0;
   // encoder (Sec. 5.1), trainable materials created with encoder_inputs > 0:
   // one allocation of 4 x enc_n floats: masters, gradient, Adam m, Adam v
@@ -97,6 +97,12 @@ nam_status check_queries(const nam_material_s* m, const nam_queries* q);
 void fill_launch(nam_ctx* ctx, const nam_material_s* m, const nam_queries* q, int64_t n, float* rgb, uint32_t flags,
                  LaunchCommon* L);
 int launch_material(const LaunchCommon& L, int precision, void* stream);
+// The words a training step clears before its kernels and reads back after.
+struct StepResult {
+  float loss;
+  int32_t failed;  // the backward's waits ran out: the step was not applied
+};
+nam_status read_step(const StepResult* dev, float* loss_out, void* stream, const char* who);
 void build_chunks(const nam_work_item* items, int32_t n_items, std::vector<Chunk>* out);
 nam_status check_multi(nam_ctx* ctx, const nam_material* mats, int32_t nmat);
 void serve_stop(nam_ctx* ctx);

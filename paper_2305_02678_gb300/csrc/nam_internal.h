@@ -203,6 +203,9 @@ struct BackwardArgs {
   int num_sms;
   int* err;                // the context's device error word
   uint64_t timeout_ns;     // limit of every wait
+  int* failed;             // may be null; set to 1 when a wait ran out (the
+                           // gradients then hold a part of their sums, and
+                           // dz_out zeros in the rows that were not reached)
   // set by the launcher: the gradient of texels [tiny_tex0, texels) is summed
   // in per-warp shared copies, that of [cta_tex0, tiny_tex0) in one shared
   // copy per CTA, before it reaches the global buffer
@@ -252,12 +255,15 @@ int launch_select_eval(const SelectArgs& a, void* stream);
 inline int64_t encoder_params_of(int K) { return 32 * (int64_t)K + 32 + 32 * 32 + 32 + 8 * 32 + 8; }
 int launch_encode(const float* W, int K, const float* attrs, int64_t n, float* z_out, int num_sms, void* stream);
 // accumulates the gradient of sum <dz, encoder(attrs)> into grad (layout of W)
+// `failed` (here and below; may be null): a device word, set by this step's
+// launch_backward if its waits ran out; the launch then leaves everything as it
+// is but for the gradient, which launch_adam clears in any case.
 int launch_encoder_backward(const float* W, int K, const float* attrs, const float* dz, int64_t n, float* grad,
-                            int num_sms, void* stream);
+                            int num_sms, const int* failed, void* stream);
 int launch_loss(const float* rgb, const float* target, int64_t n, float* grad_rgb, float* loss_accum,
                 void* stream);
 int launch_adam(float* p, const float* g, float* m, float* v, int64_t count, float lr, float b1, float b2,
-                float eps, int step, void* stream);
+                float eps, int step, const int* failed, void* stream);
 int64_t n_params_of(const Shape& s);
 
 }  // namespace nam

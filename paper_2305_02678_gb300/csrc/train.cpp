@@ -47,6 +47,21 @@ static nam_status grow_scratch(nam_ctx* ctx, nam_material m, void** buf, size_t*
   return NAM_OK;
 }
 
+nam_status nam::read_step(const StepResult* dev, float* loss_out, void* stream, const char* who) {
+  cudaStream_t s = (cudaStream_t)stream;
+  StepResult r;
+  cudaError_t ce = cudaMemcpyAsync(&r, dev, sizeof r, cudaMemcpyDeviceToHost, s);
+  if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
+  if (ce != cudaSuccess) {
+    char what[96];
+    std::snprintf(what, sizeof what, "%s: loss readback", who);
+    return cuda_fail((int)ce, what);
+  }
+  if (r.failed) return fail(NAM_ERR_TIMEOUT, "%s: a device-side wait ran past its limit; the step was not applied", who);
+  *loss_out = r.loss;
+  return NAM_OK;
+}
+
 static void fill_bwd(nam_ctx* ctx, nam_material m, const nam_queries* q, int64_t n, const float* grad_rgb,
                      float* grad_params, float* grad_pyramid, uint32_t flags, BackwardArgs* a) {
   std::memset(a, 0, sizeof *a);
@@ -102,32 +117,28 @@ static nam_status train_step(nam_ctx* ctx, nam_material m, const nam_queries* q,
   DeviceGuard g(ctx->device);
   cudaStream_t s = (cudaStream_t)stream;
   // per-material scratch: the loss accumulator (the backward kernel runs the
-  // forward and the loss itself)
+  // forward and the loss itself) and the word that says whether it failed
   st = grow_scratch(ctx, m, &m->train_scratch, &m->train_scratch_bytes, 256, s, "nam_train_step");
   if (st) return st;
-  float* loss_acc = (float*)m->train_scratch;
-  int e = (int)cudaMemsetAsync(loss_acc, 0, sizeof(float), s);
+  StepResult* res = (StepResult*)m->train_scratch;
+  int e = (int)cudaMemsetAsync(res, 0, sizeof *res, s);
   BackwardArgs a;
   const int64_t np = m->n_params, po = m->pyr_off, nt = m->pyr.texels * 8;
   fill_bwd(ctx, m, q, n, nullptr, m->grad, m->grad + po, flags, &a);
   a.target = target_rgb;
   a.target_albedo = target_albedo;
-  a.loss_acc = loss_acc;
+  a.loss_acc = &res->loss;
+  a.failed = &res->failed;
   a.loss_inv = 1.0f / (float)(3 * n);
   if (!e) e = launch_backward(a, s);
   if (!e)
     e = launch_adam(m->params, m->grad, m->adam_m, m->adam_v, np, opt->lr_params, opt->beta1, opt->beta2, opt->eps,
-                    opt->step, s);
+                    opt->step, &res->failed, s);
   if (!e)
     e = launch_adam((float*)m->pyramid, m->grad + po, m->adam_m + po, m->adam_v + po, nt, opt->lr_pyramid,
-                    opt->beta1, opt->beta2, opt->eps, opt->step, s);
+                    opt->beta1, opt->beta2, opt->eps, opt->step, &res->failed, s);
   if (e) return cuda_fail(e, "nam_train_step: launch");
-  if (loss_out) {
-    cudaError_t ce = cudaMemcpyAsync(loss_out, loss_acc, sizeof(float), cudaMemcpyDeviceToHost, s);
-    if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
-    if (ce != cudaSuccess) return cuda_fail((int)ce, "nam_train_step: loss readback");
-  }
-  return NAM_OK;
+  return loss_out ? read_step(res, loss_out, s, "nam_train_step") : NAM_OK;
 }
 
 extern "C" nam_status nam_train_step(nam_ctx* ctx, nam_material m, const nam_queries* q, const float* target_rgb,
@@ -222,7 +233,7 @@ extern "C" nam_status nam_backward_encoded(nam_ctx* ctx, nam_material m, const n
   a.z_in = z;
   a.dz_out = dz;
   if (!e) e = launch_backward(a, s);
-  if (!e) e = launch_encoder_backward(m->enc, m->enc_in, attrs, dz, n, grad_encoder, ctx->num_sms, s);
+  if (!e) e = launch_encoder_backward(m->enc, m->enc_in, attrs, dz, n, grad_encoder, ctx->num_sms, nullptr, s);
   if (e) return cuda_fail(e, "nam_backward_encoded: launch");
   return NAM_OK;
 }
@@ -244,33 +255,29 @@ extern "C" nam_status nam_train_step_encoded(nam_ctx* ctx, nam_material m, const
   float *z, *dz;
   st = encoder_scratch(ctx, m, n, s, &z, &dz, "nam_train_step_encoded");
   if (st) return st;
-  float* loss_acc = (float*)m->train_scratch;
+  StepResult* res = (StepResult*)m->train_scratch;
   const int64_t en = m->enc_n;
   float* enc_grad = m->enc + en;
-  int e = (int)cudaMemsetAsync(loss_acc, 0, sizeof(float), s);
+  int e = (int)cudaMemsetAsync(res, 0, sizeof *res, s);
   if (!e) e = launch_encode(m->enc, m->enc_in, attrs, n, z, ctx->num_sms, s);
   BackwardArgs a;
   fill_bwd(ctx, m, q, n, nullptr, m->grad, nullptr, flags, &a);
   a.target = target_rgb;
-  a.loss_acc = loss_acc;
+  a.loss_acc = &res->loss;
+  a.failed = &res->failed;
   a.loss_inv = 1.0f / (float)(3 * n);
   a.z_in = z;
   a.dz_out = dz;
   if (!e) e = launch_backward(a, s);
-  if (!e) e = launch_encoder_backward(m->enc, m->enc_in, attrs, dz, n, enc_grad, ctx->num_sms, s);
+  if (!e) e = launch_encoder_backward(m->enc, m->enc_in, attrs, dz, n, enc_grad, ctx->num_sms, &res->failed, s);
   if (!e)
     e = launch_adam(m->params, m->grad, m->adam_m, m->adam_v, m->n_params, opt->lr_params, opt->beta1, opt->beta2,
-                    opt->eps, opt->step, s);
+                    opt->eps, opt->step, &res->failed, s);
   if (!e)
     e = launch_adam(m->enc, enc_grad, m->enc + 2 * en, m->enc + 3 * en, en, opt->lr_params, opt->beta1, opt->beta2,
-                    opt->eps, opt->step, s);
+                    opt->eps, opt->step, &res->failed, s);
   if (e) return cuda_fail(e, "nam_train_step_encoded: launch");
-  if (loss_out) {
-    cudaError_t ce = cudaMemcpyAsync(loss_out, loss_acc, sizeof(float), cudaMemcpyDeviceToHost, s);
-    if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
-    if (ce != cudaSuccess) return cuda_fail((int)ce, "nam_train_step_encoded: loss readback");
-  }
-  return NAM_OK;
+  return loss_out ? read_step(res, loss_out, s, "nam_train_step_encoded") : NAM_OK;
 }
 
 extern "C" nam_status nam_material_encoder(nam_ctx* ctx, nam_material m, float** encoder_dev) {

@@ -22,9 +22,9 @@ using namespace nam;
 namespace {
 
 constexpr int64_t kMaxQueries = NAM_NOALLOC_TRAIN_MAX_QUERIES;
-constexpr int64_t kHeaderFloats = 64;  // loss accumulator, padded to 256 bytes
+constexpr int64_t kHeaderFloats = 64;  // StepResult, padded to 256 bytes
 
-// [0, 64): loss accumulator; then rgb [max][3]; then dL/drgb [max][3]
+// [0, 64): StepResult; then rgb [max][3]; then dL/drgb [max][3]
 __device__ __align__(256) float g_train_scratch[kHeaderFloats + 6 * kMaxQueries];
 
 constexpr int kMaxDevices = 64;
@@ -74,16 +74,16 @@ extern "C" nam_status nam_train_step_noalloc(nam_ctx* ctx, nam_material m, const
   st = scratch_on_device(ctx->device, &scratch);
   if (st) return st;
   cudaStream_t s = (cudaStream_t)stream;
-  float* loss_acc = scratch;
+  StepResult* res = reinterpret_cast<StepResult*>(scratch);
   float* rgb = scratch + kHeaderFloats;
   float* grad_rgb = rgb + 3 * n;
-  // the accumulator keeps the previous call's value: clear it
-  cudaError_t ce = cudaMemsetAsync(loss_acc, 0, sizeof(float), s);
+  // it keeps the previous call's values: clear it
+  cudaError_t ce = cudaMemsetAsync(res, 0, sizeof *res, s);
   if (ce != cudaSuccess) return cuda_fail((int)ce, "nam_train_step_noalloc: clear");
   LaunchCommon L;
   fill_launch(ctx, m, q, n, rgb, flags, &L);
   int e = launch_eval_f32(L, s);
-  if (!e) e = launch_loss(rgb, target_rgb, n, grad_rgb, loss_acc, s);
+  if (!e) e = launch_loss(rgb, target_rgb, n, grad_rgb, &res->loss, s);
   BackwardArgs a;
   std::memset(&a, 0, sizeof a);
   a.pyr = m->pyr;
@@ -99,19 +99,15 @@ extern "C" nam_status nam_train_step_noalloc(nam_ctx* ctx, nam_material m, const
   a.num_sms = ctx->num_sms;
   a.err = ctx->err_word;
   a.timeout_ns = ctx->timeout_ns;
+  a.failed = &res->failed;
   if (!e) e = launch_backward(a, s);
   const int64_t np = m->n_params, po = m->pyr_off, nt = m->pyr.texels * 8;
   if (!e)
     e = launch_adam(m->params, m->grad, m->adam_m, m->adam_v, np, opt->lr_params, opt->beta1, opt->beta2, opt->eps,
-                    opt->step, s);
+                    opt->step, &res->failed, s);
   if (!e)
     e = launch_adam((float*)m->pyramid, m->grad + po, m->adam_m + po, m->adam_v + po, nt, opt->lr_pyramid,
-                    opt->beta1, opt->beta2, opt->eps, opt->step, s);
+                    opt->beta1, opt->beta2, opt->eps, opt->step, &res->failed, s);
   if (e) return cuda_fail(e, "nam_train_step_noalloc: launch");
-  if (loss_out) {
-    ce = cudaMemcpyAsync(loss_out, loss_acc, sizeof(float), cudaMemcpyDeviceToHost, s);
-    if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
-    if (ce != cudaSuccess) return cuda_fail((int)ce, "nam_train_step_noalloc: loss readback");
-  }
-  return NAM_OK;
+  return loss_out ? read_step(res, loss_out, s, "nam_train_step_noalloc") : NAM_OK;
 }
