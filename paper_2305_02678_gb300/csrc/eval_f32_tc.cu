@@ -2,6 +2,9 @@
 // change (a trainable material's masters may be written between launches: it
 // keeps the per-thread kernel of fwd_f32.cu).
 //
+// Rows whose decoder input is not finite, or so large that a layer could
+// overflow (a bound from the weights' norms), are evaluated per thread.
+//
 // Latent filter, frame MLP, frame build, direction transform and output layer
 // run in FP32 per thread, in the per-thread kernel's order of operations; the
 // decoder's wide layers run as bf16 MMAs on three-way splits: an activation
@@ -54,6 +57,7 @@ struct F32Params {
   float f1[8][16], fb1[16];  // frame layer 1, [input][unit] (paper form: 12 units, its only layer)
   float f2[6][16], fb2[6];   // frame MLP layer 2, [output][input]
   float wo[6][H], bo[6];     // output layer
+  float n2_max;              // |x|^2 up to which no layer can overflow
 };
 
 template <int H, int FK, int NH, int NCH, int NF>
@@ -68,8 +72,9 @@ struct F32Smem {
   static constexpr int BYTES = TSLOT_OFF + 16;
 };
 
-// One query with the weights in global memory: for the rows whose inputs are
-// not finite (an infinity has no split), with the per-thread kernel's results.
+// One query with the weights in global memory: for the rows of which a split
+// might not be finite (an infinity has none: its lower terms are NaN), because
+// their inputs are not or because a layer could overflow.
 template <int H, int NH, int FK, bool F16P>
 __device__ __noinline__ void eval_slow(const LaunchCommon& L, int64_t i, float y[6]) {
   const float* p = L.masters;
@@ -328,7 +333,7 @@ __global__ void __launch_bounds__((NCH + NF) * 128, 1)
 #pragma unroll
       for (int k = 0; k < KX; k += 2) n2 = ptx::fma2(make_float2(x[k], x[k + 1]), make_float2(x[k], x[k + 1]), n2);
       // an infinity or NaN in z or a direction makes it through the frame to x
-      const bool finite = n2.x + n2.y < __int_as_float(0x7f800000);
+      const bool in_range = n2.x + n2.y <= O.n2_max;
 #pragma unroll
       for (int k0 = 0; k0 < KX; k0 += 16) {
         uint32_t h[8], m[8], l[8];
@@ -403,7 +408,7 @@ __global__ void __launch_bounds__((NCH + NF) * 128, 1)
 #pragma unroll
       for (int o = 0; o < 6; ++o) y[o] = s[o].x + s[o].y;
       if (valid) {
-        if (!finite) eval_slow<H, NH, FK, F16P>(L, i, y);
+        if (!in_range) eval_slow<H, NH, FK, F16P>(L, i, y);
         if (alb) {
           L.albedo[3 * i + 0] = y[3];
           L.albedo[3 * i + 1] = y[4];
@@ -463,6 +468,29 @@ bool bf16_split(float w, uint16_t t[3]) {
   return true;
 }
 
+// The largest |x|^2 of a decoder input x (with the 1 that meets the bias) for
+// which every product, partial sum and activation of every layer stays below
+// 2^120: |h_l| <= |W_l| |h_{l-1}| + |b_l| in Euclidean and Frobenius norms,
+// followed through the layers as a |x| + c.  `dec`: n layers, widths w[0 .. n].
+double input_limit(const float* dec, const int* w, int n) {
+  const double top = 0x1p120;
+  auto norm = [](const float* p, int k) {
+    double s = 0.0;
+    for (int i = 0; i < k; ++i) s += (double)p[i] * p[i];
+    return std::sqrt(s);
+  };
+  double a = 1.0, c = 0.0, r = 0x1p64;
+  for (int l = 0; l < n; ++l) {
+    const int nw = w[l + 1] * w[l];
+    const double fw = norm(dec, nw), fb = norm(dec + nw, w[l + 1]);
+    a *= l == 0 ? std::hypot(fw, fb) : fw;
+    c = l == 0 ? 0.0 : fw * c + fb;
+    r = std::fmin(r, (top - c) / std::fmax(a, 1e-300));
+    dec += nw + w[l + 1];
+  }
+  return r < 0.0 ? 0.0 : r * r;
+}
+
 template <int H>
 F32Params<H> f32_params(const NarrowW& n) {
   F32Params<H> O;
@@ -472,6 +500,7 @@ F32Params<H> f32_params(const NarrowW& n) {
   std::memcpy(O.fb2, n.fb2, sizeof O.fb2);
   for (int o = 0; o < 6; ++o) std::memcpy(O.wo[o], n.wo[o], sizeof O.wo[o]);
   std::memcpy(O.bo, n.bo, sizeof O.bo);
+  O.n2_max = n.n2_max;
   return O;
 }
 
@@ -562,6 +591,11 @@ int pack_f32_tc_blob(const Shape& s, const float* frame, const float* dec, uint8
     for (int k = 0; k < H; ++k) nw->wo[n][k] = p[n * H + k];
     nw->bo[n] = p[s.out * H + n];
   }
+  const int widths[5] = {s.in, H, H, s.NH == 3 ? H : s.out, s.out};
+  const double n2 = input_limit(dec, widths, s.NH + 1);
+  // (inputs within binary16's range: at most 20 of them below 2^16)
+  if (!(n2 >= 0x1p37)) ok = false;
+  nw->n2_max = n2 < 3e38 ? (float)n2 : 3e38f;
   return ok ? 0 : -1;
 }
 

@@ -76,6 +76,7 @@ struct NarrowW {
   // FP32 arithmetic on the tensor cores (eval_f32_tc.cu; wo not halved
   // there): its frame layers too
   float f1[8][16], fb1[16], f2[6][16], fb2[6];
+  float n2_max;  // and the largest |decoder input|^2 its splits take
 };
 
 // ---------------------------------------------------------------------------
@@ -148,7 +149,8 @@ int pack_f16_blob(const Shape& s, int precision, const float* frame, const float
                   uint8_t* out, float* weight_scales_out);
 int launch_eval_tc(const LaunchCommon& L, int precision, void* stream);
 // FP32 evaluation on the tensor cores (weights packed once; -1 if a weight is
-// too large to round to bfloat16)
+// too large to round to bfloat16, or all are so large that decoder inputs within
+// binary16's range could overflow a layer)
 int launch_eval_f32_tc(const LaunchCommon& L, void* stream);
 size_t f32_tc_blob_bytes(const Shape& s);
 int pack_f32_tc_blob(const Shape& s, const float* frame, const float* dec, uint8_t* out, NarrowW* nw);

@@ -1,0 +1,49 @@
+"""FP32 evaluation of fixed weights at the ends of FP32's range, against the
+per-thread kernel (the same material made trainable)."""
+import numpy as np
+import pytest
+
+import workloads as W
+from conftest import to_device
+
+pytestmark = pytest.mark.gpu
+
+
+def _pair(ctx, rng, H, out=3, scale=(1.0, 1.0, 1.0), frame=None):
+    """Decoder weights scaled per layer, those behind the first layer made
+    positive (so that infinite units do not cancel)."""
+    pyr = W.make_pyramid(rng[0], 64, 64, 7, dtype=np.float32)
+    m = W.make_model(rng[1], (14, H, H, out), frame)
+    dec = [(Wl * np.float32(s), bl * np.float32(s)) for (Wl, bl), s in zip(m["decoder"], scale)]
+    dec[1:] = [(np.abs(Wl), bl) for Wl, bl in dec[1:]]
+    return [ctx.material(64, 64, 7, pyr, m["frame"], dec, precision=0, trainable=t) for t in (False, True)]
+
+
+def _eval(mats, dq, out):
+    return [np.concatenate([t.cpu().numpy() for t in (m.eval_albedo(dq) if out == 6 else (m.eval(dq),))], 1)
+            .astype(np.float64) for m in mats]
+
+
+# Scales of the layers: the first overflows for the queries with directions of
+# 1e12; for nearly all; the second and the output layer for those of 1e12
+@pytest.mark.parametrize("H,out", [(16, 3), (32, 6), (64, 3)])
+@pytest.mark.parametrize("scale", [(1e28, 1.0, 1e-28), (1e38, 1.0, 1e-30), (1e6, 1e22, 1.0), (1.0, 1.0, 1e28)])
+def test_overflow_of_a_layer(gctx, H, out, scale):
+    rng = W.rng_streams(211, 3)
+    mats = _pair(gctx, rng, H, out, scale)
+    n = 700
+    q = W.uniform_queries(rng[2], n, 6.0)
+    for k, f in enumerate(("wix", "wiy", "wiz", "wox", "woy", "woz")):
+        q[f][k::35] *= 1e12
+    a, b = _eval(mats, to_device(q), out)
+    assert np.array_equal(np.isnan(a), np.isnan(b)) and np.array_equal(np.isinf(a), np.isinf(b))
+    f = np.isfinite(b)
+    assert np.array_equal(a[~f & ~np.isnan(b)], b[~f & ~np.isnan(b)])
+    # sums of positive and negative terms in different orders in the first layer,
+    # of positive ones behind it: up to 65 roundings of 2^-24 a layer, against the row's scale
+    row = np.abs(np.where(f, b, 0.0)).max(1, keepdims=True) * np.ones_like(b)
+    with np.errstate(invalid="ignore"):
+        assert (np.abs(a - b)[f] <= 3 * 65 * 2.0 ** -24 * 8 * row[f]).all()
+    for m in mats:
+        m.destroy()
+    gctx.check()
