@@ -72,9 +72,22 @@ struct F32Smem {
   static constexpr int BYTES = TSLOT_OFF + 16;
 };
 
-// One query with the weights in global memory: for the rows of which a split
+// dot_row with the weights anywhere in memory: the same two sums
+template <int N>
+__device__ __forceinline__ float dot_row_any(const float* __restrict__ row, const float* h) {
+  float s0 = 0.0f, s1 = 0.0f;
+#pragma unroll 4
+  for (int k = 0; k < N; k += 2) {
+    s0 = fmaf(row[k], h[k], s0);
+    s1 = fmaf(row[k + 1], h[k + 1], s1);
+  }
+  return s0 + s1;
+}
+
+// One query with the weights in global memory, for the rows of which a split
 // might not be finite (an infinity has none: its lower terms are NaN), because
-// their inputs are not or because a layer could overflow.
+// their inputs are not or because a layer could overflow.  The operations of
+// eval_query in its order: the per-thread kernel's results bit for bit.
 template <int H, int NH, int FK, bool F16P>
 __device__ __noinline__ void eval_slow(const LaunchCommon& L, int64_t i, float y[6]) {
   const float* p = L.masters;
@@ -83,29 +96,23 @@ __device__ __noinline__ void eval_slow(const LaunchCommon& L, int64_t i, float y
   const float wi[3] = {L.q.wix[i], L.q.wiy[i], L.q.wiz[i]}, wo[3] = {L.q.wox[i], L.q.woy[i], L.q.woz[i]};
   for (int c = 0; c < 8; ++c) x[c] = z[c];
   constexpr int IN = FK == 2 ? 20 : 14;
+  // the frame layer on z: its unit j
+  auto unit = [&](int j, int bias) {
+    float s = p[bias + j];
+    for (int c = 0; c < 8; ++c) s = fmaf(p[j * 8 + c], z[c], s);
+    return s;
+  };
   if (FK == 1) {
     float hf[16], r[6];
-    for (int j = 0; j < 16; ++j) {
-      float s = p[128 + j];
-      for (int c = 0; c < 8; ++c) s = fmaf(p[j * 8 + c], z[c], s);
-      hf[j] = fmaxf(s, 0.0f);
-    }
-    for (int j = 0; j < 6; ++j) {
-      float s = p[240 + j];
-      for (int k = 0; k < 16; ++k) s = fmaf(p[144 + j * 16 + k], hf[k], s);
-      r[j] = s;
-    }
+    for (int j = 0; j < 16; ++j) hf[j] = fmaxf(unit(j, 128), 0.0f);
+    for (int j = 0; j < 6; ++j) r[j] = p[240 + j] + dot_row_any<16>(p + 144 + j * 16, hf);
     const Frame F = build_frame(r);
     to_local(F, wi[0], wi[1], wi[2], x + 8);
     to_local(F, wo[0], wo[1], wo[2], x + 11);
     p += 246;
   } else if (FK == 2) {
     float r[12];
-    for (int j = 0; j < 12; ++j) {
-      float s = p[96 + j];
-      for (int c = 0; c < 8; ++c) s = fmaf(p[j * 8 + c], z[c], s);
-      r[j] = s;
-    }
+    for (int j = 0; j < 12; ++j) r[j] = unit(j, 96);
     const Frame F1 = paper_frame(r), F2 = paper_frame(r + 6);
     to_local(F1, wi[0], wi[1], wi[2], x + 8);
     to_local(F2, wi[0], wi[1], wi[2], x + 11);
@@ -119,18 +126,10 @@ __device__ __noinline__ void eval_slow(const LaunchCommon& L, int64_t i, float y
     }
   }
   float a[H], b[H];
-  for (int j = 0; j < H; ++j) {
-    float s = p[IN * H + j];
-    for (int k = 0; k < IN; ++k) s = fmaf(p[j * IN + k], x[k], s);
-    a[j] = fmaxf(s, 0.0f);
-  }
+  for (int j = 0; j < H; ++j) a[j] = fmaxf(p[IN * H + j] + dot_row_any<IN>(p + j * IN, x), 0.0f);
   p += IN * H + H;
   for (int l = 1; l < NH; ++l) {
-    for (int j = 0; j < H; ++j) {
-      float s = p[H * H + j];
-      for (int k = 0; k < H; ++k) s = fmaf(p[j * H + k], a[k], s);
-      b[j] = fmaxf(s, 0.0f);
-    }
+    for (int j = 0; j < H; ++j) b[j] = fmaxf(p[H * H + j] + dot_row_any<H>(p + j * H, a), 0.0f);
     for (int j = 0; j < H; ++j) a[j] = b[j];
     p += H * H + H;
   }

@@ -47,3 +47,29 @@ def test_overflow_of_a_layer(gctx, H, out, scale):
     for m in mats:
         m.destroy()
     gctx.check()
+
+
+@pytest.mark.parametrize("H,out,frame", [(16, 3, None), (32, 6, (8, 16, 6)), (64, 3, (8, 16, 6)), (64, 6, None)])
+def test_rows_out_of_range_are_the_per_thread_kernels(gctx, H, out, frame):
+    """Bit for bit, whether the results are finite (directions of up to 1e25 with
+    weights of 1e-3 and less) or not."""
+    rng = W.rng_streams(212, 3)
+    pyr = W.make_pyramid(rng[0], 64, 64, 7, dtype=np.float32)
+    m = W.make_model(rng[1], (14, H, H, out), frame)
+    dec = [(Wl * np.float32(1e-3), bl) for Wl, bl in m["decoder"]]
+    mats = [gctx.material(64, 64, 7, pyr, m["frame"], dec, precision=0, trainable=t) for t in (False, True)]
+    n = 1400
+    q = W.uniform_queries(rng[2], n, 6.0)
+    rows = np.arange(0, n, 7)
+    for f in ("wix", "wiy", "wiz", "wox", "woy", "woz"):
+        q[f][rows] *= 1e25
+    q["wix"][rows[::5]] = np.inf
+    q["woy"][rows[1::5]] = np.nan
+    dq = to_device(q)
+    a, b = ([t.cpu().numpy() for t in (m.eval_albedo(dq) if out == 6 else (m.eval(dq),))] for m in mats)
+    for x, y in zip(a, b):
+        assert np.isfinite(y[rows[2::5]]).all()
+        assert np.array_equal(x[rows].view(np.int32), y[rows].view(np.int32))
+    for m in mats:
+        m.destroy()
+    gctx.check()
