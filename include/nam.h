@@ -206,7 +206,10 @@ typedef struct {
 } nam_material_info;
 
 /* Copy the pyramid and weights to the device in the layout the kernels read
- * (FP16/FP8 weights quantised here).  NAM_ERR_BUDGET if the context's
+ * (FP16/FP8 weights quantised here).  An F32 material that is not trainable
+ * also takes its decoder's weights as tensor-core operands (up to 65 KB, part
+ * of resident_bytes) if the budget and the device have room for them, and runs
+ * the per-thread kernel otherwise.  NAM_ERR_BUDGET if the context's
  * resident bytes would pass its budget; NAM_ERR_UNSUPPORTED for widths or a
  * precision/filter combination without a kernel. */
 nam_status nam_create_material(nam_ctx* ctx, const nam_material_desc* d, nam_material* out);

@@ -371,7 +371,16 @@ extern "C" nam_status nam_create_material(nam_ctx* ctx, const nam_material_desc*
     // for params and pyramid
     resident += 3ull * (m->pyr_off + pd.texels * 8) * 4;
   }
-  if (!budget_reserve(ctx, resident)) {
+  bool reserved = budget_reserve(ctx, resident);
+  if (!reserved && !f32_blob.empty()) {
+    // the split weights only make it faster: without room for them, the
+    // per-thread kernel
+    f32_blob.clear();
+    resident -= blob_bytes;
+    blob_bytes = 0;
+    reserved = budget_reserve(ctx, resident);
+  }
+  if (!reserved) {
     delete m;
     return fail(NAM_ERR_BUDGET, "material needs %llu bytes; %llu of %llu in use", (unsigned long long)resident,
                 (unsigned long long)ctx->resident.load(), (unsigned long long)ctx->budget);
@@ -380,6 +389,14 @@ extern "C" nam_status nam_create_material(nam_ctx* ctx, const nam_material_desc*
   int e = dev_alloc(ctx, &m->pyramid, pyr_bytes);
   if (!e) e = dev_alloc(ctx, (void**)&m->params, np * 4);
   if (!e && blob_bytes) e = dev_alloc(ctx, &m->blob, blob_bytes);
+  if (e && !m->blob && m->params && !f32_blob.empty()) {
+    cudaGetLastError();
+    e = 0;
+    f32_blob.clear();
+    budget_release(ctx, blob_bytes);
+    m->info.resident_bytes -= blob_bytes;
+    blob_bytes = 0;
+  }
   if (!e && !smp.empty()) e = dev_alloc(ctx, &m->sampler, smp.size());
   if (!e && !encw.empty()) e = dev_alloc(ctx, (void**)&m->enc, 4 * encw.size() * 4);
   if (!e && d->trainable) {

@@ -73,3 +73,26 @@ def test_rows_out_of_range_are_the_per_thread_kernels(gctx, H, out, frame):
     for m in mats:
         m.destroy()
     gctx.check()
+
+
+def test_budget_without_room_for_the_split_weights():
+    """A budget that just holds the pyramid and the masters still takes the
+    material, which then runs the per-thread kernel."""
+    from paper_2305_02678_gb300 import Context, NamError
+    rng = W.rng_streams(213, 3)
+    pyr = W.make_pyramid(rng[0], 32, 32, 6, dtype=np.float32)
+    m = W.make_model(rng[1], (14, 64, 64, 3), (8, 16, 6))
+    dq = to_device(W.uniform_queries(rng[2], 500, 5.0))
+    with Context(0) as ctx:
+        t = ctx.material(32, 32, 6, pyr, m["frame"], m["decoder"], precision=0, trainable=True)
+        want = t.eval(dq).cpu().numpy()
+        need = pyr.nbytes + 4 * t.info.n_params
+        assert ctx.material(32, 32, 6, pyr, m["frame"], m["decoder"], precision=0).info.resident_bytes > need
+    with Context(0, hbm_budget_bytes=need) as ctx:
+        f = ctx.material(32, 32, 6, pyr, m["frame"], m["decoder"], precision=0)
+        assert f.info.resident_bytes == need == ctx.stats().resident_bytes
+        assert np.array_equal(f.eval(dq).cpu().numpy(), want)
+        f.destroy()
+        assert ctx.stats().resident_bytes == 0
+    with Context(0, hbm_budget_bytes=need - 1) as ctx, pytest.raises(NamError):
+        ctx.material(32, 32, 6, pyr, m["frame"], m["decoder"], precision=0)
