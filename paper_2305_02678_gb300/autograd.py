@@ -159,6 +159,7 @@ def log_l1_loss(rgb, target):
     """Mean over the batch and channels of |log(1 + max(g, 0)) - log(1 + y)|
     plus 0.01 * max(-g, 0): the paper's L1 loss in log space (Sec. 5), with a
     small linear penalty so that negative outputs still receive a gradient."""
-    if _one_pass(rgb, target):
-        return _LogL1.apply(rgb, target)
+    if not torch.jit.is_scripting():  # (scripting compiles the tensor operations)
+        if _one_pass(rgb, target):
+            return _LogL1.apply(rgb, target)
     return _log_l1_ops(rgb, target)
