@@ -110,33 +110,39 @@ def _log_l1_ops(rgb, target):
 
 
 class _LogL1(torch.autograd.Function):
-    """_log_l1_ops of contiguous FP32 CUDA tensors in one pass: the forward
-    also writes the derivative for a unit gradient.  A derivative that is
-    itself to be differentiated is taken through the tensor operations."""
+    """_log_l1_ops of contiguous FP32 CUDA tensors in one pass: (loss, x), x a
+    copy of rgb that belongs to the derivatives.  The forward also writes the
+    derivative for a unit gradient, and the copy; they are all that is saved, so
+    that, as with the tensor operations, the inputs may change or go away, the
+    graph's saved tensors (and their hooks) hold everything there is, and
+    nothing of it outlives the backward.  A derivative that is itself to be
+    differentiated is written out in tensor operations on x, whose own gradient
+    is rgb's."""
 
     @staticmethod
     def forward(ctx, rgb, target):
+        ctx.set_materialize_grads(False)
         loss = torch.empty((), dtype=torch.float32, device=rgb.device)
         work = torch.empty(304, dtype=torch.float64, device=rgb.device)
-        unit = torch.empty_like(rgb) if ctx.needs_input_grad[0] else None
-        B._check(B.lib().nam_internal_log_l1(rgb.data_ptr(), target.data_ptr(), rgb.numel(), B.ptr(unit),
+        unit, x = (torch.empty_like(rgb), torch.empty_like(rgb)) if ctx.needs_input_grad[0] else (None, None)
+        B._check(B.lib().nam_internal_log_l1(rgb.data_ptr(), target.data_ptr(), rgb.numel(), B.ptr(unit), B.ptr(x),
                                              loss.data_ptr(), work.data_ptr(), B.current_stream(rgb.device)),
                  "log_l1_loss")
         if unit is not None:
-            ctx.save_for_backward(unit)
-            ctx.inputs = rgb, target, rgb._version, target._version
-        return loss
+            ctx.save_for_backward(unit, x)
+        return loss, x
 
     @staticmethod
-    def backward(ctx, grad):
+    def backward(ctx, grad, grad_x):
+        unit, x = ctx.saved_tensors
+        if grad is None:
+            return grad_x, None
         if torch.is_grad_enabled():
-            rgb, target, *versions = ctx.inputs
-            if [rgb._version, target._version] != versions:
-                raise RuntimeError("log_l1_loss: an input needed for a second derivative was modified in place")
-            loss = _log_l1_ops(rgb, target)
-            return torch.autograd.grad(loss, rgb, grad, create_graph=True)[0], None
-        unit, = ctx.saved_tensors
-        return unit * grad, None
+            # the same derivative as a function of x; at x <= 0 it is constant
+            r = torch.relu(x)
+            unit = torch.where(x > 0, unit.sign() / x.numel() / (r + 1), unit)
+        g = unit * grad
+        return (g if grad_x is None else g + grad_x), None
 
 
 def _one_pass(rgb, target):
@@ -161,5 +167,5 @@ def log_l1_loss(rgb, target):
     small linear penalty so that negative outputs still receive a gradient."""
     if not torch.jit.is_scripting():  # (scripting compiles the tensor operations)
         if _one_pass(rgb, target):
-            return _LogL1.apply(rgb, target)
+            return _LogL1.apply(rgb, target)[0]
     return _log_l1_ops(rgb, target)

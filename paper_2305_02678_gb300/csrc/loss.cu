@@ -29,12 +29,12 @@ __device__ __forceinline__ double block_sum(double v) {
   return t;
 }
 
-// unit (may be null): d(mean)/dg.  Zeros, infinities and NaN as the tensor
+// unit, copy (may be null, both or neither): d(mean)/dg, and g again.  Zeros, infinities and NaN as the tensor
 // operations' derivatives have them: sign is 0 at 0 and NaN, no gradient through
 // max(g, 0) at g <= 0.
 __global__ void __launch_bounds__(kThreads) log_l1_kernel(const float* __restrict__ g, const float* __restrict__ y,
                                                           int64_t n, float inv_n, float* __restrict__ unit,
-                                                          double* __restrict__ partial) {
+                                                          float* __restrict__ copy, double* __restrict__ partial) {
   float sum = 0.0f;
   for (int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x; i < n; i += (int64_t)gridDim.x * kThreads) {
     const float x = g[i];
@@ -45,6 +45,7 @@ __global__ void __launch_bounds__(kThreads) log_l1_kernel(const float* __restric
       const float s = d > 0.0f ? inv_n : d < 0.0f ? -inv_n : 0.0f;
       const float a = x <= 0.0f ? 0.0f : s / (r + 1.0f);
       unit[i] = -x <= 0.0f ? a : a - 0.01f * inv_n;
+      copy[i] = x;
     }
   }
   const double t = block_sum(sum);
@@ -63,15 +64,15 @@ __global__ void __launch_bounds__(kThreads) log_l1_mean_kernel(const double* __r
 }  // namespace nam
 
 // Internal to the Python package (autograd.log_l1_loss), on the current
-// device: loss[0], unit[n] or null; work: kMaxBlocks doubles.
-extern "C" nam_status nam_internal_log_l1(const float* g, const float* y, int64_t n, float* unit, float* loss,
-                                          double* work, void* stream) {
+// device: loss[0], unit[n] and copy[n] or null; work: kMaxBlocks doubles.
+extern "C" nam_status nam_internal_log_l1(const float* g, const float* y, int64_t n, float* unit, float* copy,
+                                          float* loss, double* work, void* stream) {
   using namespace nam;
   if (n < 1) return fail(NAM_ERR_INVALID_ARG, "log_l1: no values");
   const int64_t want = (n + 4 * kThreads - 1) / (4 * kThreads);
   const int blocks = (int)(want < kMaxBlocks ? want : kMaxBlocks);
   cudaStream_t s = (cudaStream_t)stream;
-  log_l1_kernel<<<blocks, kThreads, 0, s>>>(g, y, n, 1.0f / (float)n, unit, work);
+  log_l1_kernel<<<blocks, kThreads, 0, s>>>(g, y, n, 1.0f / (float)n, unit, copy, work);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) {
     log_l1_mean_kernel<<<1, kThreads, 0, s>>>(work, blocks, n, loss);
