@@ -109,6 +109,11 @@ def _log_l1_ops(rgb, target):
     return (d.abs() + 0.01 * torch.relu(-rgb)).mean()
 
 
+# partial sums of the one-pass loss, one per block: two blocks per SM of a GB300
+# (the library launches no more blocks than it is given sums)
+_WORK = 304
+
+
 class _LogL1(torch.autograd.Function):
     """_log_l1_ops of contiguous FP32 CUDA tensors in one pass: (loss, x), x a
     copy of rgb that belongs to the derivatives.  The forward also writes the
@@ -123,10 +128,11 @@ class _LogL1(torch.autograd.Function):
     def forward(ctx, rgb, target):
         ctx.set_materialize_grads(False)
         loss = torch.empty((), dtype=torch.float32, device=rgb.device)
-        work = torch.empty(304, dtype=torch.float64, device=rgb.device)
+        work = torch.empty(_WORK, dtype=torch.float64, device=rgb.device)
         unit, x = (torch.empty_like(rgb), torch.empty_like(rgb)) if ctx.needs_input_grad[0] else (None, None)
         B._check(B.lib().nam_internal_log_l1(rgb.data_ptr(), target.data_ptr(), rgb.numel(), B.ptr(unit), B.ptr(x),
-                                             loss.data_ptr(), work.data_ptr(), B.current_stream(rgb.device)),
+                                             loss.data_ptr(), work.data_ptr(), _WORK,
+                                             B.current_stream(rgb.device)),
                  "log_l1_loss")
         if unit is not None:
             ctx.save_for_backward(unit, x)

@@ -182,7 +182,7 @@ def _load():
         "nam_cancel": (i32, [p, u64]),
         "nam_get_stats": (i32, [p, p]),
         "nam_inject_fault": (i32, [p, i32]),
-        "nam_internal_log_l1": (i32, [p, p, i64, p, p, p, p, p]),  # not in nam.h: autograd.log_l1_loss
+        "nam_internal_log_l1": (i32, [p, p, i64, p, p, p, p, i64, p]),  # not in nam.h: autograd.log_l1_loss
     }
     for name, (res, args) in sig.items():
         f = getattr(lib, name)

@@ -15,7 +15,6 @@ namespace nam {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kMaxBlocks = 304;  // two per SM; as many partial sums
 
 __device__ __forceinline__ double block_sum(double v) {
   __shared__ double s[kThreads / 32];
@@ -64,13 +63,16 @@ __global__ void __launch_bounds__(kThreads) log_l1_mean_kernel(const double* __r
 }  // namespace nam
 
 // Internal to the Python package (autograd.log_l1_loss), on the current
-// device: loss[0], unit[n] and copy[n] or null; work: kMaxBlocks doubles.
+// device: loss[0], unit[n] and copy[n] or null; work: n_work doubles, as many
+// as there are blocks at most.
 extern "C" nam_status nam_internal_log_l1(const float* g, const float* y, int64_t n, float* unit, float* copy,
-                                          float* loss, double* work, void* stream) {
+                                          float* loss, double* work, int64_t n_work, void* stream) {
   using namespace nam;
+  if (n_work < 1) return fail(NAM_ERR_INVALID_ARG, "log_l1: no workspace");
   if (n < 1) return fail(NAM_ERR_INVALID_ARG, "log_l1: no values");
   const int64_t want = (n + 4 * kThreads - 1) / (4 * kThreads);
-  const int blocks = (int)(want < kMaxBlocks ? want : kMaxBlocks);
+  const int64_t cap = n_work < 65535 ? n_work : 65535;
+  const int blocks = (int)(want < cap ? want : cap);
   cudaStream_t s = (cudaStream_t)stream;
   log_l1_kernel<<<blocks, kThreads, 0, s>>>(g, y, n, 1.0f / (float)n, unit, copy, work);
   cudaError_t e = cudaGetLastError();

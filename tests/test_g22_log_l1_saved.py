@@ -88,3 +88,18 @@ def test_hooks_see_everything_saved():
     assert torch.cuda.memory_allocated() - before <= one  # the scalar; all else is on the host
     g, = torch.autograd.grad(l, x, create_graph=True)
     assert g.requires_grad and torch.isfinite(g).all()
+
+
+@pytest.mark.parametrize("n_work", [1, 7, 304, 1000])
+def test_no_more_blocks_than_the_workspace_holds(n_work):
+    import torch
+    from paper_2305_02678_gb300 import autograd as A
+    from paper_2305_02678_gb300 import binding as B
+    x, y = _inputs(100000)
+    loss = torch.zeros((), device="cuda")
+    work = torch.full((n_work + 400,), -5.0, dtype=torch.float64, device="cuda")
+    B._check(B.lib().nam_internal_log_l1(x.data_ptr(), y.data_ptr(), x.numel(), None, None, loss.data_ptr(),
+                                         work.data_ptr(), n_work, B.current_stream(x.device)), "log_l1")
+    assert (work[n_work:] == -5.0).all()
+    # FP32 sums of up to 300,000 / 256 positive terms in a thread
+    assert abs(loss.item() - A._log_l1_ops(x.double(), y.double()).item()) <= 1200 * 2.0 ** -24 * loss.item()
