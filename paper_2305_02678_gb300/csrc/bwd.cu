@@ -10,7 +10,11 @@
 // the signs, which is two thirds of the work, runs on the tensor cores as
 // bf16 MMAs on three-way splits (x = x_h + x_m + x_l, eight significant bits
 // each; six products, FP32 accumulation, small products first), which have
-// FP32's range and lose less than its rounding.
+// FP32's range.  The deltas' terms are cut off, the other operand's (weights,
+// H1, X, HF) rounded to nearest: the three products left out are below 1.5
+// 2^-23 of a term and of either sign (with both cut off up to 3.9 2^-23 of one
+// sign).  Weight gradients against 64 bits, as a multiple of the error of every
+// product on the FMA pipes (40,000 queries): 0.74 .. 1.08.
 //  - a quad of four adjacent lanes per query: the latent fetch, the frame MLP
 //    (lane p owns frame hidden units p + 4e, the six outputs are summed over
 //    the quad), the frame construction and its backward (redundant in the
@@ -116,25 +120,33 @@ __device__ __forceinline__ void split3_one(float x, uint16_t& h, uint16_t& m, ui
   m = (uint16_t)(br >> 16);
   l = (uint16_t)(__float_as_uint(q) >> 16);
 }
-// the same of a weight, rounded to nearest: terms of either sign, so that what
+// the same of x (1 + up), rounded to nearest: terms of either sign, so that what
 // the six products leave out (middle times last, last times last) has no sign
-// of its own, and a little (4e-8) larger, for the accumulator, which cuts off:
-// dL/dz came out 1.6e-7 too small without either
-__device__ __forceinline__ void split3_weight(float x, uint16_t& h, uint16_t& m, uint16_t& l) {
+// of its own.  `up` makes up for the accumulator, which cuts off
+__device__ __forceinline__ void split3_up(float x, float up, uint16_t& h, uint16_t& m, uint16_t& l) {
   const __nv_bfloat16 a = __float2bfloat16_rn(x);
   const float r = x - __bfloat162float(a);
   const __nv_bfloat16 b = __float2bfloat16_rn(r);
   h = __bfloat16_as_ushort(a);
   m = __bfloat16_as_ushort(b);
-  l = __bfloat16_as_ushort(__float2bfloat16_rn(fmaf(x, 4e-8f, r - __bfloat162float(b))));
+  l = __bfloat16_as_ushort(__float2bfloat16_rn(fmaf(x, up, r - __bfloat162float(b))));
 }
+// (measured against 64 bits: dL/dz came out 1.6e-7 too small with cut-off weight
+// terms; the weight gradients 1.0e-7 with cut-off terms of both operands,
+// 0.6e-7 with those of H1, X and HF rounded, below 0.2e-7 with these factors)
+constexpr float kWeightUp = 4e-8f;  // W1, W2 in the products over units
+constexpr float kSumUp = 6e-8f;     // H1, X, HF in the products over queries
 // U values (consecutive units) of one query to their rows of the three terms;
-// p: the first unit's place in term 0, TS: bytes of a term
-template <int U, int TS>
+// p: the first unit's place in term 0, TS: bytes of a term.  RN: terms
+// rounded to nearest (split3_rn)
+template <int U, int TS, bool RN = false>
 __device__ __forceinline__ void put_terms(uint8_t* p, const float (&v)[U]) {
   uint32_t w[3][U / 2];
 #pragma unroll
-  for (int j = 0; j < U / 2; ++j) ptx::split3(v[2 * j], v[2 * j + 1], w[0][j], w[1][j], w[2][j]);
+  for (int j = 0; j < U / 2; ++j) {
+    if (RN) ptx::split3_rn(v[2 * j], v[2 * j + 1], kSumUp, w[0][j], w[1][j], w[2][j]);
+    else ptx::split3(v[2 * j], v[2 * j + 1], w[0][j], w[1][j], w[2][j]);
+  }
 #pragma unroll
   for (int t = 0; t < 3; ++t) {
     if constexpr (U == 4) {
@@ -340,7 +352,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const Backward
     for (int i = t; i < H * H; i += kBwdThreads) {
       const int j = i / H, k = i % H;  // W2[j][k] -> row k, K index j
       uint16_t w[3];
-      split3_weight(W2[i], w[0], w[1], w[2]);
+      split3_up(W2[i], kWeightUp, w[0], w[1], w[2]);
 #pragma unroll
       for (int e = 0; e < 3; ++e)
         *reinterpret_cast<uint16_t*>(S.W2T + e * H * H * 2 + (j / 8) * (H * 16) + k * 16 + (j % 8) * 2) = w[e];
@@ -348,7 +360,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const Backward
     for (int i = t; i < H * 16; i += kBwdThreads) {
       const int j = i / 16, c = i % 16;
       uint16_t w[3];
-      split3_weight(c < 14 ? W1[j * 14 + c] : 0.0f, w[0], w[1], w[2]);
+      split3_up(c < 14 ? W1[j * 14 + c] : 0.0f, kWeightUp, w[0], w[1], w[2]);
 #pragma unroll
       for (int e = 0; e < 3; ++e)
         *reinterpret_cast<uint16_t*>(S.W1T + e * 16 * H * 2 + (j / 8) * 256 + c * 16 + (j % 8) * 2) = w[e];
@@ -554,13 +566,13 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const Backward
       const float4 a = reinterpret_cast<const float4*>(&G.X[ql][0])[2 * p];
       const float4 b = reinterpret_cast<const float4*>(&G.X[ql][0])[2 * p + 1];
       const float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, p ? 1.0f : b.z, b.w};
-      put_terms<8, TB>(G.B + (H / 8 + p) * kBlk + ql * 16, v);
+      put_terms<8, TB, true>(G.B + (H / 8 + p) * kBlk + ql * 16, v);
     }
     if (FRAME) {
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
         uint16_t w[3];
-        split3_one(hf[e], w[0], w[1], w[2]);
+        split3_up(hf[e], kSumUp, w[0], w[1], w[2]);
         uint8_t* o = G.B + (H / 8 + 2 + (e >> 1)) * kBlk + ql * 16 + ((p + 4 * e) & 7) * 2;
 #pragma unroll
         for (int k = 0; k < 3; ++k) *reinterpret_cast<uint16_t*>(o + k * TB) = w[k];
@@ -603,7 +615,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const Backward
           v[k] = x.x; v[k + 1] = x.y; v[k + 2] = x.z; v[k + 3] = x.w;
         }
         const int u0 = U * (lane >> 3);
-        put_terms<U, TB>(G.B + (u0 / 8) * kBlk + (8 * lw + (lane & 7)) * 16 + (u0 % 8) * 2, v);
+        put_terms<U, TB, true>(G.B + (u0 / 8) * kBlk + (8 * lw + (lane & 7)) * 16 + (u0 % 8) * 2, v);
       }
       // layer 2
 #pragma unroll

@@ -308,6 +308,21 @@ __device__ __forceinline__ void split3(float a, float b, uint32_t& h, uint32_t& 
   const float2 q = sub2(r, make_float2(top(r.x), top(r.y)));
   l = pack(q.x, q.y);
 }
+// (a, b) -> the three bf16 pairs of x (1 + up), each term rounded to nearest:
+// terms of either sign, whose sum is x before the last one takes x * up.
+__device__ __forceinline__ void split3_rn(float a, float b, float up, uint32_t& h, uint32_t& m, uint32_t& l) {
+  auto pack = [](float x, float y) {
+    uint32_t r;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(y), "f"(x));
+    return r;
+  };
+  auto val = [](uint32_t p) { return make_float2(__uint_as_float(p << 16), __uint_as_float(p & 0xFFFF0000u)); };
+  h = pack(a, b);
+  const float2 r = sub2(make_float2(a, b), val(h));
+  m = pack(r.x, r.y);
+  const float2 q = fma2(make_float2(a, b), make_float2(up, up), sub2(r, val(m)));
+  l = pack(q.x, q.y);
+}
 // Read-only global load that the compiler keeps where it is written (the
 // value's first use waits on it, wherever that is).
 __device__ __forceinline__ float ld_nc_pinned(const float* p) {
