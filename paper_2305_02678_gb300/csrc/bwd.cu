@@ -41,7 +41,10 @@
 // H = 64 with the fused loss, 262,144 queries, 1024^2 pyramid: 281 us, against
 // 378 us with every product on the FMA pipes; 131,072 queries with the latents
 // given: 131 us (163).  Smaller batches and decoders, against that kernel:
-// H = 64, 10,000 queries 37 us (44); H = 16, 262,144 queries 188 us (207).
+// H = 64, 10,000 queries 33 us (43); H = 16, 262,144 queries 188 us (207),
+// 10,000 queries 23 us (25), 7,000 without the frame 18 us (22), one query
+// 12.5 us (10.4: the only sizes that lose are single tiles at H = 16 and 32
+// without the frame, to the three MMA round trips).
 // Training step variant (LOSS): the decoder blocks also finish the forward
 // (y = Wo h2 + bo, summed over the half-warp), evaluate the log-space L1
 // loss against the target and start the backward from its gradient, so a
@@ -318,54 +321,71 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const Backward
   typename Sm::Group& G = S.g[grp];
   const uint32_t bar0 = ptx::smem_u32(S.bars) + 32 * grp;
   const int bid = 4 * grp;  // named barriers bid + 1 .. bid + 4
-  // ---- parameters -> shared ---------------------------------------------------
-  {
-    const float* p = A.params;
-    if (FRAME) {
-      for (int i = t; i < 128; i += kBwdThreads) S.fW1[i] = p[i];
-      if (t < 16) S.fb1[t] = p[128 + t];
-      for (int i = t; i < 96; i += kBwdThreads) S.fW2[i] = p[144 + i];
-      if (t < 8) S.fb2[t] = t < 6 ? p[240 + t] : 0.0f;
-      p += 246;
-    }
-    auto row = [](int j) { return P == 2 ? (j >> 5) * 16 + (j & 15) : j; };
-    auto col = [](int j, int k) { return P == 2 ? 2 * k + ((j >> 4) & 1) : k; };
-    for (int i = t; i < H * 16; i += kBwdThreads) {
-      const int j = i / 16, k = i % 16;
-      S.W1[row(j)][col(j, k)] = k < 14 ? p[j * 14 + k] : 0.0f;
-    }
-    p += 14 * H;
-    for (int i = t; i < H; i += kBwdThreads) S.b1[i] = p[i];
-    p += H;
-    for (int i = t; i < H * H; i += kBwdThreads) S.W2[row(i / H)][col(i / H, i % H)] = p[i];
-    p += H * H;
-    for (int i = t; i < H; i += kBwdThreads) S.b2[i] = p[i];
-    p += H;
-    for (int i = t; i < NO * H; i += kBwdThreads) S.Wo[i] = p[i];
-    p += NO * H;
-    if (t < 8) S.bo[t] = t < NO ? p[t] : 0.0f;
+  const int64_t ntiles = (A.n + kBwdQ - 1) / kBwdQ;
+  const int64_t tile0 = blockIdx.x + (int64_t)grp * gridDim.x, tstep = 2 * (int64_t)gridDim.x;
+  // lw: this warp in its group
+  const int lw = ((warp >> 2) << 1) | (warp & 1), lt = 32 * lw + lane;
+  const int ql = lt >> 2, p = lt & 3;         // quad: query ql, lane p
+  // the fields of the next tile are loaded a tile ahead, the first one's before
+  // the parameters (its texels as well would cost more in spilled registers than
+  // their latency)
+  auto row_of = [&](int64_t tile, bool& valid) -> int64_t {
+    const int64_t start = tile * kBwdQ;
+    valid = ql < A.n - start;
+    return start + (valid ? ql : 0);
+  };
+  QuadFields nxt{};
+  if (tile0 < ntiles) {
+    bool v;
+    const int64_t i = row_of(tile0, v);
+    nxt = quad_fields<LOSS, ALB>(A, i, v, p);
   }
-  // MMA B operands of the delta products
+  // ---- parameters -> shared ---------------------------------------------------
+  // Every load of a thread is in flight before its first value is used (loops
+  // over the arrays one after the other, and the weights read twice, were ten
+  // memory latencies: 2,200 to 8,000 cycles of a small batch's 30,000 to 50,000).
   {
     const float* W1 = A.params + (FRAME ? 246 : 0);
     const float* W2 = W1 + 14 * H + H;
-    for (int i = t; i < H * H; i += kBwdThreads) {
-      const int j = i / H, k = i % H;  // W2[j][k] -> row k, K index j
-      uint16_t w[3];
-      split3_up(W2[i], kWeightUp, w[0], w[1], w[2]);
+    constexpr int kTail = H + NO * H + NO;  // b2, Wo, bo
+    static_assert(H * H / 8 <= kBwdThreads && kTail + 8 <= kBwdThreads, "one pass");
+    const float vf = FRAME && t < 246 ? __ldg(A.params + t) : 0.0f;
+    const float v1 = t < H ? __ldg(W1 + 14 * H + t) : 0.0f;
+    const float vt = t < kTail ? __ldg(W2 + H * H + t) : 0.0f;
+    // eight units j of one input each
+    const int j1 = t / 16 * 8, c1 = t % 16, j2 = t / H * 8, k2 = t % H;
+    float w1[8], w2[8];
 #pragma unroll
-      for (int e = 0; e < 3; ++e)
-        *reinterpret_cast<uint16_t*>(S.W2T + e * H * H * 2 + (j / 8) * (H * 16) + k * 16 + (j % 8) * 2) = w[e];
-    }
-    for (int i = t; i < H * 16; i += kBwdThreads) {
-      const int j = i / 16, c = i % 16;
-      uint16_t w[3];
-      split3_up(c < 14 ? W1[j * 14 + c] : 0.0f, kWeightUp, w[0], w[1], w[2]);
-#pragma unroll
-      for (int e = 0; e < 3; ++e)
-        *reinterpret_cast<uint16_t*>(S.W1T + e * 16 * H * 2 + (j / 8) * 256 + c * 16 + (j % 8) * 2) = w[e];
+    for (int e = 0; e < 8; ++e) {
+      w1[e] = j1 < H && c1 < 14 ? __ldg(W1 + (j1 + e) * 14 + c1) : 0.0f;
+      w2[e] = j2 < H ? __ldg(W2 + (j2 + e) * H + k2) : 0.0f;
     }
     for (int i = t; i < NO * H + 8; i += kBwdThreads) S.gwo[i] = 0.0f;
+    // fW1, fb1, fW2, fb2, and b2, Wo, bo, lie side by side, zeros behind them
+    if (FRAME && t < 248) (&S.fW1[0])[t] = vf;
+    if (t < H) S.b1[t] = v1;
+    if (t < kTail - NO + 8) (&S.b2[0])[t] = vt;
+    auto row = [](int j) { return P == 2 ? (j >> 5) * 16 + (j & 15) : j; };
+    auto col = [](int j, int k) { return P == 2 ? 2 * k + ((j >> 4) & 1) : k; };
+    // the eight units of a K block side by side in the B operands of the delta
+    // products: rows k (or c), K index j
+    auto operand = [](uint8_t* o, int term, const float (&w)[8]) {
+      uint32_t v[3][4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) ptx::split3_rn(w[2 * e], w[2 * e + 1], kWeightUp, v[0][e], v[1][e], v[2][e]);
+#pragma unroll
+      for (int e = 0; e < 3; ++e) *reinterpret_cast<uint4*>(o + e * term) = make_uint4(v[e][0], v[e][1], v[e][2], v[e][3]);
+    };
+    if (j1 < H) {
+#pragma unroll
+      for (int e = 0; e < 8; ++e) S.W1[row(j1 + e)][col(j1 + e, c1)] = w1[e];
+      operand(S.W1T + j1 / 8 * 256 + c1 * 16, 16 * H * 2, w1);
+    }
+    if (j2 < H) {
+#pragma unroll
+      for (int e = 0; e < 8; ++e) S.W2[row(j2 + e)][col(j2 + e, k2)] = w2[e];
+      operand(S.W2T + j2 / 8 * (H * 16) + k2 * 16, H * H * 2, w2);
+    }
   }
   if (t == 0) {
     // C1 and CF are issued by two warps
@@ -387,7 +407,6 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const Backward
   __syncthreads();
   ptx::tc_fence_after();
   const uint32_t tmem = S.tslot + cGroup * grp;
-  const int64_t ntiles = (A.n + kBwdQ - 1) / kBwdQ;
   bool bad = false;
 
   // A stage's products, one thread: six of term pairs, the small ones first.
@@ -406,10 +425,8 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const Backward
   const uint32_t aA = ptx::smem_u32(G.A), aB = ptx::smem_u32(G.B);
   const uint32_t aK = aA - grp * 64 * 16, aM = aA - grp * 8 * kBlk;
   constexpr uint32_t kMN = (1u << 15) | (1u << 16);  // both operands MN-major
-  const int64_t tile0 = blockIdx.x + (int64_t)grp * gridDim.x, tstep = 2 * (int64_t)gridDim.x;
-  // lw: this warp in its group.  Gradients of this thread's part of C2, C1 and
-  // CF: row grow of the group's half of the TMEM lanes, a quarter of the columns
-  const int lw = ((warp >> 2) << 1) | (warp & 1), lt = 32 * lw + lane;
+  // gradients of this thread's part of C2, C1 and CF: row grow of the group's
+  // half of the TMEM lanes, a quarter of the columns
   const int grow = 32 * (lw & 1) + lane, gq = lw >> 1;
   const uint32_t tl = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
   const bool use2 = 32 * (lw & 1) < H, usef = FRAME && (lw & 1) == 0;
@@ -455,25 +472,11 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const Backward
   uint32_t ph = 0;  // parity of this tile's MMAs
 
   float lsum = 0.0f;  // fused loss: this lane's share of the sum
-  const int ql = lt >> 2, p = lt & 3;         // quad: query ql, lane p
   const int hl = lt & 15, qb = (lt >> 4) * 4;  // half-warp: queries qb..qb+3, units hl + 16 jj
   const bool cosine = (A.flags & NAM_OUT_COSINE) != 0;
   uint32_t issued = 0;  // tiles whose MMAs were issued (the same in the whole group)
   bool stop = false;    // a wait ran out
   int64_t left = ntiles;  // the tile it ran out in
-  // the fields of the next tile are loaded a tile ahead (its texels as well
-  // would cost more in spilled registers than their latency)
-  auto row_of = [&](int64_t tile, bool& valid) -> int64_t {
-    const int64_t start = tile * kBwdQ;
-    valid = ql < A.n - start;
-    return start + (valid ? ql : 0);
-  };
-  QuadFields nxt{};
-  if (tile0 < ntiles) {
-    bool v;
-    const int64_t i = row_of(tile0, v);
-    nxt = quad_fields<LOSS, ALB>(A, i, v, p);
-  }
   for (int64_t tile = tile0; tile < ntiles; tile += tstep, ph ^= 1u) {
     const int64_t start = tile * kBwdQ;
     const int count = (int)((A.n - start) < kBwdQ ? (A.n - start) : kBwdQ);
@@ -1119,15 +1122,22 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const Backward
       for (int w = 0; w < 16; ++w) tot += S.lred[w];
       atomicAdd(A.loss_acc, tot * A.loss_inv);
     }
-    for (int k = t; k < 8 * A.tiny_n; k += kBwdThreads) {
-      float c = 0.0f;
-      for (int w = 0; w < 16; ++w) c += wacc[w * 8 * A.tiny_n + k];
-      if (c != 0.0f) atomicAdd(A.grad_pyramid + A.tiny_tex0 * 8 + k, c);
+    // (half a texel at a time: a float at a time, 36,000 of them at H = 16, took
+    // 3,700 cycles)
+    auto add4 = [](float* g, const float4& c) {
+      if (c.x != 0.0f || c.y != 0.0f || c.z != 0.0f || c.w != 0.0f) atomicAdd(reinterpret_cast<float4*>(g), c);
+    };
+    for (int k = t; k < 2 * A.tiny_n && t < 64; k += 64) {
+      float4 c = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      for (int w = 0; w < 16; ++w) {
+        const float4 v = reinterpret_cast<const float4*>(wacc + w * 8 * A.tiny_n)[k];
+        c = make_float4(c.x + v.x, c.y + v.y, c.z + v.z, c.w + v.w);
+      }
+      add4(A.grad_pyramid + A.tiny_tex0 * 8 + 4 * k, c);
     }
-    for (int k = t; k < 8 * A.cta_n; k += kBwdThreads) {
-      const float c = cacc[k];
-      if (c != 0.0f) atomicAdd(A.grad_pyramid + A.cta_tex0 * 8 + k, c);
-    }
+#pragma unroll 4
+    for (int k = t - 64; k < 2 * A.cta_n && t >= 64; k += kBwdThreads - 64)
+      add4(A.grad_pyramid + A.cta_tex0 * 8 + 4 * k, reinterpret_cast<const float4*>(cacc)[k]);
     // Both groups' sums of C2, C1 and CF meet in shared memory (odd row
     // lengths: no bank conflicts; the first group's operands are done with),
     // so that the atomics run along the parameters and once per CTA (straight
@@ -1200,8 +1210,18 @@ static int launch_bwd_one(const BackwardArgs& a, cudaStream_t s) {
   constexpr int kSmemMax = 227 * 1024;
   constexpr int kBase = (int)sizeof(BwdSmem<H, ALB>);
   static_assert(kBase <= kSmemMax, "backward tile does not fit in shared memory");
+  const int64_t tiles = (a.n + kBwdQ - 1) / kBwdQ;
+  // a tile per CTA while there are SMs; beyond that a CTA's two groups take one
+  // each (its time is theirs, and there are no more sums to add up than needed:
+  // with a CTA on every SM 157 tiles took as long and sent twice the atomics,
+  // whose roundings made the weight gradients' error 1.3 times as large)
+  const int64_t pairs = (tiles + 1) / 2;
+  int grid = (int)(tiles <= a.num_sms ? tiles : pairs < a.num_sms ? pairs : a.num_sms);
+  if (grid < 1) grid = 1;
   // coarse-level accumulators in what the tile leaves: per-warp copies of the
-  // coarsest levels up to kTiny texels, then one copy of the next levels
+  // coarsest levels up to kTiny texels, then one copy of the next levels, as long
+  // as a CTA's queries (four texels each) can meet there: a copy of 4,000 texels
+  // for 64 queries costs more to clear and to look through than their atomics
   constexpr int64_t kTiny = 24;
   BackwardArgs b = a;
   b.tiny_tex0 = b.cta_tex0 = a.pyr.texels;
@@ -1217,15 +1237,16 @@ static int launch_bwd_one(const BackwardArgs& a, cudaStream_t s) {
     b.tiny_n = (int32_t)(a.pyr.texels - b.tiny_tex0);
     room -= 16 * (int64_t)b.tiny_n;
     b.cta_tex0 = b.tiny_tex0;
-    for (; l >= 0 && b.tiny_tex0 - a.pyr.off[l] <= room; --l) b.cta_tex0 = a.pyr.off[l];
+    const int64_t per_cta = a.n / grid;
+    for (; l >= 0 && b.tiny_tex0 - a.pyr.off[l] <= room; --l) {
+      if ((int64_t)a.pyr.w[l] * a.pyr.h[l] > 2 * per_cta) break;
+      b.cta_tex0 = a.pyr.off[l];
+    }
     b.cta_n = (int32_t)(b.tiny_tex0 - b.cta_tex0);
   }
   const int smem = kBase + 32 * (16 * b.tiny_n + b.cta_n);
   static std::atomic<uint64_t> attr_done{0};
   once_per_device(attr_done, [&] { cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax); });
-  const int64_t tiles = (a.n + kBwdQ - 1) / kBwdQ;
-  int grid = (int)(tiles < a.num_sms ? tiles : a.num_sms);
-  if (grid < 1) grid = 1;
   k<<<grid, kBwdThreads, smem, s>>>(b);
   return (int)cudaGetLastError();
 }
