@@ -96,3 +96,41 @@ def test_budget_without_room_for_the_split_weights():
         assert ctx.stats().resident_bytes == 0
     with Context(0, hbm_budget_bytes=need - 1) as ctx, pytest.raises(NamError):
         ctx.material(32, 32, 6, pyr, m["frame"], m["decoder"], precision=0)
+
+
+def _family(kind, rng, dec):
+    """Weights other than Glorot's uniform ones."""
+    f = {"glorot": lambda w: w, "positive": np.abs,
+         "heavy": lambda w: (w / np.abs(w).max()) ** 3 * np.abs(w).max() * 2}[kind]
+    return [(np.ascontiguousarray(f(w), np.float32), b) for w, b in dec]
+
+
+@pytest.mark.parametrize("H", [16, 32, 64])
+@pytest.mark.parametrize("kind", ["glorot", "positive", "heavy"])
+def test_error_against_64_bits_is_the_per_thread_kernels(gctx, oracle, H, kind):
+    rng = W.rng_streams(214, 4)
+    pyr = W.make_pyramid(rng[0], 128, 128, 8, dtype=np.float32)
+    dec = _family(kind, rng[3], W.make_model(rng[1], (14, H, H, 3), None)["decoder"])
+    q = W.uniform_queries(rng[2], 30000, 7.0)
+    ref = oracle.eval(oracle.Model(128, 128, 8, pyr, None, dec), q)
+    dq = to_device(q)
+    err = []
+    for t in (False, True):
+        mat = gctx.material(128, 128, 8, pyr, None, dec, precision=0, trainable=t)
+        err.append(np.linalg.norm(mat.eval(dq).cpu().numpy().astype(np.float64) - ref))
+        mat.destroy()
+    assert err[0] <= 1.1 * err[1]  # (a tenth for the chance of one batch's roundings)
+
+
+def test_error_of_three_hidden_layers(gctx, oracle):
+    """No per-thread form to compare with: four layers of sums whose roundings,
+    2^-24 each, add up like random ones, are well within 2^-21 of the result."""
+    rng = W.rng_streams(215, 3)
+    pyr = W.make_pyramid(rng[0], 128, 128, 8, dtype=np.float32)
+    dec = W.make_model(rng[1], (14, 64, 64, 64, 3), None)["decoder"]
+    q = W.uniform_queries(rng[2], 30000, 7.0)
+    ref = oracle.eval(oracle.Model(128, 128, 8, pyr, None, dec), q)
+    mat = gctx.material(128, 128, 8, pyr, None, dec, precision=0)
+    err = np.linalg.norm(mat.eval(to_device(q)).cpu().numpy().astype(np.float64) - ref)
+    assert err <= 2.0 ** -21 * np.linalg.norm(ref)
+    mat.destroy()
