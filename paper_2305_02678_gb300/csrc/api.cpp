@@ -191,7 +191,6 @@ extern "C" nam_status nam_shutdown(nam_ctx* ctx) {
   ctx->materials.clear();
   cudaFree(ctx->err_word);
   cudaFree(ctx->stage_dev);
-  if (ctx->stage_stream) cudaStreamDestroy((cudaStream_t)ctx->stage_stream);
   if (ctx->h2d_stream) cudaStreamDestroy((cudaStream_t)ctx->h2d_stream);
   if (ctx->d2h_stream) cudaStreamDestroy((cudaStream_t)ctx->d2h_stream);
   for (void* ev : ctx->stage_events) cudaEventDestroy((cudaEvent_t)ev);

@@ -191,7 +191,6 @@ __global__ void __launch_bounds__(1024) bin_plan_kernel(const uint32_t* __restri
 // neighbourhoods of the caller's arrays.
 // Shared memory: cnt, run, excl [nmat] each, then the query index and the
 // material of each local position [kSeg] each.
-constexpr int kStage = 1;
 constexpr int kDirectMaterials = 4;  // segments of at most this many materials skip the ordering
 
 __global__ void __launch_bounds__(kThreads) bin_scatter_kernel(const int32_t* __restrict__ ids, int64_t n, int nmat,
@@ -203,7 +202,7 @@ __global__ void __launch_bounds__(kThreads) bin_scatter_kernel(const int32_t* __
   uint32_t* run = sh + nmat;        // [nmat] first slot of the segment's run
   uint32_t* excl = sh + 2 * nmat;   // [nmat] first local position of each material
   uint32_t* stage = sh + 3 * nmat;  // [kSeg] query index of each local position
-  int32_t* smat = reinterpret_cast<int32_t*>(stage + kStage * kSeg);  // [kSeg]
+  int32_t* smat = reinterpret_cast<int32_t*>(stage + kSeg);  // [kSeg]
   __shared__ uint32_t wsum[kThreads / 32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t seg = (int64_t)blockIdx.x * kSeg;
@@ -454,11 +453,11 @@ static int bin_eval(const BinArgs& a, const int32_t* tile_k, cudaStream_t s) {
   bin_count_kernel<<<gseg, kThreads, a.nmat * sizeof(uint32_t), s>>>(a.ids, n, a.nmat, tile_k, counts, a.L.err);
   const int gplan = (maxc + 1023) / 1024 < 16 ? (maxc + 1023) / 1024 : 16;
   bin_plan_kernel<<<gplan, 1024, 2 * (a.nmat + 1) * sizeof(uint32_t), s>>>(counts, a.nmat, cursors, chunks, n_used);
-  const int scatter_smem = (3 * a.nmat + (kStage + 1) * kSeg) * (int)sizeof(uint32_t);
+  const int scatter_smem = (3 * a.nmat + 2 * kSeg) * (int)sizeof(uint32_t);
   static std::atomic<uint64_t> scatter_attr{0};
   once_per_device(scatter_attr, [] {
     cudaFuncSetAttribute(bin_scatter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (3 * NAM_MAX_BIN_MATERIALS + (kStage + 1) * kSeg) * (int)sizeof(uint32_t));
+                         (3 * NAM_MAX_BIN_MATERIALS + 2 * kSeg) * (int)sizeof(uint32_t));
   });
   bin_scatter_kernel<<<gseg, kThreads, scatter_smem, s>>>(a.ids, n, a.nmat, tile_k, cursors, orig);
   e = (int)cudaGetLastError();

@@ -302,7 +302,7 @@ __device__ __forceinline__ QuadFields quad_fields(const BackwardArgs& A, int64_t
   return f;
 }
 
-template <int H, bool FRAME, bool F16, bool LOSS, bool ALB>
+template <int H, bool FRAME, bool LOSS, bool ALB>
 __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const BackwardArgs A) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   using Sm = BwdSmem<H, ALB>;
@@ -1204,9 +1204,9 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const Backward
   }
 }
 
-template <int H, bool FRAME, bool F16, bool LOSS, bool ALB>
+template <int H, bool FRAME, bool LOSS, bool ALB>
 static int launch_bwd_one(const BackwardArgs& a, cudaStream_t s) {
-  auto k = backward_kernel<H, FRAME, F16, LOSS, ALB>;
+  auto k = backward_kernel<H, FRAME, LOSS, ALB>;
   constexpr int kSmemMax = 227 * 1024;
   constexpr int kBase = (int)sizeof(BwdSmem<H, ALB>);
   static_assert(kBase <= kSmemMax, "backward tile does not fit in shared memory");
@@ -1255,10 +1255,10 @@ static int launch_bwd_one(const BackwardArgs& a, cudaStream_t s) {
 template <int H, bool ALB>
 static int bwd_dispatch_alb(const BackwardArgs& a, cudaStream_t s) {
   if (a.target)
-    return a.shape.frame ? launch_bwd_one<H, true, false, true, ALB>(a, s)
-                         : launch_bwd_one<H, false, false, true, ALB>(a, s);
-  return a.shape.frame ? launch_bwd_one<H, true, false, false, ALB>(a, s)
-                       : launch_bwd_one<H, false, false, false, ALB>(a, s);
+    return a.shape.frame ? launch_bwd_one<H, true, true, ALB>(a, s)
+                         : launch_bwd_one<H, false, true, ALB>(a, s);
+  return a.shape.frame ? launch_bwd_one<H, true, false, ALB>(a, s)
+                       : launch_bwd_one<H, false, false, ALB>(a, s);
 }
 
 template <int H>

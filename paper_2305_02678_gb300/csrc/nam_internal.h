@@ -157,8 +157,6 @@ int pack_f32_tc_blob(const Shape& s, const float* frame, const float* dec, uint8
 void pack_narrow(const Shape& s, const float* dec, NarrowW* out);
 
 // Weight blob sizes and packing (host side).
-size_t f32_blob_floats(const Shape& s);
-void pack_f32_blob(const Shape& s, const float* frame, const float* dec, float* out);
 size_t tc_blob_bytes(const Shape& s, int precision);
 int pack_tc_blob(const Shape& s, int precision, const float* frame, const float* dec,
                  const float* act_scale, uint8_t* out, float* weight_scales_out);
