@@ -476,7 +476,6 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const Backward
   const bool cosine = (A.flags & NAM_OUT_COSINE) != 0;
   uint32_t issued = 0;  // tiles whose MMAs were issued (the same in the whole group)
   bool stop = false;    // a wait ran out
-  int64_t left = ntiles;  // the tile it ran out in
   for (int64_t tile = tile0; tile < ntiles; tile += tstep, ph ^= 1u) {
     const int64_t start = tile * kBwdQ;
     const int count = (int)((A.n - start) < kBwdQ ? (A.n - start) : kBwdQ);
@@ -782,7 +781,6 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const Backward
     // every warp has read its H1 rows: A takes D2
     if (ptx::bar_red_or(bid + 4, kBwdGroup, bad)) {
       stop = true;
-      left = tile;
       break;
     }
     // ---- layer-2 delta d2 = (Wo^T dy) where the unit is active ---------------
@@ -892,7 +890,6 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const Backward
       // (the other half of C1's and CF's barrier)
       if (lw == 5 && ptx::elect()) ptx::mma_commit(bar0 + 24);
       stop = true;
-      left = tile;
       break;
     }
     // ---- quad: frame backward, pyramid scatter --------------------------------
@@ -1094,13 +1091,16 @@ __global__ void __launch_bounds__(kBwdThreads, 1) backward_kernel(const Backward
   // ---- flush: one atomic per parameter and coarse texel channel per CTA -------
   if (stop) {
     bad = true;
-    // the encoder's backward reads every row of dz: none is left from before
-    if (A.dz_out)
-      for (; left < ntiles; left += tstep) {
-        bool valid;
-        const int64_t i = row_of(left, valid);
-        if (valid) reinterpret_cast<float2*>(A.dz_out + 8 * i)[p] = make_float2(0.0f, 0.0f);
-      }
+    // the encoder's backward reads every row of dz: those of this group's tiles
+    // become zero, so that none is left from an earlier batch (worked out anew
+    // here: values kept for this over the loop cost the kernel 10 us in spills)
+    if (A.dz_out) {
+      const int w = threadIdx.x >> 5, g = (w >> 1) & 1;
+      const int r = 32 * (((w >> 2) << 1) | (w & 1)) + (threadIdx.x & 31);
+      for (int64_t k = blockIdx.x + (int64_t)g * gridDim.x; k * kBwdQ < A.n; k += 2 * (int64_t)gridDim.x)
+        if (k * kBwdQ + (r >> 2) < A.n)
+          reinterpret_cast<float2*>(A.dz_out)[4 * k * kBwdQ + r] = make_float2(0.0f, 0.0f);
+    }
   } else if (tile0 < ntiles) {
     bad |= !ptx::mbar_wait(bar0 + 24, ph ^ 1u, A.timeout_ns);
     collect();
