@@ -474,6 +474,9 @@ nam_status nam_scene_render_paths(nam_ctx* ctx, const nam_scene* scene, const na
  * gradients are reduced per CTA then added with one atomic per parameter and
  * CTA; pyramid gradients are scattered with atomics (tap weight x dL/dz).
  * ReLU'(0) = 0.  No gradient flows through the degenerate-frame fallbacks.
+ * An output gradient that is not finite makes the gradients it reaches not
+ * finite (NaN also where a product of FP32 values would be an infinity: the
+ * products take FP32 operands as sums of bf16 terms).
  * After a device-side wait that ran out (nam_check_device_error) the buffers
  * hold a part of the sums. */
 nam_status nam_backward(nam_ctx* ctx, nam_material m, const nam_queries* q, int64_t n,

@@ -38,13 +38,13 @@
 // What bounds it: the latency of the tile's chain of stages (16 warps a CTA,
 // which shared memory and registers allow no more of; the forward on the FMA
 // pipes is a fifth of a tile's time, the fetch and the scatter a sixth each).
-// H = 64 with the fused loss, 262,144 queries, 1024^2 pyramid: 281 us, against
+// H = 64 with the fused loss, 262,144 queries, 1024^2 pyramid: 279 us, against
 // 378 us with every product on the FMA pipes; 131,072 queries with the latents
-// given: 131 us (163).  Smaller batches and decoders, against that kernel:
-// H = 64, 10,000 queries 33 us (43); H = 16, 262,144 queries 188 us (207),
-// 10,000 queries 23 us (25), 7,000 without the frame 18 us (22), one query
-// 12.5 us (10.4: the only sizes that lose are single tiles at H = 16 and 32
-// without the frame, to the three MMA round trips).
+// given: 131 us (163).  Smaller batches and decoders, against that kernel
+// (512^2, no loss): H = 64, 10,000 queries 29 us (35); H = 16, 262,144 queries
+// 187 us (206), 10,000 queries 20.6 us (22.7), 7,000 without the frame 16.5 us
+// (18.6), one query 12.4 us (10.4: the only sizes that lose are single tiles at
+// H = 16 and 32 without the frame, to the three MMA round trips).
 // Training step variant (LOSS): the decoder blocks also finish the forward
 // (y = Wo h2 + bo, summed over the half-warp), evaluate the log-space L1
 // loss against the target and start the backward from its gradient, so a
@@ -1341,7 +1341,7 @@ __global__ void adam_kernel(float* __restrict__ p, float* __restrict__ g, float*
 // 16-byte vector form of the same per-element update, bound by HBM: four
 // streams read, three written, and the gradient cleared only where a query
 // reached the texel (262,144 queries, training step with a 2048^2 pyramid 557
-// -> 544 us, 1024^2 357 -> 355, 256^2, where all are reached, the same).
+// -> 544 us, 1024^2 384 -> 381, 256^2, where all are reached, the same).
 __global__ void adam4_kernel(float4* __restrict__ p, float4* __restrict__ g, float4* __restrict__ m,
                              float4* __restrict__ v, int64_t count4, const AdamStep a,
                              const int* __restrict__ failed) {

@@ -26,9 +26,10 @@
 // MMA round trips per tile.  TMEM columns of a chain: accumulator [0, H),
 // then the operand: three terms of the decoder input (KX / 2 columns each)
 // or of a hidden layer (H / 2 columns each).
-// What bounds it: instruction issue (the splits take 11 instructions per pair
-// of activations) and, at H = 64, three chains per SM (160 columns each).
-// 1280x720, H = 64, frame MLP: 84 us, 334 in the per-thread kernel (fed from
+// What bounds it: at H = 64, three chains per SM (160 columns each): 20 warps
+// keep 57 % of the issue slots (the splits take 11 instructions per pair of
+// activations) and 35 % of the tensor pipe busy.
+// 1280x720, H = 64, frame MLP: 81 us, 334 in the per-thread kernel (fed from
 // shared memory at a third of the FP32 rate).
 #include "eval_tc.cuh"
 #include "f32_body.cuh"

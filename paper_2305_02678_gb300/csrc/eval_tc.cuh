@@ -22,10 +22,9 @@
 // hi + lo, hi = x with its 13 low mantissa bits cleared, exact in FP16; lo =
 // x - hi, rounded), i.e. at ~22-bit accuracy; the other hidden layers are
 // rounded to FP16 once; the output layer reads the last one in FP32.
-// What bounds it (1920x1080, H = 64): instruction issue (1,170 thread
+// What bounds it (1920x1080, H = 64): instruction issue (1,028 thread
 // instructions per query, 70 % of the issue slots) and the chain of MMA round
-// trips; the L1 data pipe, which takes a cycle per texel sector that misses,
-// is 42 % busy.  Measured on the way, 1920x1080: 117 us with the fetch in the
+// trips.  Measured on the way, 1920x1080: 117 us with the fetch in the
 // chains' own warps through cp.async, 112 with fetch warps staging through
 // cp.async, 111 with the texels in their registers, 98 with the output layer
 // on the FMA pipes (its operand split and MMA round trip cost more than its

@@ -15,7 +15,7 @@
 // [x_hi | x_lo | 1 1] x [W_hi | W_hi | b_hi b_lo] and one over x_hi x W_lo give
 // W x + b up to the dropped W_lo x_lo term, a relative 2^-22.  The proxy's
 // activations, density and sampling run per thread in FP32.
-// What bounds it: instruction issue (73 % of the slots); 1920x1080, sample and
+// What bounds it: instruction issue (75 % of the slots); 1920x1080, sample and
 // density: 97 us, 146 with the fetch in the chains' own warps.
 #include <cuda_runtime.h>
 
