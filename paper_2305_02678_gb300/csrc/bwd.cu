@@ -14,7 +14,7 @@
 // H1, X, HF) rounded to nearest: the three products left out are below 1.5
 // 2^-23 of a term and of either sign (with both cut off up to 3.9 2^-23 of one
 // sign).  Weight gradients against 64 bits, as a multiple of the error of every
-// product on the FMA pipes (40,000 queries): 0.74 .. 1.08.
+// product on the FMA pipes (40,000 queries, by layer): 0.70 .. 1.08.
 //  - a quad of four adjacent lanes per query: the latent fetch, the frame MLP
 //    (lane p owns frame hidden units p + 4e, the six outputs are summed over
 //    the quad), the frame construction and its backward (redundant in the
